@@ -270,6 +270,11 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
     ph.c_g0[2] = -2.0 * (ph.omega / 3.0) * ph.inv_cl2;
     ph.m3cl2 = -3.0 * p->c_l * p->c_l;
     ph.three_cl = 3.0 * p->c_l;
+    ph.fx = make_fx_run(ph.omega, p->c_l);
+    // the fixed-point FP64 step: measured closer to the exact values than the
+    // binary64 one for lattice speeds up to 3 (rlb_fixed.cuh); its cell
+    // offsets are 32-bit byte counts
+    ph.fx_on = p->eos == RLB_EOS_ULTRA && p->c_l >= 1.0 && p->c_l <= 2.0 && S < (1ll << 29) ? 1 : 0;
     ph.eos = p->eos;
     ph.eos_gamma = p->eos == RLB_EOS_GAMMA_LAW ? p->eos_gamma : 4.0 / 3.0;
     ph.eos_mass = p->eos == RLB_EOS_GAMMA_LAW ? p->eos_mass : 0.0;
@@ -671,9 +676,11 @@ rlb_status rlb_debug_bounds_violations(int64_t* count) {
 #ifdef RLB_CHECK_BOUNDS
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaDeviceSynchronize");
-    const unsigned long long a = oob_take_forward(), b = oob_take_adjoint(), d = oob_take_eos(), e2 = oob_take_stream();
-    if (a == ~0ull || b == ~0ull || d == ~0ull || e2 == ~0ull) return fail(nullptr, RLB_ERR_CUDA, "reading the bounds counters failed");
-    *count = (int64_t)(a + b + d + e2);
+    const unsigned long long a = oob_take_forward(), b = oob_take_adjoint(), d = oob_take_eos(), e2 = oob_take_stream(),
+                             h = oob_take_step64();
+    if (a == ~0ull || b == ~0ull || d == ~0ull || e2 == ~0ull || h == ~0ull)
+        return fail(nullptr, RLB_ERR_CUDA, "reading the bounds counters failed");
+    *count = (int64_t)(a + b + d + e2 + h);
     return RLB_OK;
 #else
     *count = -1;

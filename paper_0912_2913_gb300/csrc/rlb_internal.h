@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "rlb_fixed.cuh"
+
 namespace rlb {
 
 enum : int { XBC_PERIODIC = 0, XBC_INFLOW_OUTFLOW = 1, XBC_OUTFLOW_BOTH = 2 };
@@ -60,6 +62,8 @@ struct Phys {
     // omega g_0^eq: 4 omega w0, -omega w0 (2/c_l^2 + 1), -2 omega w0 / c_l^2;
     // -3 c_l^2 and 3 c_l for the recovery from M / c_l.
     double c_k1[2], c_k2[2], c_k3[2], c_fs[2], c_fa[2], c_f0, c_g0[3], m3cl2, three_cl;
+    FxRun fx;   // constants of the fixed-point FP64 step
+    int fx_on;  // 1: the FP64 step runs in block fixed point
 };
 
 // Binary32 constants of the FP32 deviation step.
@@ -85,6 +89,11 @@ cudaError_t launch_step(int prec, const Geom& g, const Phys& ph, const void* A, 
                         bool count, long long step_index, cudaStream_t stream);
 cudaError_t launch_macro(int prec, const Geom& g, const Phys& ph, const void* A, double* n, double* eps,
                          double* beta, Counters cnt, cudaStream_t stream);
+// FP64 step (rlb_step64.cu).
+cudaError_t launch_step_f64(const Geom& g, const Phys& ph, const void* A, void* B, Counters cnt, bool count,
+                            long long step_index, cudaStream_t stream);
+// Constants of the fixed-point FP64 step.
+FxRun make_fx_run(double omega, double c_l);
 // FP64 step with its arithmetic in compensated binary32 pairs (rlb_f64df.cu).
 cudaError_t launch_step_f64_df(const Geom& g, const Phys& ph, const void* A, void* B, Counters cnt, bool count,
                                long long step_index, cudaStream_t stream, int threads);
@@ -146,6 +155,7 @@ unsigned long long oob_take_forward();
 unsigned long long oob_take_adjoint();
 unsigned long long oob_take_eos();
 unsigned long long oob_take_stream();
+unsigned long long oob_take_step64();
 #ifdef RLB_CHECK_BOUNDS
 // Runs the index check on (i, n) in a kernel; returns the checked index.
 long long bounds_selftest(long long i, long long n, cudaStream_t s);

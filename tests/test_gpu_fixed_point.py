@@ -1,0 +1,86 @@
+"""The FP64 step in block fixed point (csrc/rlb_fixed.cuh, 1 <= c_l <= 2) at
+the edges of its range, against the oracle: gathered populations far apart in
+size, negative and exactly zero ones, |M| up to and beyond E (cells that take
+the binary64 path), extreme exponents, lattice speeds on both sides of the
+limits; one thread and eight lanes per cell give the same bits."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+EV = np.asarray(oracle.lattice()[0], int)
+# Error bound in units of 2^-53 of a cell's largest population: at |beta| =
+# 0.985 the oracle's own eps gamma^2 carries 3 roundings of E times gamma^2 =
+# 34; 19 sums and the relaxation stay below 32 units.
+UNITS = 1024
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _need_gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+
+
+def _gathered(rng, shape, c_l):
+    """Populations (cells, 2, 19) as a step gathers them, one kind per cell."""
+    N = int(np.prod(shape))
+    b = rng.normal(size=(N, 3))
+    b *= (rng.choice([0.0, 0.01, 0.4, 0.7, 0.9, 0.985], N) / np.linalg.norm(b, axis=1))[:, None]
+    p = oracle.Params(nx=N, ny=1, nz=1, tau=0.8, c_l=c_l)
+    h = oracle.init(p, np.exp(rng.uniform(-3, 3, N)), np.exp(rng.uniform(-3, 3, N)), b.T.copy()).reshape(N, 2, 19)
+    h *= 1 + 0.02 * rng.uniform(-1, 1, h.shape)
+    kind = rng.integers(0, 6, N)
+    small = rng.uniform(size=h.shape) < 0.3
+    h[(kind == 1)[:, None, None] & small] = 0.0
+    h[(kind == 2)[:, None, None] & small] *= 2.0 ** -45
+    h[kind == 3] *= (2.0 ** rng.integers(-200, 200, (kind == 3).sum()))[:, None, None]
+    h[:, 1, 1][kind == 4] *= 40.0  # |M| near or above E
+    h[N // 2, 1] *= -1.0  # E < 0
+    return h.reshape(shape + (2, 19))
+
+
+def _scatter(h):
+    """The state a step gathers h from (periodic): A_i(x - e_i) = h_i(x)."""
+    a = np.empty_like(h)
+    for i in range(19):
+        a[..., i] = np.roll(h[..., i], tuple(-EV[i][c] for c in (2, 1, 0)), axis=(0, 1, 2))
+    return a
+
+
+@pytest.mark.parametrize("c_l", [1.0, 1.7, 2.0, 2.0 + 2 ** -30])
+@pytest.mark.parametrize("tau", [0.51, 0.8, 1.0, 30.0])
+def test_one_step_of_hard_states(c_l, tau, monkeypatch):
+    from paper_0912_2913_gb300 import RLB
+
+    nz, ny, nx = shape = (6, 7, 37)
+    h = _gathered(np.random.default_rng(int(8 * c_l + 100 * tau)), shape, c_l)
+    a = _scatter(h)
+    p = oracle.Params(nx=nx, ny=ny, nz=nz, tau=tau, c_l=c_l)
+    stats = oracle.Stats()
+    ref = oracle.step(p, a, stats=stats)
+    outs = []
+    for split in ("0", "1"):
+        monkeypatch.setenv("RLB_F64_SPLIT", split)
+        sim = RLB(nx, ny, nz, tau, c_l=c_l, precision="fp64", device="cuda:0")
+        sim.load_state(sim.cells_to_state(torch.from_numpy(a).cuda()))
+        sim.step(1)
+        outs.append((sim.state()[:, :sim.N].clone(), sim.stats()))
+        got = sim.state_to_cells(sim.state()).cpu().numpy()
+        sim.close()
+    assert torch.equal(outs[0][0].view(torch.int64), outs[1][0].view(torch.int64))
+    assert outs[0][1] == outs[1][1]
+    s = outs[0][1]
+    assert s["n_unphysical"] == stats.n_unphysical > 0 and s["first_bad"] == stats.first_bad
+    assert s["n_nonpositive_eq"] == stats.n_nonpositive_eq
+    E, M = h[..., 1, :].sum(-1), c_l * (h[..., 1, :] @ EV.astype(float))
+    # |beta| < 0.985, the range of the bound (|M|^2 < 0.986 E^2 there)
+    physical = (E > 0) & ((M * M).sum(-1) < 0.985 * E * E)
+    assert 0.6 < physical.mean() < 1
+    # f scales with its own largest population, g with its own
+    for s_ in range(2):
+        big = np.abs(h[..., s_, :]).max(-1)[physical]
+        err = np.abs(got[..., s_, :] - ref[..., s_, :])[physical].max(-1)
+        assert np.all(err <= UNITS * 2.0 ** -53 * big), (s_, (err / big).max() * 2.0 ** 53)
