@@ -22,8 +22,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(HERE, "_build")
-SOURCES = ["rlb_forward.cu", "rlb_step64.cu", "rlb_stream.cu", "rlb_adjoint.cu", "rlb_eos.cu", "rlb_f64df.cu", "rlb_api.cu"]
-HEADERS = ["rlb_internal.h", "rlb_device.cuh", "rlb_collide.cuh", "rlb_tma.cuh", "rlb_dfloat.cuh", "rlb_fixed.cuh"]
+SOURCES = ["rlb_forward.cu", "rlb_step64.cu", "rlb_fields.cu", "rlb_stream.cu", "rlb_adjoint.cu", "rlb_eos.cu", "rlb_f64df.cu", "rlb_api.cu"]
+HEADERS = ["rlb_internal.h", "rlb_device.cuh", "rlb_collide.cuh", "rlb_tma.cuh", "rlb_dfloat.cuh", "rlb_fixed.cuh", "rlb_fixed_host.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: no implicit a*b+c contraction, so every kernel computes exactly
 # the operations its source writes (fused ones are explicit fma/fmaf calls) and

@@ -271,6 +271,7 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
     ph.m3cl2 = -3.0 * p->c_l * p->c_l;
     ph.three_cl = 3.0 * p->c_l;
     ph.fx = make_fx_run(ph.omega, p->c_l);
+    ph.fi = make_fx_init(ph, p->prec);
     // the fixed-point FP64 step: measured closer to the exact values than the
     // binary64 one for lattice speeds up to 3 (rlb_fixed.cuh); its cell
     // offsets are 32-bit byte counts
@@ -677,10 +678,10 @@ rlb_status rlb_debug_bounds_violations(int64_t* count) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "cudaDeviceSynchronize");
     const unsigned long long a = oob_take_forward(), b = oob_take_adjoint(), d = oob_take_eos(), e2 = oob_take_stream(),
-                             h = oob_take_step64();
-    if (a == ~0ull || b == ~0ull || d == ~0ull || e2 == ~0ull || h == ~0ull)
+                             h = oob_take_step64(), k = oob_take_fields();
+    if (a == ~0ull || b == ~0ull || d == ~0ull || e2 == ~0ull || h == ~0ull || k == ~0ull)
         return fail(nullptr, RLB_ERR_CUDA, "reading the bounds counters failed");
-    *count = (int64_t)(a + b + d + e2 + h);
+    *count = (int64_t)(a + b + d + e2 + h + k);
     return RLB_OK;
 #else
     *count = -1;

@@ -31,11 +31,11 @@
 // functions compile for the host as well (checks of the arithmetic).
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
 #ifndef __CUDACC__
-#include <math.h>
 #define RLB_FX static inline
 #else
 #define RLB_FX __host__ __device__ __forceinline__
@@ -65,6 +65,24 @@ struct FxRun {
     float q_scale;  // beta = q_scale x (high word of w)
     float c_l;
 };
+
+// Per-run constants of the equilibrium initialisation (make_fx_init).
+struct FxInit {
+    FxConst k6;    // 1 / (6 c_l^2)               x 2^65
+    FxConst kEp;   // 1 / (108 c_l^2)             x 2^65
+    FxConst k29;   // 2 / 9                       x 2^62
+    FxConst kU;    // 2 c_l / 3                   x 2^(62 - sU)
+    FxConst kQ, kG;  // as in FxRun
+    FxConst k0;    // (1 - 2 / (3 c_l^2)) / 3     x 2^64
+    FxConst kS;    // 1 / 36                      x 2^65
+    FxConst kS12;  // 1 / (12 c_l)                x 2^65
+    double rf, rg, rg0;  // reference populations: diagonal f and g, rest g
+    int sU, on;
+    int lo, hi;      // high words between which n and eps have to lie
+    int re_f, re_g;  // least exponents of S and eps gamma^2 against the reference
+};
+
+#include "rlb_fixed_host.h"
 
 RLB_FX int32_t fx_hi(double v) {
 #ifdef __CUDA_ARCH__

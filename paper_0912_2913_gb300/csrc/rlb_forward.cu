@@ -195,125 +195,6 @@ __global__ void __launch_bounds__(256, 3) k_step_f32_pipe(const float* __restric
     }
 }
 
-// ---------------------------------------------------------------------------
-// Equilibria of given fields in FP64 (initialisation and inflow plane):
-// Eqs. (equil1s), (equil2as), (equil2bs).
-// ---------------------------------------------------------------------------
-__device__ void equilibrium_f64(double n, double eps, double bx, double by, double bz, const Phys& ph, double* f,
-                                double* g) {
-    const double b2 = bx * bx + by * by + bz * bz;
-    const double gam2 = 1.0 / (1.0 - b2);
-    const double ng = n * sqrt(gam2);
-    const double eg = eps * gam2;
-    const double q[9] = {bx, by, bz, bx + by, bx - by, bx + bz, bx - bz, by + bz, by - bz};
-    f[0] = kW0 * ng;
-    g[0] = kW0 * (4.0 * eg - eps * (2.0 * ph.inv_cl2 + 1.0) - 2.0 * eg * b2 * ph.inv_cl2);
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        const double w = pair_w(p);
-        const double fa = 3.0 * q[p] * ph.inv_cl;
-        f[2 * p + 1] = w * ng * (1.0 + fa);
-        f[2 * p + 2] = w * ng * (1.0 - fa);
-        const double gs = eps * ph.inv_cl2 + eg * (6.0 * q[p] * q[p] - 2.0 * b2) * ph.inv_cl2;
-        const double ga = eg * 4.0 * q[p] * ph.inv_cl;
-        g[2 * p + 1] = w * (gs + ga);
-        g[2 * p + 2] = w * (gs - ga);
-    }
-}
-
-// Rest equilibrium of the FP32 deviation reference.
-__device__ __forceinline__ void reference_eq(const Phys& ph, double* fr, double* gr) {
-    fr[0] = kW0 * ph.n_ref;
-    gr[0] = kW0 * ph.eps_ref * (3.0 - 2.0 * ph.inv_cl2);
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-        const double w = pair_w(p);
-        fr[2 * p + 1] = fr[2 * p + 2] = w * ph.n_ref;
-        gr[2 * p + 1] = gr[2 * p + 2] = w * ph.eps_ref * ph.inv_cl2;
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128) k_init(const double* __restrict__ n, const double* __restrict__ eps,
-                                              const double* __restrict__ beta, const uint8_t* __restrict__ solid,
-                                              T* __restrict__ A, T* __restrict__ B, Geom g, Phys ph) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= g.N) return;
-    const long long S = g.S;
-    if (solid && solid[idx]) {
-        T m;
-        if constexpr (sizeof(T) == 8) m = solid_marker_d(); else m = solid_marker_f();
-        for (int q = 0; q < 38; ++q) A[RLB_CHK(q * S + idx, 38ll * S)] = B[RLB_CHK(q * S + idx, 38ll * S)] = m;
-        return;
-    }
-    const int x = idx % g.nx;
-    double f[19], gg[19];
-    if (g.xbc == XBC_INFLOW_OUTFLOW && x == 0)
-        equilibrium_f64(ph.n_in, ph.eps_in, ph.beta_in[0], ph.beta_in[1], ph.beta_in[2], ph, f, gg);
-    else
-        equilibrium_f64(n[idx], eps[idx], beta[idx], beta[g.N + idx], beta[2 * (long long)g.N + idx], ph, f, gg);
-    if constexpr (sizeof(T) == 4) {
-        double fr[19], gr[19];
-        reference_eq(ph, fr, gr);
-        for (int i = 0; i < 19; ++i) {
-            f[i] -= fr[i];
-            gg[i] -= gr[i];
-        }
-    }
-    for (int i = 0; i < 19; ++i) {
-        A[RLB_CHK(i * S + idx, 38ll * S)] = B[RLB_CHK(i * S + idx, 38ll * S)] = (T)f[i];
-        A[RLB_CHK((19 + i) * S + idx, 38ll * S)] = B[RLB_CHK((19 + i) * S + idx, 38ll * S)] = (T)gg[i];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Macroscopic output of a stored state (no gather: the moments of the
-// post-collision populations equal those of the gathered ones, the
-// collision conserves them).  IEEE sqrt and division.
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(128) k_macro(const T* __restrict__ A, double* __restrict__ n,
-                                               double* __restrict__ eps, double* __restrict__ beta, Geom g,
-                                               Phys ph, unsigned long long* bad_count) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= g.N) return;
-    const long long S = g.S;
-    if (is_solid(A[RLB_CHK(idx, 38ll * S)])) {
-        const double nan = __longlong_as_double(0x7FF8000000000000ll);
-        n[idx] = eps[idx] = beta[idx] = beta[g.N + idx] = beta[2 * (long long)g.N + idx] = nan;
-        return;
-    }
-    double f[19], gg[19];
-    for (int i = 0; i < 19; ++i) {
-        f[i] = (double)A[RLB_CHK(i * S + idx, 38ll * S)];
-        gg[i] = (double)A[RLB_CHK((19 + i) * S + idx, 38ll * S)];
-    }
-    double sf, E, mx, my, mz;
-    moments_pairs(f, gg, sf, E, mx, my, mz);
-    if constexpr (sizeof(T) == 4) {
-        sf += ph.n_ref;
-        E += ph.eps_ref;
-    }
-    mx *= ph.c_l;
-    my *= ph.c_l;
-    mz *= ph.c_l;
-    const double m2 = mx * mx + my * my + mz * mz;
-    const double disc = 4.0 * E * E - 3.0 * m2;
-    const double e = sqrt(disc) - E;
-    const double D = 3.0 * E + e;
-    const double bx = 3.0 * mx / D, by = 3.0 * my / D, bz = 3.0 * mz / D;
-    const double b2 = bx * bx + by * by + bz * bz;
-    const double nn = sf * sqrt(1.0 - b2);
-    n[idx] = nn;
-    eps[idx] = e;
-    beta[idx] = bx;
-    beta[g.N + idx] = by;
-    beta[2 * (long long)g.N + idx] = bz;
-    const bool bad = !(pos_finite(sf) && pos_finite(E) && nonneg_finite(disc) && pos_finite(e) && below_one(b2) &&
-                       pos_finite(nn));
-    if (bad) atomicAdd(bad_count, 1ull);
-}
-
 __global__ void k_conversions(const float* __restrict__ fi, const double* __restrict__ di, long long n,
                               double* __restrict__ fo, float* __restrict__ dout) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
@@ -403,16 +284,6 @@ Dev32 make_dev32(const Phys& ph) {
     c.inv_cl_d = ph.inv_cl;
     c.inv_cl2_d = ph.inv_cl2;
     return c;
-}
-
-cudaError_t launch_init(int prec, const Geom& g, const Phys& ph, const double* n, const double* eps,
-                        const double* beta, const uint8_t* solid, void* A, void* B, cudaStream_t st) {
-    g_last_launches = 1;
-    if (prec == 0)
-        k_init<double><<<blocks_for(g.N, 128), 128, 0, st>>>(n, eps, beta, solid, (double*)A, (double*)B, g, ph);
-    else
-        k_init<float><<<blocks_for(g.N, 128), 128, 0, st>>>(n, eps, beta, solid, (float*)A, (float*)B, g, ph);
-    return cudaGetLastError();
 }
 
 static int sm_count() {
@@ -535,16 +406,6 @@ cudaError_t launch_step(int prec, const Geom& g, const Phys& ph, const void* A, 
             break;
         default: launch_step_t<XBC_OUTFLOW_BOTH, true>(prec, g, ph, A, B, cnt, count, step_index, st); break;
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_macro(int prec, const Geom& g, const Phys& ph, const void* A, double* n, double* eps,
-                         double* beta, Counters cnt, cudaStream_t st) {
-    g_last_launches = 1;
-    if (prec == 0)
-        k_macro<double><<<blocks_for(g.N, 128), 128, 0, st>>>((const double*)A, n, eps, beta, g, ph, cnt.macro_bad);
-    else
-        k_macro<float><<<blocks_for(g.N, 128), 128, 0, st>>>((const float*)A, n, eps, beta, g, ph, cnt.macro_bad);
     return cudaGetLastError();
 }
 

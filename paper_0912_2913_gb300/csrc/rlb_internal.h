@@ -63,6 +63,7 @@ struct Phys {
     // -3 c_l^2 and 3 c_l for the recovery from M / c_l.
     double c_k1[2], c_k2[2], c_k3[2], c_fs[2], c_fa[2], c_f0, c_g0[3], m3cl2, three_cl;
     FxRun fx;   // constants of the fixed-point FP64 step
+    FxInit fi;  // constants of the fixed-point initialisation
     int fx_on;  // 1: the FP64 step runs in block fixed point
 };
 
@@ -94,6 +95,8 @@ cudaError_t launch_step_f64(const Geom& g, const Phys& ph, const void* A, void* 
                             long long step_index, cudaStream_t stream);
 // Constants of the fixed-point FP64 step.
 FxRun make_fx_run(double omega, double c_l);
+// Constants of the fixed-point initialisation (c_l and the reference of ph).
+FxInit make_fx_init(const Phys& ph, int prec);
 // FP64 step with its arithmetic in compensated binary32 pairs (rlb_f64df.cu).
 cudaError_t launch_step_f64_df(const Geom& g, const Phys& ph, const void* A, void* B, Counters cnt, bool count,
                                long long step_index, cudaStream_t stream, int threads);
@@ -156,6 +159,7 @@ unsigned long long oob_take_adjoint();
 unsigned long long oob_take_eos();
 unsigned long long oob_take_stream();
 unsigned long long oob_take_step64();
+unsigned long long oob_take_fields();
 #ifdef RLB_CHECK_BOUNDS
 // Runs the index check on (i, n) in a kernel; returns the checked index.
 long long bounds_selftest(long long i, long long n, cudaStream_t s);

@@ -684,17 +684,6 @@ __global__ void __launch_bounds__(128)
 // ---------------------------------------------------------------------------
 namespace {
 
-// (hi + lo) 2^s as a split constant; |value| < 2^63
-FxConst fx_const(double hi, double lo, int s) {
-    const int64_t v = (int64_t)ldexp(hi, s) + (int64_t)llrint(ldexp(lo, s));
-    return {(int32_t)(v >> 32), (int32_t)((uint32_t)v >> 1)};
-}
-// a / b as an unevaluated pair (b exact)
-void div2(double a, double b, double& hi, double& lo) {
-    hi = a / b;
-    lo = fma(-hi, b, a) / b;
-}
-
 template <int XBC>
 void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B, Counters cnt, bool count,
                        long long step_index, cudaStream_t st) {
@@ -738,20 +727,20 @@ void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B
 FxRun make_fx_run(double omega, double c_l) {
     FxRun k;
     double qh, ql, th, tl, c2h = c_l * c_l, c2l = fma(c_l, c_l, -c2h);
-    div2(omega, 36.0, qh, ql);
+    fx_div2(omega, 36.0, qh, ql);
     th = qh / c2h;
     tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
     k.kE = fx_const(th, tl, 65);
     k.kS = fx_const(qh, ql, 65);
-    div2(omega, 12.0, qh, ql);
+    fx_div2(omega, 12.0, qh, ql);
     k.kU = fx_const(qh, ql, 65);
     // omega (1 - 2 / (3 c_l^2)) = omega - 24 omega / (36 c_l^2)
     const int64_t kE65 = (int64_t)ldexp(th, 65) + (int64_t)llrint(ldexp(tl, 65));
     const int64_t v = (int64_t)ldexp(omega, 62) - 3 * kE65;
     k.k0 = {(int32_t)(v >> 32), (int32_t)((uint32_t)v >> 1)};
-    div2(5.0, 9.0, qh, ql);
+    fx_div2(5.0, 9.0, qh, ql);
     k.kQ = fx_const(qh, ql, 63);
-    div2(1.0, 6.0, qh, ql);
+    fx_div2(1.0, 6.0, qh, ql);
     k.kG = fx_const(qh, ql, 63);
     k.om4 = 0.25 * omega;
     k.omw = 1.0 - omega;
