@@ -213,12 +213,14 @@ RLB_API rlb_status rlb_adjoint_step(rlb_ctx* ctx, const void* state_t, const voi
  * or memory pool that owns all device memory, or a real-time loop that must
  * not synchronise (cudaMalloc/cudaFree can synchronise the device).
  * Same arguments, results and errors as rlb_adjoint_step, and the same
- * kernels: FP64 the persistent register kernel (SMs x 2 blocks), FP32 the
+ * kernels: FP64 the fixed-point kernel (SMs x 6 blocks of 64, or eight lanes
+ * per cell on small lattices; outside 1 <= c_l <= 2 the persistent register
+ * kernel, SMs x 2 blocks of 128), FP32 the
  * persistent shared-memory staged kernel (SMs x 3 blocks of 128; with
  * RLB_ADJ_PIPE=0 or 1 the persistent register kernel, SMs x 4 blocks), grids
- * capped at N/128 blocks.  The per-warp partial sums live in one static
+ * capped at the lattice's block count.  The per-warp partial sums live in one static
  * device array of 32768 doubles (256 KiB) per device: a launch that would
- * need more (16 doubles per block) returns RLB_ERR_ARG and enqueues nothing;
+ * need more (4 doubles per warp) returns RLB_ERR_ARG and enqueues nothing;
  * every launch writes all the slots it reads, so nothing needs to start at
  * zero.  The first call on each device (and the first after the device's
  * context was reset) does the set-up: it takes the array's address and loads

@@ -29,6 +29,7 @@
 #include <mutex>
 
 #include "rlb_device.cuh"
+#include "rlb_fixed.cuh"
 
 namespace rlb {
 
@@ -825,6 +826,656 @@ __global__ void __launch_bounds__(128, MINB)
 }
 
 // ---------------------------------------------------------------------------
+// FP64 step adjoint with its sums in 64-bit fixed point (rlb_fixed.cuh),
+// lattice speeds 1 <= c_l <= 2.
+//
+// With d = M / c_l, D = 2 E + s, s = sqrt(4 E^2 - 3 M^2), u = d / D and the
+// equilibria written as in rlb_fixed.cuh, mu enters through integer moments
+// (weights times 36): S1 = sum w sigma_p, T = sum w sigma_p e_p e_p^T,
+// V = sum w delta_p e_p over the g pairs, F1 and F likewise over the f pairs:
+//   G     = 13.5 T + (1.5 w0 mu_0 - 7.5 S1) I,     y = G u,
+//   a_E   = S1 / c_l^2 + w0 mu_0 (3 - 2 / c_l^2),
+//   a_S   = w0 mu_f0 + F1 + 9 F.u,
+//   a_D   = -(u.y + 9 (S / D) F.u),
+//   v_E   = a_E + a_D (2 + 4 E / s),
+//   v_d   = 2 y + 3 V + 9 (S / D) F - 3 c_l^2 (a_D / s) d,
+//   nu_f  = (1 - omega) mu_f + omega a_S,
+//   nu_g  = (1 - omega) mu_g + omega (v_E + e_i.v_d),
+//   sum mu eq = S a_S + E a_E + D u.y + 3 V.d,
+// no gamma^2, 1 / (1 - b2) or weights per population.  sum mu h is an integer
+// dot product.
+//
+// k_adjoint_step<double> (the other lattice speeds) issues 408 FP64
+// instructions per collided cell, 26,500 clocks of a scheduler's FP64 pipe per
+// 32 cells, against 5,400 for the cell's 912 bytes at the HBM rate; here 110
+// remain (72 for recovery and algebra, 38 relaxations) beside 6,000
+// instructions in all.  What bounds it now is the speed of a warp: with 12
+// warps per SM 46 % of the issue slots and 51 % of the FP64 pipe are used, the
+// rest being instruction latency and fetch.  mu and the gathered populations
+// are staged in a shared-memory column per thread by asynchronous copies, so
+// that they hold no registers, and the velocity pairs are walked in three
+// rounds by one loop body (a third of the code to fetch).  200x100x100 sphere
+// 1.51 -> 0.85 ms, 192^3 box 5.1 -> 2.35 ms; blocks of 64 threads: 5, 6 and 7
+// per SM 2.65, 2.35 and 2.49 ms; all values in registers and unrolled, 3
+// blocks of 128: 2.35 ms on the box, 0.854 on the sphere.
+// Error against 113-bit references: nu 1.2e-16 (2 to 3e-16 before), the terms
+// of dL/dtau 7.4e-17 rms and below 3e-17 in the mean (1.5e-16 and 7e-17).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async4(uint32_t saddr, const void* gptr) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(gptr) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t saddr, const void* gptr) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(saddr), "l"(gptr) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gptr) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+struct AdjFx {
+    FxConst kS1;  // 5 / 3                        x 2^62
+    FxConst kE1;  // 1 / (36 c_l^2)               x 2^65
+    FxConst kE0;  // (3 - 2 / c_l^2) / 3          x 2^62
+    FxConst kS36;  // 1 / 36                      x 2^65
+};
+
+// A cell in binary64 throughout (any state); the terms of dL/dtau returned.
+template <int XBC>
+__device__ __noinline__ double adjoint_cell_general(const double* A, const double* Lin, double* Lout, const Geom& g,
+                                                    const AdjConst<double>& c, int idx) {
+    const long long S = g.S;
+    int x, y, z;
+    cell_coords(g, idx, x, y, z);
+    const PullOffsets o(g, x, y, z);
+    const int dup = dup_of<XBC>(x, g.nx);
+    auto load_mu = [&](double* mu, int base) {
+#pragma unroll
+        for (int i = 0; i < 19; ++i) mu[i] = Lin[RLB_CHK((base + i) * S + idx, 38ll * S)];
+        if (dup) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx + dup, 38ll * S)];
+        }
+    };
+    unsigned bounced = 0u;
+    double h[19], mug[19], muf[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) h[i] = A[RLB_CHK((19 + i) * S + idx + o.src(i), 38ll * S)];
+#pragma unroll
+    for (int i = 1; i < 19; ++i) {
+        if (is_solid(h[i])) {
+            bounced |= 1u << i;
+            h[i] = A[RLB_CHK((19 + opp(i)) * S + idx, 38ll * S)];
+        }
+    }
+    load_mu(mug, 19);
+    CellG<double> r;
+    cell_g64(h, mug, c, r);
+#pragma unroll
+    for (int i = 0; i < 19; ++i)
+        h[i] = (bounced >> i) & 1u ? A[RLB_CHK(opp(i) * S + idx, 38ll * S)] : A[RLB_CHK(i * S + idx + o.src(i), 38ll * S)];
+    load_mu(muf, 0);
+    double tf, aS, fbx, fby, fbz, vE, vx, vy, vz;
+    cell_f64(h, muf, r, c, tf, aS, fbx, fby, fbz);
+    recovery_adjoint64(r.ae, fbx + r.gbx, fby + r.gby, fbz + r.gbz, r, c, vE, vx, vy, vz);
+    scatter_cell64(muf, mug, aS, vE, vx, vy, vz, c, [&](int q, int i, double v) {
+        if ((bounced >> i) & 1u)
+            Lout[RLB_CHK((q - i + opp(i)) * S + idx, 38ll * S)] = v;
+        else
+            Lout[RLB_CHK(q * S + idx + o.src(i), 38ll * S)] = v;
+    });
+    return (r.tacc + tf) * c.inv_tau2;
+}
+
+// What the f phase and the output need of a cell (see the formulas above).
+struct AdjFxCell {
+    double x, y, z, E4, rs, rD, ux, uy, uz, yx, yy, yz, uy_, vx, vy, vz, aE;  // d, 4 E, 1/s, 1/D, u, G u, u.y, 36 V, a_E
+    double tsum;                      // sum mu (h - eq)
+    double nuE, nuS, tx, ty, tz;      // omega v_E, omega a_S, omega v_d
+};
+
+// Recovery and the g moments of mu in binary64.  S*, P*, T*: the sums of
+// sigma_p over the axis pairs (doubled), and over each plane's two diagonal
+// pairs and their difference; units 2^-56 of the block exponents eh, em.
+__device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int64_t dz, int64_t dot, int64_t m0, int64_t Sx,
+                                         int64_t Sy, int64_t Sz, int64_t Pxy, int64_t Pyz, int64_t Pzx, int64_t Txy,
+                                         int64_t Tyz, int64_t Tzx, int64_t Vx, int64_t Vy, int64_t Vz, int eh, int em,
+                                         const Phys& ph, const AdjFx& k, AdjFxCell& t) {
+    const int kh = eh - 1079, km = em - 1079;
+    const double Ed = fx_to(E, kh);
+    t.x = fx_to(dx, kh), t.y = fx_to(dy, kh), t.z = fx_to(dz, kh);
+    const double E2 = Ed + Ed;
+    t.E4 = E2 + E2;
+    const double dd = fma(t.x, t.x, fma(t.y, t.y, t.z * t.z));
+    const double disc = fma(ph.fx.m3cl2, dd, E2 * E2);
+    double ys, hs;
+    rsqrt_seed(disc, ys, hs);
+    double sq = disc * ys;
+    sq = fma(fma(-sq, sq, disc), hs, sq);
+    sq = fma(fma(-sq, sq, disc), hs, sq);
+    const double e1 = fma(-sq, ys, 1.0);
+    t.rs = fma(ys, fma(e1, e1, e1), ys);
+    const double D = E2 + sq;
+    const double r0 = rcp_seed(D);
+    const double e2 = fma(-D, r0, 1.0);
+    t.rD = fma(r0, fma(e2, e2, e2), r0);
+    t.ux = t.x * t.rD, t.uy = t.y * t.rD, t.uz = t.z * t.rD;
+    const FxSplit sp = fx_split((Sx + Sy + Sz) + (Pxy + Pyz + Pzx));
+    // 8 G: 13.5 / 36 = 3/8; the partial sums may wrap, the result does not
+    const int64_t kap = (m0 << 2) - (fx_mul(sp, k.kS1) << 2) + 4;
+    auto g38 = [](int64_t v, int64_t k8) { return (v + (v << 1) + k8) >> 3; };
+    const double Gxx = fx_to(g38(Sx + Pxy + Pzx, kap), km), Gyy = fx_to(g38(Sy + Pxy + Pyz, kap), km),
+                 Gzz = fx_to(g38(Sz + Pyz + Pzx, kap), km);
+    const double Gxy = fx_to(g38(Txy, 4), km), Gxz = fx_to(g38(Tzx, 4), km), Gyz = fx_to(g38(Tyz, 4), km);
+    t.yx = fma(Gxx, t.ux, fma(Gxy, t.uy, Gxz * t.uz));
+    t.yy = fma(Gxy, t.ux, fma(Gyy, t.uy, Gyz * t.uz));
+    t.yz = fma(Gxz, t.ux, fma(Gyz, t.uy, Gzz * t.uz));
+    t.aE = fx_to(fx_mul(sp, k.kE1) + fx_mul(fx_split(m0 << 3), k.kE0), km - 1);
+    t.uy_ = fma(t.ux, t.yx, fma(t.uy, t.yy, t.uz * t.yz));
+    t.vx = fx_to(Vx, km), t.vy = fx_to(Vy, km), t.vz = fx_to(Vz, km);
+    const double Vd = fma(t.vx, t.x, fma(t.vy, t.y, t.vz * t.z));
+    t.tsum = fx_to(dot, em + eh - 2102) - fma(Ed, t.aE, fma(D, t.uy_, Vd * (1.0 / 12.0)));
+}
+
+// The f moments (36 w0 mu_f0 + F1 and F times 36, S, the dot product) and the
+// coefficients of the output.
+__device__ __forceinline__ void adj_fx_f(int64_t Sf, int64_t fd, int64_t Fs, int64_t Fx, int64_t Fy, int64_t Fz, int fh,
+                                         int ef, const Phys& ph, const AdjFx& k, AdjFxCell& t) {
+    const double Sd = fx_to(Sf, fh - 1079);
+    const int kf = ef - 1079;
+    const double fx = fx_to(Fx, kf), fy = fx_to(Fy, kf), fz = fx_to(Fz, kf);
+    const double Fu = fma(fx, t.ux, fma(fy, t.uy, fz * t.uz));
+    const double aS = fma(0.25, Fu, fx_to(fx_mul(fx_split(Fs), k.kS36), kf - 1));
+    t.tsum += fx_to(fd, ef + fh - 2102) - Sd * aS;
+    const double sD = (0.25 * Sd) * t.rD;
+    const double aD = -fma(sD, Fu, t.uy_);
+    t.nuE = ph.omega * fma(aD, fma(t.E4, t.rs, 2.0), t.aE);
+    t.nuS = ph.omega * aS;
+    const double c2 = (ph.fx.m3cl2 * t.rs) * aD;
+    t.tx = ph.omega * fma(2.0, t.yx, fma(t.vx, 1.0 / 12.0, fma(sD, fx, c2 * t.x)));
+    t.ty = ph.omega * fma(2.0, t.yy, fma(t.vy, 1.0 / 12.0, fma(sD, fy, c2 * t.y)));
+    t.tz = ph.omega * fma(2.0, t.yz, fma(t.vz, 1.0 / 12.0, fma(sD, fz, c2 * t.z)));
+}
+
+// The 18 moving velocities as three rounds r = 0, 1, 2 over the axes
+// (a, b) = (x, y), (y, z), (z, x): the axis pair of a and the two diagonal
+// pairs of the plane (a, b).  Velocity numbers of a round: +-a at ax, ax + 1;
+// (+,+) and (-,-) at pp, pp + 1; (+,-) at pm and (-,+) at mp.
+struct Round {
+    int ax, pp, pm, mp;
+    __device__ __forceinline__ explicit Round(int r)
+        : ax(1 + 2 * r), pp((0x0B0F07 >> (8 * r)) & 0xFF), pm((0x0E1109 >> (8 * r)) & 0xFF),
+          mp((0x0D120A >> (8 * r)) & 0xFF) {}
+};
+__device__ __forceinline__ int opp_rt(int i) { return ((i - 1) ^ 1) + 1; }  // i > 0
+template <typename V>
+__device__ __forceinline__ void rotate3(V& a, V& b, V& c) {
+    const V t = a;
+    a = b;
+    b = c;
+    c = t;
+}
+
+constexpr int kAdjFxThreads = 64;  // threads per block (columns of the staging area)
+constexpr int kAdjFxBlocks = 6;    // resident blocks per SM
+
+template <int XBC>
+__global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
+    k_adjoint_step_fx(const double* __restrict__ A, const double* __restrict__ Lin, double* __restrict__ Lout,
+                      const __grid_constant__ Geom g, const __grid_constant__ Phys ph,
+                      const __grid_constant__ AdjConst<double> c, const __grid_constant__ AdjFx k, double* red,
+                      const double* __restrict__ inflow_t) {
+    const long long S = g.S;
+    // This thread's column: mu_f (0..18), mu_g (19..37), then h_g and later
+    // h_f (38..56).  No other thread reads it.
+    __shared__ double col[57][kAdjFxThreads];
+    const int tid = threadIdx.x;
+    const uint32_t scol = (uint32_t)__cvta_generic_to_shared(&col[0][tid]);
+    auto stage = [&](int slot, const double* p) { cp_async8(scol + (uint32_t)(slot * kAdjFxThreads * 8), p); };
+    double tau_acc = 0;
+    double bin0 = 0.0, bin1 = 0.0, bin2 = 0.0;
+    bool has_b = false;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long li = (long long)blockIdx.x * blockDim.x + tid; li < g.N; li += stride) {
+        const int idx = (int)li;
+        int x, y, z;
+        cell_coords(g, idx, x, y, z);
+        if constexpr (XBC == XBC_INFLOW_OUTFLOW) {
+            // dL/dbeta_in at the fluid inflow ghosts of this warp, their 38
+            // products with the table spread over the active lanes
+            const unsigned act = __activemask();
+            unsigned m = __ballot_sync(act, x == 0 && !is_solid(A[RLB_CHK(idx, 38ll * S)]));
+            if (m) {
+                const int lane = tid & 31;
+                const int rank = __popc(act & ((1u << lane) - 1u)), cnt = __popc(act);
+                while (m) {
+                    const int src = __ffs(m) - 1;
+                    m &= m - 1;
+                    const int gidx = __shfl_sync(act, idx, src);
+                    for (int q = rank; q < 38; q += cnt) {
+                        const double l = Lin[RLB_CHK((long long)q * S + gidx, 38ll * S)];
+                        bin0 = fma(l, inflow_t[3 * q + 0], bin0);
+                        bin1 = fma(l, inflow_t[3 * q + 1], bin1);
+                        bin2 = fma(l, inflow_t[3 * q + 2], bin2);
+                    }
+                    has_b = true;
+                }
+            }
+        }
+        if ((XBC != XBC_PERIODIC) && (x == 0 || x == g.nx - 1)) {
+            const int inward = x == 0 ? 1 : -1;
+#pragma unroll 1
+            for (int i = 0; i < 19; ++i) {
+                if (vel_x(i) != inward) {
+                    Lout[RLB_CHK(i * S + idx, 38ll * S)] = 0.0;
+                    Lout[RLB_CHK((19 + i) * S + idx, 38ll * S)] = 0.0;
+                }
+            }
+            continue;
+        }
+        const PullOffsets o(g, x, y, z);
+        const int dup = dup_of<XBC>(x, g.nx);
+        const double* Ac = A + idx;
+        const double* Lc = Lin + idx;
+        // offsets of the sources x - e along the axes: minus and plus
+        int am = o.xm, ap = o.xp, bm = o.ym, bp = o.yp, cm = o.zm, cp = o.zp;
+        auto gather = [&](int base) {  // the 19 pulled populations of a set
+            stage(38, Ac + RLB_CHK_OFF(base * S, idx, 38ll * S));
+#pragma unroll 1
+            for (int r = 0; r < 3; ++r) {
+                const Round v(r);
+                auto one = [&](int i, int off) { stage(38 + i, Ac + RLB_CHK_OFF((base + i) * S + off, idx, 38ll * S)); };
+                one(v.ax, am);
+                one(v.ax + 1, ap);
+                one(v.pp, am + bm);
+                one(v.pp + 1, ap + bp);
+                one(v.pm, am + bp);
+                one(v.mp, ap + bm);
+                rotate3(am, bm, cm);
+                rotate3(ap, bp, cp);
+            }
+        };
+        gather(19);
+#pragma unroll 1
+        for (int q = 19; q < 38; ++q) stage(q, Lc + RLB_CHK_OFF(q * S, idx, 38ll * S));
+        cp_async_commit();
+#pragma unroll 1
+        for (int q = 0; q < 19; ++q) stage(q, Lc + RLB_CHK_OFF(q * S, idx, 38ll * S));
+        cp_async_commit();
+        cp_async_wait<1>();
+        if (is_solid(col[38][tid])) {  // never updated: identity
+            cp_async_wait<0>();
+#pragma unroll 1
+            for (int q = 0; q < 38; ++q) Lout[RLB_CHK(q * S + idx, 38ll * S)] = col[q][tid];
+            continue;
+        }
+        auto max_exp = [&](int base) {
+            uint32_t m = 0;
+#pragma unroll 4
+            for (int i = 0; i < 19; ++i) m = max(m, (uint32_t)__double2hiint(col[base + i][tid]) << 1);
+            return (int)(m >> 21);
+        };
+        // mu also takes lambda of the outflow ghost that copies x
+        auto add_dup = [&](int base) {
+#pragma unroll 4
+            for (int i = 0; i < 19; ++i) col[base + i][tid] += Lc[RLB_CHK_OFF((base + i) * S + dup, idx, 38ll * S)];
+        };
+        int eh = max_exp(38);
+        unsigned bounced = 0u;
+        if (eh == 0x7FF) {  // links to solid cells, or a non-finite population
+#pragma unroll 1
+            for (int i = 1; i < 19; ++i) {
+                if (is_solid(col[38 + i][tid])) {
+                    bounced |= 1u << i;
+                    col[38 + i][tid] = Ac[RLB_CHK_OFF((19 + opp_rt(i)) * S, idx, 38ll * S)];
+                }
+            }
+            eh = max_exp(38);
+        }
+        if (dup) add_dup(19);
+        // ---- g: moments of h and mu, their dot product
+        int em = max_exp(19);
+        bool ok = eh >= 100 && eh <= 1900 && em <= 1900;
+        em = em < 100 ? 100 : em;
+        int64_t E, dx = 0, dy = 0, dz = 0, m0;
+        FxDot dot{};
+        // moments of mu: axis sums, plane sums and differences (xy, yz, zx), V
+        int64_t Sx = 0, Sy = 0, Sz = 0, Pxy = 0, Pyz = 0, Pzx = 0, Txy = 0, Tyz = 0, Tzx = 0, Vx = 0, Vy = 0, Vz = 0;
+        {
+            const int64_t h0 = fx_from(col[38][tid], eh), u0 = fx_from(col[19][tid], em);
+            E = fx_round4(h0);
+            m0 = fx_round4(u0);
+            dot.add(fx_split(h0), fx_split(u0));
+#pragma unroll 1
+            for (int r = 0; r < 3; ++r) {
+                const Round v(r);
+                int64_t d, sg, dl;
+                auto pair = [&](int i, int j) {
+                    const int64_t a = fx_from(col[38 + i][tid], eh), b = fx_from(col[38 + j][tid], eh);
+                    const int64_t ua = fx_from(col[19 + i][tid], em), ub = fx_from(col[19 + j][tid], em);
+                    E += fx_round4(a + b);
+                    dot.add(fx_split(a), fx_split(ua));
+                    dot.add(fx_split(b), fx_split(ub));
+                    d = fx_round4(a - b);
+                    sg = fx_round4(ua + ub);
+                    dl = fx_round4(ua - ub);
+                };
+                pair(v.ax, v.ax + 1);
+                dx += d;
+                Sx = sg << 1;
+                Vx += dl << 1;
+                pair(v.pp, v.pp + 1);
+                dx += d, dy += d;
+                Vx += dl, Vy += dl;
+                Pxy = sg, Txy = sg;
+                pair(v.pm, v.mp);
+                dx += d, dy -= d;
+                Vx += dl, Vy -= dl;
+                Pxy += sg, Txy -= sg;
+                rotate3(dx, dy, dz);
+                rotate3(Sx, Sy, Sz);
+                rotate3(Vx, Vy, Vz);
+                rotate3(Pxy, Pyz, Pzx);
+                rotate3(Txy, Tyz, Tzx);
+            }
+        }
+        gather(0);  // the h_f slots: every h_g of this column has been read
+        cp_async_commit();
+        {
+            const int32_t Eh = (int32_t)(E >> 32);
+            const float Ef = (float)Eh, xf = (float)(int32_t)(dx >> 32), yf = (float)(int32_t)(dy >> 32),
+                        zf = (float)(int32_t)(dz >> 32);
+            ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
+        }
+        if (!ok) {
+            cp_async_wait<0>();
+            tau_acc += adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
+            zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
+            continue;
+        }
+        AdjFxCell t;
+        adj_fx_g(E, dx, dy, dz, dot.result(19), m0, Sx, Sy, Sz, Pxy, Pyz, Pzx, Txy, Tyz, Tzx, Vx, Vy, Vz, eh, em, ph, k, t);
+        // ---- f
+        cp_async_wait<0>();
+        if (bounced) {
+#pragma unroll 1
+            for (int i = 1; i < 19; ++i)
+                if ((bounced >> i) & 1u) col[38 + i][tid] = Ac[RLB_CHK_OFF(opp_rt(i) * S, idx, 38ll * S)];
+        }
+        if (dup) add_dup(0);
+        {
+            int fh = max_exp(38), ef = max_exp(0);
+            ok = fh <= 1900 && ef <= 1900;
+            fh = fh < 100 ? 100 : fh;
+            ef = ef < 100 ? 100 : ef;
+            const int64_t h0 = fx_from(col[38][tid], fh), u0 = fx_from(col[0][tid], ef);
+            int64_t Sf = fx_round4(h0);
+            FxDot fd{};
+            fd.add(fx_split(h0), fx_split(u0));
+            const int64_t u4 = fx_round4(u0);
+            int64_t Fs = (u4 << 3) + (u4 << 2);  // 36 w0 mu_f0
+            int64_t Fx = 0, Fy = 0, Fz = 0;
+#pragma unroll 1
+            for (int r = 0; r < 3; ++r) {
+                const Round v(r);
+                int64_t sg, dl;
+                auto pair = [&](int i, int j) {
+                    const int64_t a = fx_from(col[38 + i][tid], fh), b = fx_from(col[38 + j][tid], fh);
+                    const int64_t ua = fx_from(col[i][tid], ef), ub = fx_from(col[j][tid], ef);
+                    Sf += fx_round4(a + b);
+                    fd.add(fx_split(a), fx_split(ua));
+                    fd.add(fx_split(b), fx_split(ub));
+                    sg = fx_round4(ua + ub);
+                    dl = fx_round4(ua - ub);
+                };
+                pair(v.ax, v.ax + 1);
+                Fs += sg << 1;
+                Fx += dl << 1;
+                pair(v.pp, v.pp + 1);
+                Fs += sg;
+                Fx += dl, Fy += dl;
+                pair(v.pm, v.mp);
+                Fs += sg;
+                Fx += dl, Fy -= dl;
+                rotate3(Fx, Fy, Fz);
+            }
+            adj_fx_f(Sf, fd.result(19), Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
+        }
+        if (!ok) {
+            tau_acc += adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
+            zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
+            continue;
+        }
+        tau_acc = fma(t.tsum, c.inv_tau2, tau_acc);
+        // ---- nu = (1 - omega) mu + omega (...), scattered.  omega (v_E +
+        // e_i.v_d) as integers of one exponent; values beyond its range
+        // (ek >= 1900) are non-finite or about to overflow
+        const double nuE = t.nuE, nuS = t.nuS, kv[4] = {t.nuE, t.tx, t.ty, t.tz};
+        int ek = fx_max_exponent<4>(kv);
+        if (ek >= 1900) {
+            adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
+            zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
+            continue;
+        }
+        ek = ek < 100 ? 100 : ek;
+        const int64_t kE = fx_from(nuE, ek);
+        int64_t ka = fx_from(t.tx, ek), kb = fx_from(t.ty, ek), kc = fx_from(t.tz, ek);
+        double* Lo = Lout + idx;
+        Lo[RLB_CHK_OFF(0, idx, 38ll * S)] = fma(ph.fx.omw, col[0][tid], nuS);
+        Lo[RLB_CHK_OFF(19 * S, idx, 38ll * S)] = fma(ph.fx.omw, col[19][tid], nuE);
+#pragma unroll 1
+        for (int r = 0; r < 3; ++r) {
+            const Round v(r);
+            auto put = [&](int i, int off, int64_t kt) {
+                const bool back = (bounced >> i) & 1u;
+                const long long at = (long long)(back ? opp_rt(i) : i) * S + (back ? 0 : off);
+                Lo[RLB_CHK_OFF(at, idx, 38ll * S)] = fma(ph.fx.omw, col[i][tid], nuS);
+                Lo[RLB_CHK_OFF(19 * S + at, idx, 38ll * S)] = fma(ph.fx.omw, col[19 + i][tid], fx_to(kt, ek - 1083));
+            };
+            put(v.ax, am, kE + ka);
+            put(v.ax + 1, ap, kE - ka);
+            put(v.pp, am + bm, kE + ka + kb);
+            put(v.pp + 1, ap + bp, kE - ka - kb);
+            put(v.pm, am + bp, kE + ka - kb);
+            put(v.mp, ap + bm, kE - ka + kb);
+            rotate3(ka, kb, kc);
+            rotate3(am, bm, cm);
+            rotate3(ap, bp, cp);
+        }
+        zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
+    }
+    warp_partials<double>(tau_acc, bin0, bin1, bin2, has_b, red);
+}
+
+// Eight lanes per cell (lattices of at most 32 cells per SM, two warps per
+// scheduler, where a step takes the time of one warp's instructions: 1600
+// cells 29 -> 21 us, 4800 cells 29 -> 23 us): lane j holds pair j, lane 0 also pair 8,
+// lane 1 the rest populations; the sums are gathered by shuffles and the
+// binary64 part is repeated on every lane.
+template <int XBC>
+__global__ void __launch_bounds__(128)
+    k_adjoint_step_fx_split(const double* __restrict__ A, const double* __restrict__ Lin, double* __restrict__ Lout,
+                            const __grid_constant__ Geom g, const __grid_constant__ Phys ph,
+                            const __grid_constant__ AdjConst<double> c, const __grid_constant__ AdjFx k, double* red,
+                            const double* __restrict__ inflow_t) {
+    const unsigned full = 0xffffffffu;
+    const long long S = g.S;
+    const long long t8 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = threadIdx.x & 7, base = threadIdx.x & 24;  // lane of the group, its first lane in the warp
+    const bool live = (t8 >> 3) < g.N;
+    const int idx = live ? (int)(t8 >> 3) : 0;
+    int x, y, z;
+    cell_coords(g, idx, x, y, z);
+    const bool ghost = XBC != XBC_PERIODIC && (x == 0 || x == g.nx - 1);
+    const PullOffsets o(g, x, y, z);
+    const int dup = dup_of<XBC>(x, g.nx);
+    // this lane's velocities: 2j + 1, 2j + 2 and (lane 0) 17, 18 or (lane 1) 0
+    const int iv[4] = {2 * j + 1, 2 * j + 2, j == 0 ? 17 : 0, 18};
+    const int nv = j == 0 ? 4 : (j == 1 ? 3 : 2);
+    double hf[4], hg[4], uf[4], ug[4];
+    unsigned back = 0u;
+    double tau_acc = 0.0, bin0 = 0.0, bin1 = 0.0, bin2 = 0.0;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        hf[n] = hg[n] = uf[n] = ug[n] = 0.0;
+        if (live && n < nv) {
+            uf[n] = __ldg(Lin + RLB_CHK(iv[n] * S + idx, 38ll * S));
+            ug[n] = __ldg(Lin + RLB_CHK((19 + iv[n]) * S + idx, 38ll * S));
+            if (!ghost) {
+                const int src = idx + o.src(iv[n]);
+                hf[n] = __ldg(A + RLB_CHK(iv[n] * S + src, 38ll * S));
+                hg[n] = __ldg(A + RLB_CHK((19 + iv[n]) * S + src, 38ll * S));
+                if (dup) {
+                    uf[n] += __ldg(Lin + RLB_CHK(iv[n] * S + idx + dup, 38ll * S));
+                    ug[n] += __ldg(Lin + RLB_CHK((19 + iv[n]) * S + idx + dup, 38ll * S));
+                }
+            }
+        }
+    }
+    const bool own_solid = j == 1 && is_solid(ghost ? __ldg(A + RLB_CHK(idx, 38ll * S)) : hf[2]);
+    const bool solid = __shfl_sync(full, own_solid, base + 1);
+    const bool work = live && !ghost && !solid;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        if (work && n < nv && iv[n] > 0 && is_solid(hf[n])) {  // link bounce-back
+            back |= 1u << n;
+            hf[n] = __ldg(A + RLB_CHK(opp_rt(iv[n]) * S + idx, 38ll * S));
+            hg[n] = __ldg(A + RLB_CHK((19 + opp_rt(iv[n])) * S + idx, 38ll * S));
+        }
+    }
+    int eh = fx_max_exponent<4>(hg), em = fx_max_exponent<4>(ug), fh = fx_max_exponent<4>(hf), ef = fx_max_exponent<4>(uf);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+        eh = max(eh, __shfl_xor_sync(full, eh, off));
+        em = max(em, __shfl_xor_sync(full, em, off));
+        fh = max(fh, __shfl_xor_sync(full, fh, off));
+        ef = max(ef, __shfl_xor_sync(full, ef, off));
+    }
+    bool ok = eh >= 100 && eh <= 1900 && em <= 1900 && fh <= 1900 && ef <= 1900;
+    eh = max(eh, 100), em = max(em, 100), fh = max(fh, 100), ef = max(ef, 100);
+    long long hx[4], ux[4];
+    // g
+#pragma unroll
+    for (int n = 0; n < 4; ++n) hx[n] = fx_from(hg[n], eh), ux[n] = fx_from(ug[n], em);
+    auto dot4 = [&]() {
+        FxDot d{};
+#pragma unroll
+        for (int n = 0; n < 4; ++n) d.add(fx_split(hx[n]), fx_split(ux[n]));
+        return d.result(j == 0 ? 4 : (j == 1 ? 3 : 2));
+    };
+    long long E = fx_round4(hx[0] + hx[1]) + fx_round4(hx[2] + hx[3]), dot = dot4();
+    const long long d_j = fx_round4(hx[0] - hx[1]), d_8 = fx_round4(hx[2] - hx[3]);
+    const long long s_j = fx_round4(ux[0] + ux[1]), s_8 = fx_round4(ux[2] + ux[3]);  // lane 1's s_8: the rest population
+    const long long l_j = fx_round4(ux[0] - ux[1]), l_8 = fx_round4(ux[2] - ux[3]);
+    // f
+#pragma unroll
+    for (int n = 0; n < 4; ++n) hx[n] = fx_from(hf[n], fh), ux[n] = fx_from(uf[n], ef);
+    long long Sf = fx_round4(hx[0] + hx[1]) + fx_round4(hx[2] + hx[3]), fd = dot4();
+    const long long sf_j = fx_round4(ux[0] + ux[1]), sf_8 = fx_round4(ux[2] + ux[3]);
+    const long long lf_j = fx_round4(ux[0] - ux[1]), lf_8 = fx_round4(ux[2] - ux[3]);
+    long long Fs = (j < 3 ? sf_j << 1 : sf_j) + (j == 0 ? sf_8 : (j == 1 ? (sf_8 << 3) + (sf_8 << 2) : 0));
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+        E += __shfl_xor_sync(full, E, off);
+        dot += __shfl_xor_sync(full, dot, off);
+        Sf += __shfl_xor_sync(full, Sf, off);
+        fd += __shfl_xor_sync(full, fd, off);
+        Fs += __shfl_xor_sync(full, Fs, off);
+    }
+    auto all9 = [&](long long vj, long long v8, long long* v) {  // the nine pairs' values
+#pragma unroll
+        for (int p = 0; p < 8; ++p) v[p] = __shfl_sync(full, vj, base + p);
+        v[8] = __shfl_sync(full, v8, base);
+    };
+    auto vec9 = [](const long long* v, int sh, int64_t& a, int64_t& b, int64_t& d) {  // sum v_p e_p, axis pairs << sh
+        a = (v[0] << sh) + ((v[3] + v[4]) + (v[5] + v[6]));
+        b = (v[1] << sh) + ((v[3] - v[4]) + (v[7] + v[8]));
+        d = (v[2] << sh) + ((v[5] - v[6]) + (v[7] - v[8]));
+    };
+    long long v[9];
+    int64_t dx, dy, dz, Vx, Vy, Vz, Fx, Fy, Fz;
+    all9(d_j, d_8, v);
+    vec9(v, 0, dx, dy, dz);
+    all9(l_j, l_8, v);
+    vec9(v, 1, Vx, Vy, Vz);
+    all9(lf_j, lf_8, v);
+    vec9(v, 1, Fx, Fy, Fz);
+    all9(s_j, s_8, v);
+    const long long m0 = __shfl_sync(full, s_8, base + 1);
+    const int32_t Eh = (int32_t)(E >> 32);
+    const float Ef = (float)Eh, xf = (float)(int32_t)(dx >> 32), yf = (float)(int32_t)(dy >> 32), zf = (float)(int32_t)(dz >> 32);
+    ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
+    AdjFxCell t;
+    int ek = 0;
+    if (ok) {
+        adj_fx_g(E, dx, dy, dz, dot, m0, v[0] << 1, v[1] << 1, v[2] << 1, v[3] + v[4], v[7] + v[8], v[5] + v[6], v[3] - v[4],
+                 v[7] - v[8], v[5] - v[6], Vx, Vy, Vz, eh, em, ph, k, t);
+        adj_fx_f(Sf, fd, Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
+        const double kv[4] = {t.nuE, t.tx, t.ty, t.tz};
+        ek = fx_max_exponent<4>(kv);
+        ok = ek < 1900;
+        ek = max(ek, 100);
+    }
+    if (work && ok) {
+        const int64_t kE = fx_from(t.nuE, ek), kx = fx_from(t.tx, ek), ky = fx_from(t.ty, ek), kz = fx_from(t.tz, ek);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            if (n < nv) {
+                const int i = iv[n];
+                const int ex = vel_x(i), ey = vel_y(i), ez = vel_z(i);
+                const int64_t kt = kE + (ex > 0 ? kx : (ex < 0 ? -kx : 0)) + (ey > 0 ? ky : (ey < 0 ? -ky : 0)) +
+                                   (ez > 0 ? kz : (ez < 0 ? -kz : 0));
+                const bool bk = (back >> n) & 1u;
+                const long long at = (long long)(bk ? opp_rt(i) : i) * S + idx + (bk ? 0 : o.src(i));
+                Lout[RLB_CHK(at, 38ll * S)] = fma(ph.fx.omw, uf[n], t.nuS);
+                Lout[RLB_CHK(19 * S + at, 38ll * S)] = fma(ph.fx.omw, ug[n], i == 0 ? t.nuE : fx_to(kt, ek - 1083));
+            }
+        }
+        if (j == 0) tau_acc = t.tsum * c.inv_tau2;
+    } else if (work) {
+        if (j == 0) tau_acc = adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
+    }
+    if (live && !work) {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            if (n < nv) {
+                const int i = iv[n];
+                if (ghost) {  // zero where nobody reads the population; the inflow's dL/dbeta_in
+                    if (vel_x(i) != (x == 0 ? 1 : -1)) {
+                        Lout[RLB_CHK(i * S + idx, 38ll * S)] = 0.0;
+                        Lout[RLB_CHK((19 + i) * S + idx, 38ll * S)] = 0.0;
+                    }
+                    if (XBC == XBC_INFLOW_OUTFLOW && x == 0 && !solid) {
+                        const double* tf = inflow_t + 3 * i;
+                        const double* tg = tf + 57;
+                        bin0 = fma(uf[n], tf[0], fma(ug[n], tg[0], bin0));
+                        bin1 = fma(uf[n], tf[1], fma(ug[n], tg[1], bin1));
+                        bin2 = fma(uf[n], tf[2], fma(ug[n], tg[2], bin2));
+                    }
+                } else {  // solid: identity
+                    Lout[RLB_CHK(i * S + idx, 38ll * S)] = uf[n];
+                    Lout[RLB_CHK((19 + i) * S + idx, 38ll * S)] = ug[n];
+                }
+            }
+        }
+    }
+    if (XBC != XBC_PERIODIC && work && (x == 1 || x == g.nx - 2)) {  // populations that a ghost would pull
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const int ex = vel_x(iv[n]);
+            if (n < nv && ((x == 1 && ex == -1) || (x == g.nx - 2 && ex == 1))) {
+                Lout[RLB_CHK(iv[n] * S + idx, 38ll * S)] = 0.0;
+                Lout[RLB_CHK((19 + iv[n]) * S + idx, 38ll * S)] = 0.0;
+            }
+        }
+    }
+    warp_partials<double>(tau_acc, bin0, bin1, bin2, XBC == XBC_INFLOW_OUTFLOW, red);
+}
+
+// ---------------------------------------------------------------------------
 // Shared-memory staged FP32 kernel.  Persistent grid-stride loop; every
 // thread stages the 38 values of each phase of its cells (19 pulled
 // populations + 19 lambda_{t+1}) in its own column of a three-slot ring with
@@ -840,18 +1491,6 @@ __global__ void __launch_bounds__(128, MINB)
 constexpr int kStageThreads = 128;
 constexpr int kStageSlots = 3;
 constexpr size_t kStageSmemBytes = sizeof(float) * kStageSlots * 38 * kStageThreads;
-
-__device__ __forceinline__ void cp_async4(uint32_t saddr, const void* gptr) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(gptr) : "memory");
-}
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gptr) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 // Base address of each of the 38 planes of the three buffers, a kernel
 // parameter: with every plane number a compile-time constant after
@@ -1425,13 +2064,52 @@ cudaError_t smem_opt_in(const void* kern, int bytes) {
 }
 }  // namespace
 
+// Launch of the fixed-point FP64 adjoint: eight lanes per cell while the
+// lanes fit two warps per scheduler, else persistent blocks of 64 threads.
+// warps(): how many write partial sums (4 each).
+struct AdjFxShape {
+    bool split;
+    int grid, threads;
+    int warps() const { return grid * (threads / 32); }
+};
+static AdjFxShape adj_fx_shape(long long N, int nsm) {
+    if (N <= kAdjSplitCells && N <= 32ll * nsm) return {true, (int)((8 * N + 127) / 128), 128};
+    const long long nb = (N + kAdjFxThreads - 1) / kAdjFxThreads, most = (long long)nsm * kAdjFxBlocks;
+    return {false, (int)(nb < most ? nb : most), kAdjFxThreads};
+}
+
+static void launch_adjoint_fx(const Geom& g, const Phys& ph, const AdjConst<double>& c, const double* A,
+                              const double* Li, double* Lo, double* red, const AdjFxShape& sh, const double* inflow_t,
+                              cudaStream_t st) {
+    AdjFx k;
+    double qh, ql;
+    fx_div2(5.0, 3.0, qh, ql);
+    k.kS1 = fx_const(qh, ql, 62);
+    fx_div2(1.0, 36.0, qh, ql);
+    k.kS36 = fx_const(qh, ql, 65);
+    k.kE1 = ph.fx.kE1;
+    k.kE0 = ph.fx.kE0;
+    auto go = [&](auto kern) { kern<<<sh.grid, sh.threads, 0, st>>>(A, Li, Lo, g, ph, c, k, red, inflow_t); };
+    switch (g.xbc) {
+        case XBC_PERIODIC:
+            sh.split ? go(k_adjoint_step_fx_split<XBC_PERIODIC>) : go(k_adjoint_step_fx<XBC_PERIODIC>);
+            break;
+        case XBC_INFLOW_OUTFLOW:
+            sh.split ? go(k_adjoint_step_fx_split<XBC_INFLOW_OUTFLOW>) : go(k_adjoint_step_fx<XBC_INFLOW_OUTFLOW>);
+            break;
+        default:
+            sh.split ? go(k_adjoint_step_fx_split<XBC_OUTFLOW_BOTH>) : go(k_adjoint_step_fx<XBC_OUTFLOW_BOTH>);
+            break;
+    }
+}
+
 template <typename T>
 static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li, T* Lo, double* red, int nb,
                           const double* inflow_d, cudaStream_t st) {
     const AdjConst<T> c = make_adj_const<T>(ph);
     const T* inflow_t = inflow_table<T>(inflow_d);
+    static int nsm = 0;
     auto persistent_grid = [&](int minb) {
-        static int nsm = 0;
         if (nsm == 0) {
             int dev = 0;
             cudaGetDevice(&dev);
@@ -1479,6 +2157,12 @@ static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li
     }
     if constexpr (sizeof(T) == 8) {
         // persistent (the instantiation the allocation-free step runs too)
+        if (ph.fx_on) {
+            persistent_grid(1);  // the SM count
+            const AdjFxShape sh = adj_fx_shape(g.N, nsm);
+            launch_adjoint_fx(g, ph, c, A, Li, Lo, red, sh, inflow_t, st);
+            return sh.warps();
+        }
         switch (g.xbc) {
             case XBC_PERIODIC: warps = go(k_adjoint_step<T, XBC_PERIODIC, 2, true>, true, 2); break;
             case XBC_INFLOW_OUTFLOW: warps = go(k_adjoint_step<T, XBC_INFLOW_OUTFLOW, 2, true>, true, 2); break;
@@ -1578,6 +2262,12 @@ cudaError_t scratch_for_device(int dev, double** ptr, int* nsm) {
             (const void*)k_adjoint_step<float, XBC_PERIODIC, 4, true>,
             (const void*)k_adjoint_step<float, XBC_INFLOW_OUTFLOW, 4, true>,
             (const void*)k_adjoint_step<float, XBC_OUTFLOW_BOTH, 4, true>,
+            (const void*)k_adjoint_step_fx<XBC_PERIODIC>,
+            (const void*)k_adjoint_step_fx<XBC_INFLOW_OUTFLOW>,
+            (const void*)k_adjoint_step_fx<XBC_OUTFLOW_BOTH>,
+            (const void*)k_adjoint_step_fx_split<XBC_PERIODIC>,
+            (const void*)k_adjoint_step_fx_split<XBC_INFLOW_OUTFLOW>,
+            (const void*)k_adjoint_step_fx_split<XBC_OUTFLOW_BOTH>,
             (const void*)k_finalize,
         };
         for (const void* k : kernels) {
@@ -1641,6 +2331,17 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
     e = scratch_for_device(dev, &red, &nsm);
     if (e != cudaSuccess) return e;
     const int nb = adj_blocks(g.N);
+    if (prec == 0 && ph.fx_on) {
+        const AdjFxShape sh = adj_fx_shape(g.N, nsm);
+        const long long need = 4ll * sh.warps();
+        if (need_doubles) *need_doubles = need;
+        if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
+        set_last_launch_count(2);
+        launch_adjoint_fx(g, ph, make_adj_const<double>(ph), (const double*)A, (const double*)lam_in, (double*)lam_out,
+                          red, sh, inflow_table<double>(inflow_d), st);
+        k_finalize<<<1, 1024, 0, st>>>(red, sh.warps(), dtau, dbeta_in);
+        return cudaGetLastError();
+    }
     if (prec != 0 && g.adj_pipe == 2) {
         // FP32 with the default kernel choice: the staged kernel that
         // rlb_adjoint_step runs (persistent, SMs x 3 blocks of 128)

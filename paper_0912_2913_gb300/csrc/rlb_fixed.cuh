@@ -36,17 +36,19 @@
 #include <string.h>
 
 #ifndef __CUDACC__
-#define RLB_FX static inline
+#define RLB_FX inline
 #else
 #define RLB_FX __host__ __device__ __forceinline__
 #endif
 
 namespace rlb {
 
-// A constant in [-2^63, 2^63) as the two 32-bit halves that the products use:
-// value = h 2^32 + 2 l.
+// A constant in [-2^63, 2^63) as the two 32-bit halves that the products use,
+// value = h 2^32 + 2 l, and the rounding term of fx_mul: one half plus the
+// mean of the low product it drops.
 struct FxConst {
     int32_t h, l;
+    uint32_t r;
 };
 
 // Per-run constants (made on the host, make_fx_run).
@@ -57,6 +59,8 @@ struct FxRun {
     FxConst k0;   // omega (1 - 2 / (3 c_l^2))     x 2^62
     FxConst kQ;   // 5 / 9                         x 2^63
     FxConst kG;   // 1 / 6                         x 2^63
+    FxConst kE1;  // 1 / (36 c_l^2)                x 2^65 (adjoint)
+    FxConst kE0;  // (3 - 2 / c_l^2) / 3           x 2^62 (adjoint)
     double om4;   // omega / 4
     double omw;   // 1 - omega
     double m3cl2; // -3 c_l^2
@@ -185,12 +189,26 @@ struct FxSplit {
 RLB_FX FxSplit fx_split(int64_t a) {
     return {(int32_t)(a >> 32), (int32_t)((uint32_t)a >> 1)};
 }
-// (a b) 2^-64 up to two units
-template <class A, class B>
-RLB_FX int64_t fx_mul(const A& a, const B& b) {
-    const int64_t mid = (int64_t)a.h * b.l + (int64_t)a.l * b.h;
+// (a b) 2^-64 within one unit, without bias: the product of the low halves is
+// replaced by its mean (2^29 in the units of mid for two arbitrary factors).
+RLB_FX int64_t fx_mul(const FxSplit& a, const FxConst& b) {
+    const int64_t mid = (int64_t)a.h * b.l + ((int64_t)a.l * b.h + (int64_t)(uint64_t)b.r);
     return (int64_t)a.h * b.h + (mid >> 31);
 }
+RLB_FX int64_t fx_mul(const FxSplit& a, const FxSplit& b) {
+    const int64_t mid = (int64_t)a.h * b.l + ((int64_t)a.l * b.h + 0x60000000ll);
+    return (int64_t)a.h * b.h + (mid >> 31);
+}
+// sum of up to 19 products (a b) 2^-64 of values below 2^61, rounded once
+struct FxDot {
+    int64_t hh, mid;
+    RLB_FX void add(const FxSplit& a, const FxSplit& b) {
+        hh += (int64_t)a.h * b.h;
+        mid += ((int64_t)a.h * b.l + (int64_t)a.l * b.h) >> 6;
+    }
+    // n: how many of the products have low halves (their mean is added)
+    RLB_FX int64_t result(int n) const { return hh + ((mid + ((int64_t)n << 23) + (1 << 24)) >> 25); }
+};
 
 // What a cell's equilibria are made of, in units of 2^-62 of the normalised
 // scale (g0: 2^-59), the antisymmetric f terms for S.

@@ -6,8 +6,11 @@ inline void fx_div2(double a, double b, double& hi, double& lo) {
     hi = a / b;
     lo = fma(-hi, b, a) / b;
 }
+inline FxConst fx_const(int64_t v) {
+    const int32_t l = (int32_t)((uint32_t)v >> 1);
+    return {(int32_t)(v >> 32), l, (1u << 30) + ((uint32_t)l >> 1)};
+}
 // (hi + lo) 2^s as a constant for fx_mul; |value| < 2^63
 inline FxConst fx_const(double hi, double lo, int s) {
-    const int64_t v = (int64_t)ldexp(hi, s) + (int64_t)llrint(ldexp(lo, s));
-    return {(int32_t)(v >> 32), (int32_t)((uint32_t)v >> 1)};
+    return fx_const((int64_t)ldexp(hi, s) + (int64_t)llrint(ldexp(lo, s)));
 }

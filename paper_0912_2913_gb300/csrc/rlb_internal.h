@@ -118,8 +118,10 @@ cudaError_t launch_check_solid_planes(const Geom& g, const uint8_t* solid, unsig
 cudaError_t launch_halo_exchange(int elem, long long nxy, void* lower, long long S_lower, int nz_lower, void* upper,
                                  long long S_upper, cudaStream_t stream);
 
-// Adjoint.  'red' holds 4 doubles of partial sums per 32-cell warp.
-inline long long adj_red_doubles(long long N) { return 4 * 4 * ((N + 127) / 128); }
+// Adjoint.  'red' holds 4 doubles of partial sums per warp: of 32 cells, or
+// of 4 in the eight-lane form of small lattices (at most kAdjSplitCells).
+constexpr long long kAdjSplitCells = 8192;
+inline long long adj_red_doubles(long long N) { return N <= kAdjSplitCells ? N + 64 : 4 * 4 * ((N + 127) / 128); }
 cudaError_t launch_adjoint_macro(int prec, const Geom& g, const Phys& ph, const void* A, const double* dn,
                                  const double* deps, const double* dbeta, void* lam, cudaStream_t stream);
 cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const void* A, const void* lam_in,

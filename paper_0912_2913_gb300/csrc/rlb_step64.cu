@@ -737,7 +737,13 @@ FxRun make_fx_run(double omega, double c_l) {
     // omega (1 - 2 / (3 c_l^2)) = omega - 24 omega / (36 c_l^2)
     const int64_t kE65 = (int64_t)ldexp(th, 65) + (int64_t)llrint(ldexp(tl, 65));
     const int64_t v = (int64_t)ldexp(omega, 62) - 3 * kE65;
-    k.k0 = {(int32_t)(v >> 32), (int32_t)((uint32_t)v >> 1)};
+    k.k0 = fx_const(v);
+    fx_div2(1.0, 36.0, qh, ql);
+    th = qh / c2h;
+    tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
+    k.kE1 = fx_const(th, tl, 65);
+    // (3 - 2 / c_l^2) / 3 = 1 - 24 / (36 c_l^2)
+    k.kE0 = fx_const(1.0 - 24.0 * th, fma(-24.0, th, 1.0) - (1.0 - 24.0 * th) - 24.0 * tl, 62);
     fx_div2(5.0, 9.0, qh, ql);
     k.kQ = fx_const(qh, ql, 63);
     fx_div2(1.0, 6.0, qh, ql);

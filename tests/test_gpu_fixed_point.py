@@ -84,3 +84,43 @@ def test_one_step_of_hard_states(c_l, tau, monkeypatch):
         big = np.abs(h[..., s_, :]).max(-1)[physical]
         err = np.abs(got[..., s_, :] - ref[..., s_, :])[physical].max(-1)
         assert np.all(err <= UNITS * 2.0 ** -53 * big), (s_, (err / big).max() * 2.0 ** 53)
+
+
+@pytest.mark.parametrize("size", [(5, 4, 3), (23, 15, 15)], ids=["eight_lanes", "staged"])
+@pytest.mark.parametrize("xbc", [0, 1, 2])
+@pytest.mark.parametrize("c_l,lam_scale", [(1.0, 1.0), (2.0, 1e-200), (2.0 + 2 ** -30, 1.0)])
+def test_adjoint_step(size, xbc, c_l, lam_scale):
+    """One FP64 adjoint step on lattices of either kernel (at most 32 cells per
+    SM: eight lanes per cell), solid cells and every boundary, lambda zero in
+    part of the lattice: lambda_t, dL/dtau and
+    dL/dbeta_in against the oracle's taped adjoint.  Bound: 1e-11 of the
+    largest |lambda| (the sums of a cell, 57 terms, and gamma^2 <= 2 stay
+    below 10^3 units of 2^-53)."""
+    from paper_0912_2913_gb300 import RLB
+    from tests._helpers import tiny_workload
+
+    nx, ny, nz = size
+    solids = ((2, 1, 1),) if nx < 10 else ((9, 7, 7), (10, 7, 7), (9, 8, 7))
+    w = tiny_workload(nx, ny, nz, xbc, seed=3, c_l=c_l, solid_cells=solids, bmax=0.5)
+    p = oracle.Params(**w.params())
+    st = oracle.init(p, w.n, w.eps, w.beta, w.solid)
+    oracle.run(p, st, 2, solid=w.solid)
+    rng = np.random.default_rng(nx + xbc)
+    lam = rng.normal(size=st.shape) * lam_scale
+    lam[: nz // 2, 0] = 0.0
+    lam_o, dtau_o, dbin_o = oracle.adjoint_step(p, st, lam, w.solid)
+    sim = RLB.from_workload(w, "fp64", device="cuda:0").init_fields(w.n, w.eps, w.beta, w.solid)
+    cells = sim.state_to_cells(sim.state()).cpu().numpy()  # its solid markers
+    fluid = w.solid == 0
+    cells[fluid] = st[fluid]
+    lo = sim.new_state()
+    acc = torch.zeros(4, dtype=torch.float64, device="cuda")
+    sim.adjoint_step(sim.cells_to_state(torch.from_numpy(cells).cuda()), sim.cells_to_state(torch.from_numpy(lam).cuda()), lo,
+                     acc[0:1], acc[1:4])
+    got = sim.state_to_cells(lo).cpu().numpy()
+    acc = acc.cpu().numpy()
+    sim.close()
+    assert np.max(np.abs(got - lam_o)) <= 1e-11 * np.max(np.abs(lam_o))
+    N = nx * ny * nz
+    assert abs(acc[0] - dtau_o) <= 1e-11 * N * np.max(np.abs(lam))
+    assert np.max(np.abs(acc[1:] - dbin_o)) <= 1e-11 * N * np.max(np.abs(lam))
