@@ -250,6 +250,7 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
     ph.omega = 1.0 / p->tau;
     ph.c_l = p->c_l;
     ph.inv_cl = 1.0 / p->c_l;
+    ph.cl2 = p->c_l * p->c_l;
     ph.inv_cl2 = 1.0 / (p->c_l * p->c_l);
     ph.n_in = p->n_in;
     ph.eps_in = p->eps_in;

@@ -68,31 +68,6 @@ __device__ __noinline__ void init_cell_general(T* A, const Geom& g, const Phys& 
     }
 }
 
-// 1/sqrt(a) for 0 < a <= 1, a normal: binary32 seed y, then the third-order
-// step y (1 + e/2 + 3 e^2/8), e = 1 - a y^2.
-__device__ __forceinline__ double rsqrt_unit(double a) {
-    const double y = fx_widen(rsqrtf(fx_seed_f32(a)));
-    const double e = fma(-a * y, y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-// The mantissa of a positive normal v in [2^61, 2^62) and its exponent:
-// v = x 2^(e - 1023 - 61).
-__device__ __forceinline__ int64_t fx_mantissa(double v, int& e) {
-    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-    e = (int)(hi >> 20);
-    return (int64_t)((((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo) << 9);
-}
-// v 2^s / 2^(e - 1023) for |v| below that range (truncated; s <= 62)
-__device__ __forceinline__ int64_t fx_scaled(double v, int e, int s) {
-    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-    const int ev = (int)((hi << 1) >> 21);
-    const uint64_t m = ((uint64_t)((hi << 11) | (lo >> 21) | 0x80000000u) << 32) | (uint64_t)(lo << 11);
-    const uint64_t x = ev == 0 ? 0 : fx_shr(m, (uint32_t)(63 - s + e - ev));
-    const int64_t sg = (int64_t)((int32_t)hi >> 31);
-    return (int64_t)((x ^ (uint64_t)sg) - (uint64_t)sg);
-}
-
 // t 2^eb rounded to binary32 (c1 c2 = 2^(eb + 32)), and whether a value within
 // 128 (d7 - 1) of t could round to another one: t is normalised to 31 leading
 // bits and the bits below the 24th compared with one half.  d7 <= 2^nd.

@@ -160,6 +160,13 @@ RLB_FX int64_t fx_from(double v, int emax) {
     return (int64_t)((x ^ (uint64_t)s) - (uint64_t)s);
 }
 
+// v 2^s for v >= 0 with v 2^s < 2^63 (truncated)
+RLB_FX int64_t fx_fixed(double v, int s) {
+    const uint32_t hi = (uint32_t)fx_hi(v), lo = fx_lo(v);
+    const uint64_t m = ((uint64_t)((hi << 11) | (lo >> 21) | 0x80000000u) << 32) | (uint64_t)(lo << 11);
+    return (int64_t)fx_shr(m, (uint32_t)(1086 - s - (int)(hi >> 20)));
+}
+
 // (x + 8) >> 4: from units of 2^-60 to 2^-56 of the block, rounded to nearest
 RLB_FX int64_t fx_round4(int64_t x) { return (x + 8) >> 4; }
 
@@ -294,10 +301,7 @@ RLB_FX bool fx_g_terms(int64_t E, int64_t dx, int64_t dy, int64_t dz, int emax, 
     double D;
     r_d = fx_reciprocal_D(Ed, u_d[0], u_d[1], u_d[2], k, D);
     const double rW = r_d * k.om4;  // (omega / 4) / D
-    // rW 2^65
-    const uint32_t rh = (uint32_t)fx_hi(rW), rl = fx_lo(rW);
-    const uint64_t rm = ((uint64_t)((rh << 11) | (rl >> 21) | 0x80000000u) << 32) | (uint64_t)(rl << 11);
-    const FxSplit r = fx_split((int64_t)fx_shr(rm, 1021u - (rh >> 20)));
+    const FxSplit r = fx_split(fx_fixed(rW, 65));
     const FxSplit sx = fx_split(dx), sy = fx_split(dy), sz = fx_split(dz);
     // w = d r: (d 2^61)(rW 2^65) 2^-64 = w 2^62, then x 8
     t.wx = fx_split(fx_mul(sx, r) << 3);
@@ -368,5 +372,33 @@ RLB_FX void fx_f_pair(const FxF& t, int p, int64_t& sym, int64_t& asy) {
         default: asy = t.Fy - t.Fz; break;
     }
 }
+
+#ifdef __CUDACC__
+// 1/sqrt(a) for 0 < a <= 1, a normal: binary32 seed y, then the third-order
+// step y (1 + e/2 + 3 e^2/8), e = 1 - a y^2.
+__device__ __forceinline__ double rsqrt_unit(double a) {
+    const double y = fx_widen(rsqrtf(fx_seed_f32(a)));
+    const double e = fma(-a * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// The mantissa of a positive normal v in [2^61, 2^62) and its exponent:
+// v = x 2^(e - 1023 - 61).
+__device__ __forceinline__ int64_t fx_mantissa(double v, int& e) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    e = (int)(hi >> 20);
+    return (int64_t)((((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo) << 9);
+}
+// v 2^s / 2^(e - 1023) for |v| below that range (truncated; s <= 62)
+__device__ __forceinline__ int64_t fx_scaled(double v, int e, int s) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const int ev = (int)((hi << 1) >> 21);
+    const uint64_t m = ((uint64_t)((hi << 11) | (lo >> 21) | 0x80000000u) << 32) | (uint64_t)(lo << 11);
+    const uint64_t x = ev == 0 ? 0 : fx_shr(m, (uint32_t)(63 - s + e - ev));
+    const int64_t sg = (int64_t)((int32_t)hi >> 31);
+    return (int64_t)((x ^ (uint64_t)sg) - (uint64_t)sg);
+}
+
+#endif
 
 }  // namespace rlb

@@ -50,7 +50,7 @@ struct Geom {
 // Physical parameters, with the derived constants the kernels use.
 struct Phys {
     double tau, omega, c_l;
-    double inv_cl, inv_cl2;
+    double inv_cl, inv_cl2, cl2;
     double n_in, eps_in, beta_in[3];
     double n_ref, eps_ref;  // FP32 deviation reference (beta = 0)
     int eos;                // 0: eps = 3P; 1: P = (eos_gamma - 1)(eps - n eos_mass)

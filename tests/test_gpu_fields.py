@@ -99,3 +99,24 @@ def test_fp32_init_keeps_the_binary64_bits(monkeypatch):
             want[..., 0, i] = w * ng * (1.0 + s * fa) - w * n_ref
             want[..., 1, i] = w * (gs + s * ga) - w * e_ref * 1.0
     assert np.array_equal(got.view(np.int32), want.view(np.int32))
+
+
+@pytest.mark.parametrize("c_l", [1.0, 2.0, 2.0 + 2 ** -30])
+@pytest.mark.parametrize("gamma,mass", [(1.2, 0.3), (5 / 3, 0.0), (2.0, 0.9)])
+def test_general_eos_init(gamma, mass, c_l):
+    """Initial equilibria of the general equation of state, pressures from
+    below zero to eps among them.  Bound as above; the relative error of
+    P / ((eps + P) gamma^2) in the equilibria is covered by 4 units more."""
+    from paper_0912_2913_gb300 import RLB
+
+    n, e, b = _fields(int(10 * c_l + 7 * gamma), 1.0)
+    p = oracle.Params(nx=41, ny=5, nz=3, tau=0.8, c_l=c_l, eos=1, eos_gamma=gamma, eos_mass=mass)
+    ref = oracle.init(p, n, e, b)
+    sim = RLB(41, 5, 3, 0.8, c_l=c_l, precision="fp64", eos="gamma_law", eos_gamma=gamma, eos_mass=mass, device="cuda:0")
+    sim.init_fields(n, e, b)
+    got = sim.state_to_cells(sim.state()).cpu().numpy()
+    sim.close()
+    gam2 = 1 / (1 - (b * b).sum(0))
+    # a pressure formed by cancellation: eps - m n against their size
+    size = np.abs(ref).max(-1, keepdims=True) + ((e + mass * n) * gam2)[..., None, None]
+    assert np.all(np.abs(got - ref) <= 20 * U * gam2[..., None, None] * size)

@@ -124,3 +124,40 @@ def test_adjoint_step(size, xbc, c_l, lam_scale):
     N = nx * ny * nz
     assert abs(acc[0] - dtau_o) <= 1e-11 * N * np.max(np.abs(lam))
     assert np.max(np.abs(acc[1:] - dbin_o)) <= 1e-11 * N * np.max(np.abs(lam))
+
+
+@pytest.mark.parametrize("gamma,mass", [(4 / 3, 0.0), (1.2, 0.3), (5 / 3, 0.1), (2.0, 0.0), (1.01, 0.5)])
+@pytest.mark.parametrize("c_l", [1.0, 2.0, 2.0 + 2 ** -30])
+def test_general_eos_one_step(gamma, mass, c_l):
+    """One step and the macroscopic output under the general equation of state
+    at the edges of the fixed-point form: the hard states above (unphysical
+    ones and |M| near E on the binary64 path).  Bound: the oracle stops its
+    iteration at |dP| <= 1e-14 (P + E); 2048 units of 2^-53 of a cell's largest
+    population cover that, its roundings and gamma^2 <= 34."""
+    from paper_0912_2913_gb300 import RLB
+
+    nz, ny, nx = shape = (4, 7, 37)
+    h = _gathered(np.random.default_rng(int(8 * c_l + 100 * gamma)), shape, c_l)
+    a = _scatter(h)
+    p = oracle.Params(nx=nx, ny=ny, nz=nz, tau=0.8, c_l=c_l, eos=1, eos_gamma=gamma, eos_mass=mass)
+    ref = oracle.step(p, a)
+    sim = RLB(nx, ny, nz, 0.8, c_l=c_l, precision="fp64", eos="gamma_law", eos_gamma=gamma, eos_mass=mass, device="cuda:0")
+    sim.load_state(sim.cells_to_state(torch.from_numpy(a).cuda()))
+    n0, e0, b0, _ = sim.macro(state=sim.cells_to_state(torch.from_numpy(h).cuda()), where="host")
+    sim.step(1)
+    got = sim.state_to_cells(sim.state()).cpu().numpy()
+    sim.close()
+    rn, re, rb, _ = oracle.macro(p, h)
+    E, M, S = h[..., 1, :].sum(-1), c_l * (h[..., 1, :] @ EV.astype(float)), h[..., 0, :].sum(-1)
+    # clearly physical: |M| < 0.98 E, a mass share below 0.3 of the rest-frame energy
+    ok = (E > 0) & ((M * M).sum(-1) < 0.96 * E * E) & (S > 0) & (mass * S < 0.3 * np.sqrt(np.maximum(E * E - (M * M).sum(-1), 0)))
+    ok &= np.isfinite(ref).all((-1, -2))
+    assert ok.mean() > 0.05
+    for s_ in range(2):
+        big = np.abs(h[..., s_, :]).max(-1)[ok]
+        err = np.abs(got[..., s_, :] - ref[..., s_, :])[ok].max(-1)
+        assert np.all(err <= 2 * UNITS * 2.0 ** -53 * big), (s_, (err / big).max() * 2.0 ** 53)
+    tol = 2 * UNITS * 2.0 ** -53
+    assert np.all(np.abs(n0 - rn)[ok] <= tol * np.abs(h[..., 0, :]).sum(-1)[ok])
+    assert np.all(np.abs(e0 - re)[ok] <= tol * np.abs(h[..., 1, :]).sum(-1)[ok])
+    assert np.all(np.abs(b0 - rb)[:, ok] <= tol * (c_l * np.abs(h[..., 1, :]).sum(-1) / E)[ok])
