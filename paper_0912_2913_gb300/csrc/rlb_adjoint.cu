@@ -1914,17 +1914,11 @@ cudaError_t launch_inflow_derivs(const Phys& ph, double* out, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // Adjoint of the macroscopic output: n = S sqrt(1 - b2), eps, beta.
 // ---------------------------------------------------------------------------
+// One cell in binary64 with IEEE roots and divisions, any state.
 template <typename T>
-__global__ void __launch_bounds__(128) k_adjoint_macro(const T* __restrict__ A, const double* __restrict__ dn,
-                                                       const double* __restrict__ deps, const double* __restrict__ dbeta,
-                                                       T* __restrict__ lam, Geom g, Phys ph) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= g.N) return;
+__device__ __noinline__ void adjoint_macro_general(const T* A, const double* dn, const double* deps, const double* dbeta,
+                                                   T* lam, const Geom& g, const Phys& ph, int idx) {
     const long long S = g.S;
-    if (is_solid(A[RLB_CHK(idx, 38ll * S)])) {
-        for (int q = 0; q < 38; ++q) lam[RLB_CHK(q * S + idx, 38ll * S)] = (T)0;
-        return;
-    }
     double h[38];
     for (int q = 0; q < 38; ++q) h[q] = (double)A[RLB_CHK(q * S + idx, 38ll * S)];
     double sf = 0, E = 0, Mx = 0, My = 0, Mz = 0;
@@ -1962,37 +1956,226 @@ __global__ void __launch_bounds__(128) k_adjoint_macro(const T* __restrict__ A, 
     }
 }
 
+// FP64 instructions: 60 instead of some 190, which bound the kernel (sphere
+// lattice, FP32: 1.14 -> 0.29 ms).  The
+// moments are integers (fx_moments); s = sqrt(4 E^2 - 3 M^2), 1/s, 1/D and
+// sqrt(1 - beta^2) = 2 sqrt(eps / D) come from binary32 seeds; the 18 moving g
+// values are integer sums of c_l v and v_E.  Binary32 lambdas keep the bits of
+// the binary64 form: a cell with a value within its rounding error (64 u
+// gamma^2 of the terms' sizes) of a binary32 midpoint is left to it.
+template <typename T>
+__global__ void __launch_bounds__(128, 6) k_adjoint_macro(const T* __restrict__ A, const double* __restrict__ dn,
+                                                       const double* __restrict__ deps, const double* __restrict__ dbeta,
+                                                       T* __restrict__ lam, const __grid_constant__ Geom g,
+                                                       const __grid_constant__ Phys ph) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= g.N) return;
+    const long long S = g.S;
+    T* Lc = lam + idx;
+    auto put = [&](int q, T v) { Lc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v; };
+    const double gn = __ldg(dn + idx), ge = __ldg(deps + idx), gx = __ldg(dbeta + idx), gy = __ldg(dbeta + g.N + idx),
+                 gz = __ldg(dbeta + 2 * (long long)g.N + idx);
+    T h[19], f[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) f[i] = __ldg(RLB_CHK_PTR(A, i * S + idx, 38ll * S));
+    if (is_solid(f[0]) || (gn == 0.0 && ge == 0.0 && gx == 0.0 && gy == 0.0 && gz == 0.0)) {
+#pragma unroll
+        for (int q = 0; q < 38; ++q) put(q, (T)0);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 19; ++i) h[i] = __ldg(RLB_CHK_PTR(A, (19 + i) * S + idx, 38ll * S));
+    FxMoments m;
+    if (fx_moments(h, f, ph.fx.m3cl2, ph.n_ref, ph.eps_ref, m)) {
+        const double E2 = m.E + m.E;
+        double ys, hs;
+        rsqrt_seed(m.disc, ys, hs);
+        double sq = m.disc * ys;
+        sq = fma(fma(-sq, sq, m.disc), hs, sq);
+        sq = fma(fma(-sq, sq, m.disc), hs, sq);
+        const double e1 = fma(-sq, ys, 1.0);
+        const double rs = fma(ys, fma(e1, e1, e1), ys);
+        const double D = E2 + sq;
+        const double x0 = rcp_seed(D);
+        const double e2 = fma(-D, x0, 1.0);
+        const double rD = fma(x0, fma(e2, e2, e2), x0);
+        const double r3 = rD * ph.three_cl;
+        const double bx = m.x * r3, by = m.y * r3, bz = m.z * r3;
+        // 1/sqrt(1 - beta^2) and its inverse from 4 eps / D
+        const double w = 4.0 * (fma(m.t, rD, m.E) * rD);
+        const double gam = rsqrt_unit(w);
+        const double aS = gn * (w * gam), cc = -(gn * m.S) * gam;
+        const double ax = fma(cc, bx, gx), ay = fma(cc, by, gy), az = fma(cc, bz, gz);
+        const double ab = fma(ax, bx, fma(ay, by, az * bz)) * rD;
+        const double dE = fma(E2 + E2, rs, -1.0);
+        const double vE = fma(ge, dE, -ab * (3.0 + dE));
+        const double c3 = (ph.three_cl * rs) * (ab - ge), rD3 = 3.0 * rD;
+        // c_l v: v_a = 3 ab_a / D + 3 M_a (...) / s, M = c_l d
+        const double vx = ph.c_l * fma(c3, m.x, ax * rD3), vy = ph.c_l * fma(c3, m.y, ay * rD3),
+                     vz = ph.c_l * fma(c3, m.z, az * rD3);
+        const double kv[4] = {vE, vx, vy, vz};
+        const int ek = fx_max_exponent<4>(kv);
+        bool ok = ek >= 200 && ek < 1800;
+        if constexpr (sizeof(T) == 4) ok = ok && ek > 1023 - 80 && ek < 1023 + 80;
+        if (ok) {
+            const int64_t kE = fx_from(vE, ek), kx = fx_from(vx, ek), ky = fx_from(vy, ek), kz = fx_from(vz, ek);
+            if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                for (int i = 0; i < 19; ++i) put(i, aS);
+                auto gput = [&](int p, int64_t t) {
+                    put(20 + 2 * p, fx_to(kE + t, ek - 1083));
+                    put(21 + 2 * p, fx_to(kE - t, ek - 1083));
+                };
+                put(19, vE);
+                gput(0, kx), gput(1, ky), gput(2, kz), gput(3, kx + ky), gput(4, kx - ky), gput(5, kx + kz), gput(6, kx - kz);
+                gput(7, ky + kz), gput(8, ky - kz);
+                return;
+            } else {
+                // the rounding error of the binary64 form in units of 2^(ek - 1083):
+                // 64 u gamma^2 at the size of the terms
+                auto mag = [](double v) { return fabsf(d2f_seed(v)); };
+                const float B = 3.0f * mag(ge) + 6.0f * mag(ab) + 3.0f * (float)ph.c_l * mag(rD) * (mag(ax) + mag(ay) + mag(az)) +
+                                3.0f * mag(ph.cl2 * rs) * (mag(m.x) + mag(m.y) + mag(m.z)) * (mag(ab) + mag(ge));
+                const float g1 = d2f_seed(gam), g2 = g1 * g1;
+                const float units = 8192.0f * g2 * B * pow2f(1023 - ek);
+                F32Out o;
+                const int kb = ek - 1083 + 32;
+                o.c1 = pow2f(kb >> 1), o.c2 = pow2f(kb - (kb >> 1));
+                ok = units < 0x1p28f;
+                o.d7 = (uint32_t)(units * (1.03f / 128.0f)) + 2u;
+                o.nd = 32 - __clz((int)o.d7);
+                bool ambiguous = !ok;
+                float fs = 0.0f;
+                if (gn != 0.0) {
+                    int es;
+                    const double as = fabs(aS);
+                    const int64_t xs = fx_mantissa(as, es);
+                    F32Out of;
+                    const int kf = es - 1084 + 32;
+                    ambiguous |= es < 1023 - 80 || es > 1023 + 80;
+                    of.c1 = pow2f(kf >> 1), of.c2 = pow2f(kf - (kf >> 1));
+                    of.d7 = (uint32_t)(256.0f * g2 * 1.03f) + 2u;
+                    of.nd = 32 - __clz((int)of.d7);
+                    fs = copysignf(fx_to_f32(xs, of, ambiguous), gn > 0.0 ? 1.0f : -1.0f);
+                }
+                if (!ambiguous) {
+#pragma unroll
+                    for (int i = 0; i < 19; ++i) put(i, fs);
+                    auto gput = [&](int p, int64_t t) {
+                        put(20 + 2 * p, fx_to_f32(kE + t, o, ambiguous));
+                        put(21 + 2 * p, fx_to_f32(kE - t, o, ambiguous));
+                    };
+                    put(19, fx_to_f32(kE, o, ambiguous));
+                    gput(0, kx), gput(1, ky), gput(2, kz), gput(3, kx + ky), gput(4, kx - ky), gput(5, kx + kz),
+                        gput(6, kx - kz);
+                    gput(7, ky + kz), gput(8, ky - kz);
+                    if (!ambiguous) return;
+                }
+            }
+        }
+    }
+    adjoint_macro_general<T>(A, dn, deps, dbeta, lam, g, ph, idx);
+}
+
 // ---------------------------------------------------------------------------
 // Adjoint of the initialisation A_0 = eq(n0, eps0, beta0).
 // ---------------------------------------------------------------------------
+// The lambda moments are integers (weights times 36): S1, T, V over the g
+// pairs, F1, F over the f pairs; with y = T beta, eg = eps gamma^2 and
+//   Q = [6 beta.y - 2 |beta|^2 S1] / c_l^2 + 4 V.beta / c_l + w0 l_0 (4 - 2 |beta|^2 / c_l^2):
+//   a_eps  = S1 / c_l^2 - w0 l_0 (2 / c_l^2 + 1) + gamma^2 Q
+//   a_beta = eg [(12 y - 4 (S1 + w0 l_0) beta) / c_l^2 + 4 V / c_l + 2 gamma^2 Q beta]
+//   a_S    = w0 l_f0 + F1 + 3 F.beta / c_l,   a_n = gamma a_S,
+//   a_beta += 3 n gamma F / c_l + n gamma^3 a_S beta.
+// 80 FP64 instructions instead of some 250 with the conversions, which bound
+// the kernel (sphere lattice, FP32 lambdas: 1.72 -> 0.41 ms).
 template <typename T>
-__global__ void __launch_bounds__(128) k_adjoint_fields(const double* __restrict__ n0, const double* __restrict__ e0,
+__global__ void __launch_bounds__(128, 4) k_adjoint_fields(const double* __restrict__ n0, const double* __restrict__ e0,
                                                         const double* __restrict__ b0, const T* __restrict__ A0,
                                                         const T* __restrict__ lam, double* __restrict__ dn,
-                                                        double* __restrict__ de, double* __restrict__ db, Geom g,
-                                                        Phys ph, double* red) {
+                                                        double* __restrict__ de, double* __restrict__ db,
+                                                        const __grid_constant__ Geom g, const __grid_constant__ Phys ph,
+                                                        double* red) {
     const long long S = g.S;
     double bin0 = 0.0, bin1 = 0.0, bin2 = 0.0;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.N; idx = g.N) {
-        const int x = idx % g.nx;
-        double lf[19], lg[19];
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx < g.N) {
         double an = 0, ae = 0, ax = 0, ay = 0, az = 0;
-        const bool solid = is_solid(A0[RLB_CHK(idx, 38ll * S)]);
-        if (!solid) {
-            for (int i = 0; i < 19; ++i) {
-                lf[i] = (double)lam[RLB_CHK(i * S + idx, 38ll * S)];
-                lg[i] = (double)lam[RLB_CHK((19 + i) * S + idx, 38ll * S)];
-            }
-            if (g.xbc == XBC_INFLOW_OUTFLOW && x == 0) {
-                eq_fields_adjoint(lf, lg, ph.n_in, ph.eps_in, ph.beta_in[0], ph.beta_in[1], ph.beta_in[2], ph, an,
-                                  ae, ax, ay, az);
-                bin0 += ax;
-                bin1 += ay;
-                bin2 += az;
-                an = ae = ax = ay = az = 0;
+        if (!is_solid(A0[RLB_CHK(idx, 38ll * S)])) {
+            const bool inflow = g.xbc == XBC_INFLOW_OUTFLOW && idx % g.nx == 0;
+            double n, e, bx, by, bz;
+            if (inflow) {
+                n = ph.n_in, e = ph.eps_in, bx = ph.beta_in[0], by = ph.beta_in[1], bz = ph.beta_in[2];
             } else {
-                eq_fields_adjoint(lf, lg, n0[idx], e0[idx], b0[idx], b0[g.N + idx], b0[2 * (long long)g.N + idx], ph,
-                                  an, ae, ax, ay, az);
+                n = __ldg(n0 + idx), e = __ldg(e0 + idx);
+                bx = __ldg(b0 + idx), by = __ldg(b0 + g.N + idx), bz = __ldg(b0 + 2 * (long long)g.N + idx);
+            }
+            T lf[19], lg[19];
+#pragma unroll
+            for (int i = 0; i < 19; ++i) lg[i] = __ldg(RLB_CHK_PTR(lam, (19 + i) * S + idx, 38ll * S));
+#pragma unroll
+            for (int i = 0; i < 19; ++i) lf[i] = __ldg(RLB_CHK_PTR(lam, i * S + idx, 38ll * S));
+            constexpr int BIAS = sizeof(T) == 4 ? 127 : 1023, LO = sizeof(T) == 4 ? 64 : 100, HI = sizeof(T) == 4 ? 250 : 1900;
+            int em = fx_max_exponent<19>(lg), ef = fx_max_exponent<19>(lf);
+            const double b2 = fma(bx, bx, fma(by, by, bz * bz));
+            const double omb2 = 1.0 - b2;
+            const int oh = __double2hiint(omb2);
+            if (em <= HI && ef <= HI && oh > 0x3F900000 && oh < 0x3FF00001) {
+                em = em < LO ? LO : em;
+                ef = ef < LO ? LO : ef;
+                const int km = em - BIAS - 56, kf = ef - BIAS - 56;
+                int64_t Sx = 0, Sy = 0, Sz = 0, Pxy = 0, Pxz = 0, Pyz = 0, Txy = 0, Txz = 0, Tyz = 0, Vx = 0, Vy = 0, Vz = 0;
+                int64_t Fx = 0, Fy = 0, Fz = 0;
+                const int64_t m0 = fx_round4(fx_from(lg[0], em)), u0 = fx_round4(fx_from(lf[0], ef));
+                int64_t Fs = (u0 << 3) + (u0 << 2);
+#pragma unroll
+                for (int p = 0; p < 9; ++p) {
+                    const int64_t a = fx_from(lg[2 * p + 1], em), b = fx_from(lg[2 * p + 2], em);
+                    const int64_t c = fx_from(lf[2 * p + 1], ef), d = fx_from(lf[2 * p + 2], ef);
+                    const int sh = p < 3 ? 1 : 0;
+                    const int64_t sg = fx_round4(a + b) << sh, dl = fx_round4(a - b) << sh, df = fx_round4(c - d) << sh;
+                    Fs += fx_round4(c + d) << sh;
+                    if (p == 0) Sx = sg;
+                    if (p == 1) Sy = sg;
+                    if (p == 2) Sz = sg;
+                    if (p == 3 || p == 4) Pxy += sg, Txy += p == 3 ? sg : -sg;
+                    if (p == 5 || p == 6) Pxz += sg, Txz += p == 5 ? sg : -sg;
+                    if (p == 7 || p == 8) Pyz += sg, Tyz += p == 7 ? sg : -sg;
+                    if (pair_ex(p)) Vx += dl, Fx += df;
+                    if (pair_ey(p) > 0) Vy += dl, Fy += df;
+                    if (pair_ey(p) < 0) Vy -= dl, Fy -= df;
+                    if (pair_ez(p) > 0) Vz += dl, Fz += df;
+                    if (pair_ez(p) < 0) Vz -= dl, Fz -= df;
+                }
+                const double i2 = ph.inv_cl2, i1 = ph.inv_cl;
+                const double gam = rsqrt_unit(omb2);
+                const double gam2 = gam * gam, eg = e * gam2 * (1.0 / 36.0);
+                const double S1 = fx_to((Sx + Sy + Sz) + (Pxy + Pxz + Pyz), km), l0 = 12.0 * fx_to(m0, km);
+                const double Txx = fx_to(Sx + Pxy + Pxz, km), Tyy = fx_to(Sy + Pxy + Pyz, km), Tzz = fx_to(Sz + Pxz + Pyz, km);
+                const double txy = fx_to(Txy, km), txz = fx_to(Txz, km), tyz = fx_to(Tyz, km);
+                const double yx = fma(Txx, bx, fma(txy, by, txz * bz)), yy = fma(txy, bx, fma(Tyy, by, tyz * bz)),
+                             yz = fma(txz, bx, fma(tyz, by, Tzz * bz));
+                const double vx = fx_to(Vx, km), vy = fx_to(Vy, km), vz = fx_to(Vz, km);
+                const double by_ = fma(bx, yx, fma(by, yy, bz * yz)), vb = fma(bx, vx, fma(by, vy, bz * vz));
+                const double b2i = b2 * i2;
+                const double Q = fma(6.0 * i2, by_, fma(4.0 * i1, vb, fma(-2.0 * b2i, S1 + l0, 4.0 * l0)));
+                ae = fma(gam2, Q, fma(i2, S1, -l0 * fma(2.0, i2, 1.0))) * (1.0 / 36.0);
+                const double cb = fma(-4.0 * i2, S1 + l0, 2.0 * gam2 * Q) * eg, cy = 12.0 * i2 * eg, cv = 4.0 * i1 * eg;
+                const double fx = fx_to(Fx, kf), fy = fx_to(Fy, kf), fz = fx_to(Fz, kf);
+                const double fb = fma(bx, fx, fma(by, fy, bz * fz));
+                an = fma(3.0 * i1, fb, fx_to(Fs, kf)) * (gam * (1.0 / 36.0));
+                const double ng = n * gam * (1.0 / 12.0) * i1, cs = fma(an * n, gam2, cb);
+                ax = fma(cy, yx, fma(cv, vx, fma(ng, fx, cs * bx)));
+                ay = fma(cy, yy, fma(cv, vy, fma(ng, fy, cs * by)));
+                az = fma(cy, yz, fma(cv, vz, fma(ng, fz, cs * bz)));
+            } else {
+                double df[19], dg[19];
+                for (int i = 0; i < 19; ++i) df[i] = (double)lf[i], dg[i] = (double)lg[i];
+                eq_fields_adjoint(df, dg, n, e, bx, by, bz, ph, an, ae, ax, ay, az);
+            }
+            if (inflow) {
+                bin0 = ax, bin1 = ay, bin2 = az;
+                an = ae = ax = ay = az = 0;
             }
         }
         dn[idx] = an;

@@ -399,6 +399,111 @@ __device__ __forceinline__ int64_t fx_scaled(double v, int e, int s) {
     return (int64_t)((x ^ (uint64_t)sg) - (uint64_t)sg);
 }
 
+// t 2^eb rounded to binary32 (c1 c2 = 2^(eb + 32)), and whether a value within
+// 128 (d7 - 1) of t could round to another one: t is normalised to 31 leading
+// bits and the bits below the 24th compared with one half.  d7 <= 2^nd.
+struct F32Out {
+    float c1, c2;
+    uint32_t d7;
+    int nd;
+};
+__device__ __forceinline__ float fx_to_f32(int64_t t, const F32Out& o, bool& ambiguous) {
+    const int32_t hi = (int32_t)(t >> 32);
+    const int n = __clz(hi ^ (hi >> 31)) - 1;
+    const uint32_t nh = __funnelshift_l((uint32_t)t, (uint32_t)hi, n), nl = (uint32_t)t << n;
+    const uint32_t w = __funnelshift_r(nl, nh, 7);  // the 32 bits below the 24 kept
+    const uint32_t d = o.d7 << n;
+    ambiguous |= (w + 0x80000000u + d) < 2u * d;
+    ambiguous |= n + o.nd > 29;  // (also t = 0 and t below 2^32)
+    // bit 0 set: the bits dropped from nh then never turn into a tie (an exact
+    // tie is ambiguous)
+    return (float)(int32_t)(nh | 1u) * __uint_as_float((uint32_t)(127 - n) << 23) * o.c1 * o.c2;
+}
+__device__ __forceinline__ float pow2f(int k) { return __uint_as_float((uint32_t)(127 + k) << 23); }
+// Binary32 values to fixed point: as fx_from, v 2^60 / 2^(emax - 127).
+__device__ __forceinline__ int64_t fx_from(float v, int emax) {
+    const uint32_t u = __float_as_uint(v);
+    const int e = (int)((u << 1) >> 24);
+    const uint64_t m = (uint64_t)((u << 8) | 0x80000000u) << 32;
+    const uint64_t x = fx_shr(m, (uint32_t)(emax + 3 - e));
+    const int64_t s = (int64_t)((int32_t)u >> 31);
+    return (int64_t)((x ^ (uint64_t)s) - (uint64_t)s);
+}
+template <int N>
+__device__ __forceinline__ int fx_max_exponent(const float* v) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t t = __float_as_uint(v[i]) << 1;
+        m = t > m ? t : m;
+    }
+    return (int)(m >> 24);
+}
+
+// The moments of a stored state's cell: E, S and d = M / c_l in binary64 (d
+// also as integers x 2^(kb - 2)), t = -3 |M|^2 and 4 E^2 - 3 |M|^2.  T = float:
+// deviations from (n_ref, eps_ref).  False unless the cell is clearly
+// physical (E, S > 0, |M|^2 < 0.98 E^2) and its exponents are in range.
+struct FxMoments {
+    double E, S, x, y, z, t, disc;
+    int64_t ix, iy, iz;
+    int kb;
+};
+template <typename T>
+__device__ __forceinline__ bool fx_moments(const T* h, const T* f, double m3cl2, double n_ref, double eps_ref, FxMoments& m) {
+    constexpr bool DEV = sizeof(T) == 4;
+    constexpr int BIAS = DEV ? 127 : 1023, LO = DEV ? 64 : 128, HI = DEV ? 250 : 1900;
+    // the moving populations share an exponent; FP64: the rest population,
+    // 9 c_l^2 times larger, is added in binary64; FP32: it shares it too (its
+    // deviation carries 24 bits)
+    const int em = DEV ? fx_max_exponent<19>(h) : fx_max_exponent<18>(h + 1);
+    const int ef = fx_max_exponent<19>(f);
+    bool ok = ((DEV && em == 0) || em > LO) && em < HI && ((DEV && ef == 0) || ef > LO) && ef < HI;
+    double E = 0, sf = 0, dx = 0, dy = 0, dz = 0;
+    if (!ok) return false;
+    {
+        int64_t ix = 0, iy = 0, iz = 0;
+        int64_t e = DEV ? fx_round4(fx_from(h[0], em)) : 0, d[9];
+        int64_t s = fx_round4(fx_from(f[0], ef));
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            const int64_t a = fx_from(h[2 * p + 1], em), b = fx_from(h[2 * p + 2], em);
+            e += fx_round4(a + b);
+            d[p] = (a - b + 2) >> 2;  // units of 2^-58
+            s += fx_round4(fx_from(f[2 * p + 1], ef) + fx_from(f[2 * p + 2], ef));
+        }
+        const int kb = em - BIAS - 56;
+        if (DEV && em == 0) {  // every deviation zero
+        } else {
+            E = fx_to(e, kb);
+            ix = ((d[0] + d[3]) + (d[4] + d[5])) + d[6];
+            iy = ((d[1] + d[3]) - d[4]) + (d[7] + d[8]);
+            iz = ((d[2] + d[5]) - d[6]) + (d[7] - d[8]);
+            dx = fx_to(ix, kb - 2);
+            dy = fx_to(iy, kb - 2);
+            dz = fx_to(iz, kb - 2);
+        }
+        if (!(DEV && ef == 0)) sf = fx_to(s, ef - BIAS - 56);
+        E += DEV ? eps_ref : (double)h[0];
+        if (DEV) sf += n_ref;
+        const double E2 = E + E;
+        const double t = m3cl2 * fma(dx, dx, fma(dy, dy, dz * dz));  // -3 |M|^2
+        const double disc = fma(E2, E2, t);
+        // E and S positive, exponents in range, |M|^2 < 0.98 E^2
+        const int Eh = __double2hiint(E), Sh = __double2hiint(sf), Dh = __double2hiint(disc);
+        const int k = (Eh >> 20) - 1023;
+        ok = Eh > (600 << 20) && Eh < (1500 << 20) && Sh > (600 << 20) && Sh < (1500 << 20) && Dh > 0;
+        if (ok) {
+            const float Em = fx_seed_f32(fx_double((uint32_t)Eh - ((uint32_t)k << 20), (uint32_t)__double2loint(E)));
+            const float Dm = fx_seed_f32(fx_double((uint32_t)Dh - ((uint32_t)k << 21), (uint32_t)__double2loint(disc)));
+            ok = Dm > 1.06f * Em * Em && Dm < 4.001f * Em * Em;
+        }
+        m.E = E, m.S = sf, m.x = dx, m.y = dy, m.z = dz, m.t = t, m.disc = disc;
+        m.ix = ix, m.iy = iy, m.iz = iz, m.kb = kb;
+    }
+    return ok;
+}
+
 #endif
 
 }  // namespace rlb

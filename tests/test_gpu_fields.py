@@ -120,3 +120,59 @@ def test_general_eos_init(gamma, mass, c_l):
     # a pressure formed by cancellation: eps - m n against their size
     size = np.abs(ref).max(-1, keepdims=True) + ((e + mass * n) * gam2)[..., None, None]
     assert np.all(np.abs(got - ref) <= 20 * U * gam2[..., None, None] * size)
+
+
+@pytest.mark.parametrize("c_l", [1.0, 2.0, 10.0])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_macro_and_field_adjoints(prec, c_l):
+    """Adjoints of the macroscopic output and of the initial equilibria over
+    the fields above, zero output gradients in part of the lattice and lambda
+    of very different sizes.  Bounds: 64 roundings times gamma^2 (the velocity
+    terms of eps and n) of the sum of the terms' sizes; stored binary32 lambdas
+    one rounding more."""
+    from paper_0912_2913_gb300 import RLB
+
+    n, e, b = _fields(int(10 * c_l) + 5, 1.0)
+    shape = n.shape
+    p = oracle.Params(nx=shape[2], ny=shape[1], nz=shape[0], tau=0.8, c_l=c_l)
+    n_ref, e_ref = 0.7, 0.2
+    sim = RLB(shape[2], shape[1], shape[0], 0.8, c_l=c_l, precision=prec, n_ref=n_ref, eps_ref=e_ref, device="cuda:0")
+    sim.init_fields(n, e, b)
+    full = sim.state_to_cells(sim.state()).double().cpu().numpy()
+    if prec == "fp32":
+        full = full + oracle.init(oracle.Params(nx=1, ny=1, nz=1, tau=0.8, c_l=c_l), np.full((1, 1, 1), n_ref),
+                                  np.full((1, 1, 1), e_ref), np.zeros((3, 1, 1, 1)))
+    rng = np.random.default_rng(4)
+    gn, ge = rng.normal(size=(2,) + shape)
+    gb = rng.normal(size=(3,) + shape)
+    gn[0] = 0.0
+    ge[0, 0] = 0.0
+    gb[:, 0] = 0.0
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    lam = sim.new_state()
+    sim.adjoint_macro(sim.state(), t(gn), t(ge), t(gb), lam)
+    got = sim.state_to_cells(lam).double().cpu().numpy()
+    want = oracle.adjoint_macro(p, np.ascontiguousarray(full), gn, ge, gb)
+    E, S = full[..., 1, :].sum(-1), full[..., 0, :].sum(-1)
+    gam2 = 1 / (1 - (b * b).sum(0))
+    size = np.abs(ge) * 9 + (np.abs(gb).sum(0) + np.abs(gn) * np.abs(S) * np.sqrt(gam2)) * (1 + c_l) * 6 / E + np.abs(gn)
+    tol = 64 * U * gam2 * size * (np.abs(full).sum((-1, -2)) / np.minimum(np.abs(E), np.abs(S)))
+    tol = np.broadcast_to(tol[..., None, None], want.shape)
+    if prec == "fp32":
+        tol = tol + 2.0 ** -24 * 1.01 * np.abs(got) + 1e-45
+    m = gam2 < 40
+    assert np.all((np.abs(got - want) <= tol)[m]), np.max((np.abs(got - want) / tol)[m])
+    # the initial fields
+    l0 = rng.normal(size=got.shape) * np.exp(rng.uniform(-20, 20, size=shape))[..., None, None]
+    l0[0, 1] = 0.0
+    ls = sim.cells_to_state(t(l0))
+    l0 = sim.state_to_cells(ls).double().cpu().numpy()
+    outs = [torch.empty(shape, dtype=torch.float64, device="cuda") for _ in range(2)]
+    db, acc = torch.empty((3,) + shape, dtype=torch.float64, device="cuda"), torch.zeros(3, dtype=torch.float64, device="cuda")
+    sim.adjoint_fields(t(n), t(e), t(b), ls, outs[0], outs[1], db, acc)
+    ref = oracle.adjoint_fields(p, n, e, b, np.ascontiguousarray(l0))
+    sim.close()
+    big = np.abs(l0).max((-1, -2)) * gam2
+    assert np.all(np.abs(outs[0].cpu().numpy() - ref[0]) <= 64 * U * gam2 * big)
+    assert np.all(np.abs(outs[1].cpu().numpy() - ref[1]) <= 64 * U * gam2 * big * 8)
+    assert np.all(np.abs(db.cpu().numpy() - ref[2]) <= 64 * U * gam2 ** 2 * big * 16 * (n + e))
