@@ -20,8 +20,9 @@
 // that is a ghost plane), or the identity at solid cells (never updated).
 // dL/dtau = sum mu_i (h_i - eq_i)/tau^2 and, at the inflow plane (held at
 // eq(n_in, eps_in, beta_in)), dL/dbeta_in = sum lambda_{t+1} d eq/d beta_in
-// are summed per warp (binary32 for the FP32 path, binary64 otherwise) and
-// then over the warp partials in a fixed order (k_finalize).
+// are summed per warp (binary32 for the FP32 path, binary64 otherwise), per
+// block, and over the blocks in a fixed order: by the block that ends last
+// (block_sums, FP64) or by a second kernel (k_finalize).
 #include <cuda.h>  // CUcontext type only; cuCtxGetCurrent is taken through the runtime
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -178,38 +179,121 @@ __device__ __forceinline__ void block_reduce4(double v0, double v1, double v2, d
     }
 }
 
-// Sum the partial-sum slots (one per warp or per block, 4 doubles each) and
-// add them to the accumulators.  256 threads per component; thread t sums
-// slots t, t+256, ... in a fixed grouping, then a fixed tree combines the 256
-// sums: the result does not depend on scheduling.
-__global__ void __launch_bounds__(1024) k_finalize(const double* __restrict__ red, int nslots, double* dtau,
-                                                   double* dbeta_in) {
-    __shared__ double sm[4][256];
-    const int k = threadIdx.x >> 8, t = threadIdx.x & 255;
-    // eight independent partial sums so that eight loads are in flight; the
-    // grouping depends only on nslots (deterministic)
-    double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int b = t;
-    for (; b + 7 * 256 < nslots; b += 8 * 256) {
+// Where a persistent adjoint kernel leaves its sums: red[block*4 + k], then,
+// by the last block to arrive at the ticket (which it resets to 0), the sum
+// over the blocks added to the accumulators.
+struct AdjSums {
+    double* red;
+    unsigned* ticket;
+    double* dtau;
+    double* dbeta_in;
+};
+
+// The tail of a persistent adjoint kernel, reached by every thread of its
+// (at most 128-thread) blocks.  The last block sums the block partials in an
+// order that depends on the grid alone, so the result does not depend on
+// scheduling; nothing waits.  Saves a launch per step (1600 cells 21 -> 18 us;
+// in the staged FP32 kernels it cost the main loop 1.5 % on the 256^3 box, so
+// they keep k_finalize).  BIN: the dL/dbeta_in terms exist (an inflow plane).
+template <typename T, bool BIN>
+__device__ __forceinline__ void block_sums(double tau, double b0, double b1, double b2, bool has_b, const AdjSums& out) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int NC = BIN ? 4 : 1;
+    __shared__ double part[4][NC];
+    __shared__ double sm[128];
+    __shared__ bool last;
+    double v[4] = {tau, b0, b1, b2};
+    if constexpr (sizeof(T) == 4) {
+        float t = (float)tau;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) a[j] += red[(b + j * 256) * 4 + k];
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(full, t, off);
+        v[0] = (double)t;
+    } else {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v[0] += __shfl_xor_sync(full, v[0], off);
     }
+    if (BIN && __any_sync(full, has_b)) {
 #pragma unroll
-    for (int j = 0; j < 7; ++j)
-        if (b + j * 256 < nslots) a[j] += red[(b + j * 256) * 4 + k];
-    sm[k][t] = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+        for (int k = 1; k < 4; ++k)
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(full, v[k], off);
+    }
+    const int tid = threadIdx.x, nw = blockDim.x >> 5;
+    if ((tid & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < NC; ++k) part[tid >> 5][k] = v[k];
     __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (t < h) sm[k][t] += sm[k][t + h];
+    if (tid < NC) {
+        double s = part[0][tid];
+        for (int w = 1; w < nw; ++w) s += part[w][tid];
+        out.red[blockIdx.x * 4 + tid] = s;
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) {
+        last = atomicAdd(out.ticket, 1u) == gridDim.x - 1;
+        if (last) *out.ticket = 0u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int k = tid % NC, step = (int)blockDim.x / NC, nb = (int)gridDim.x;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int b = tid / NC;
+    for (; b + 3 * step < nb; b += 4 * step)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[j] += __ldcg(out.red + (b + j * step) * 4 + k);
+    for (int j = 0; j < 3; ++j)
+        if (b + j * step < nb) a[j] += __ldcg(out.red + (b + j * step) * 4 + k);
+    sm[tid] = (a[0] + a[1]) + (a[2] + a[3]);
+    __syncthreads();
+    for (int h = (int)blockDim.x / 2; h >= NC; h >>= 1) {
+        if (tid < h) sm[tid] += sm[tid + h];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        if (dtau) *dtau += sm[0][0];
-        if (dbeta_in) {
-            dbeta_in[0] += sm[1][0];
-            dbeta_in[1] += sm[2][0];
-            dbeta_in[2] += sm[3][0];
+    if (tid == 0) {
+        *out.dtau += sm[0];
+        if (BIN) {
+            out.dbeta_in[0] += sm[NC > 1 ? 1 : 0];
+            out.dbeta_in[1] += sm[NC > 1 ? 2 : 0];
+            out.dbeta_in[2] += sm[NC > 1 ? 3 : 0];
         }
+    }
+}
+
+// Sum the partial-sum slots (one per warp or per block, 4 doubles each) and
+// add them to the accumulators: block k sums component k (each on its own SM:
+// the additions of the four together were bound by one SM's FP64 pipe, 10 us
+// for 1824 slots), block 0 alone without an inflow plane, whose terms are all
+// zero.  Thread t sums slots t, t+256, ... in a fixed grouping, then a fixed
+// tree combines the 256 sums: the result does not depend on scheduling.
+__global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ red, int nslots, double* dtau,
+                                                  double* dbeta_in) {
+    __shared__ double sm[256];
+    const int k = blockIdx.x, t = threadIdx.x;
+    if (k == 0 && !dtau) return;
+    // four independent partial sums so that four loads are in flight; the
+    // grouping depends only on nslots (deterministic)
+    double a[4] = {0, 0, 0, 0};
+    int b = t;
+    for (; b + 3 * 256 < nslots; b += 4 * 256) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[j] += red[(b + j * 256) * 4 + k];
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+        if (b + j * 256 < nslots) a[j] += red[(b + j * 256) * 4 + k];
+    sm[t] = (a[0] + a[1]) + (a[2] + a[3]);
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if (t < h) sm[t] += sm[t + h];
+        __syncthreads();
+    }
+    if (t == 0) {
+        if (k == 0)
+            *dtau += sm[0];
+        else
+            dbeta_in[k - 1] += sm[0];
     }
 }
 
@@ -694,7 +778,7 @@ __device__ __forceinline__ int dup_of(int x, int nx) {
 template <typename T, int XBC, int MINB, bool PIPE>
 __global__ void __launch_bounds__(128, MINB)
     k_adjoint_step(const T* __restrict__ A, const T* __restrict__ Lin, T* __restrict__ Lout, Geom g, Phys ph,
-                   AdjConst<T> c, double* red, const T* __restrict__ inflow_t) {
+                   AdjConst<T> c, const AdjSums sums, const T* __restrict__ inflow_t) {
     const long long S = g.S;
     T tau_acc = 0;
     double bin0 = 0.0, bin1 = 0.0, bin2 = 0.0;
@@ -822,7 +906,10 @@ __global__ void __launch_bounds__(128, MINB)
             scatter_cell(muf, mug, aS, vE, vx, vy, vz, c, put);
         zero_to_ghost<T, XBC>(x, g.nx, idx, S, Lout);
     }
-    warp_partials<T>((double)tau_acc, bin0, bin1, bin2, has_b, red);
+    if constexpr (PIPE)
+        block_sums<T, XBC == XBC_INFLOW_OUTFLOW>((double)tau_acc, bin0, bin1, bin2, has_b, sums);
+    else
+        warp_partials<T>((double)tau_acc, bin0, bin1, bin2, has_b, sums.red);
 }
 
 // ---------------------------------------------------------------------------
@@ -945,7 +1032,7 @@ __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int6
                                          int64_t Tyz, int64_t Tzx, int64_t Vx, int64_t Vy, int64_t Vz, int eh, int em,
                                          const Phys& ph, const AdjFx& k, AdjFxCell& t) {
     const int kh = eh - 1079, km = em - 1079;
-    const double Ed = fx_to(E, kh);
+    const double Ed = fx_to_even(E, kh);
     t.x = fx_to(dx, kh), t.y = fx_to(dy, kh), t.z = fx_to(dz, kh);
     const double E2 = Ed + Ed;
     t.E4 = E2 + E2;
@@ -966,7 +1053,7 @@ __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int6
     const FxSplit sp = fx_split((Sx + Sy + Sz) + (Pxy + Pyz + Pzx));
     // 8 G: 13.5 / 36 = 3/8; the partial sums may wrap, the result does not
     const int64_t kap = (m0 << 2) - (fx_mul(sp, k.kS1) << 2) + 4;
-    auto g38 = [](int64_t v, int64_t k8) { return (v + (v << 1) + k8) >> 3; };
+    auto g38 = [](int64_t v, int64_t k8) { return fx_weight((v + (v << 1) + k8) >> 3); };
     const double Gxx = fx_to(g38(Sx + Pxy + Pzx, kap), km), Gyy = fx_to(g38(Sy + Pxy + Pyz, kap), km),
                  Gzz = fx_to(g38(Sz + Pyz + Pzx, kap), km);
     const double Gxy = fx_to(g38(Txy, 4), km), Gxz = fx_to(g38(Tzx, 4), km), Gyz = fx_to(g38(Tyz, 4), km);
@@ -984,9 +1071,9 @@ __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int6
 // coefficients of the output.
 __device__ __forceinline__ void adj_fx_f(int64_t Sf, int64_t fd, int64_t Fs, int64_t Fx, int64_t Fy, int64_t Fz, int fh,
                                          int ef, const Phys& ph, const AdjFx& k, AdjFxCell& t) {
-    const double Sd = fx_to(Sf, fh - 1079);
+    const double Sd = fx_to_even(Sf, fh - 1079);
     const int kf = ef - 1079;
-    const double fx = fx_to(Fx, kf), fy = fx_to(Fy, kf), fz = fx_to(Fz, kf);
+    const double fx = fx_to(fx_weight(Fx), kf), fy = fx_to(fx_weight(Fy), kf), fz = fx_to(fx_weight(Fz), kf);
     const double Fu = fma(fx, t.ux, fma(fy, t.uy, fz * t.uz));
     const double aS = fma(0.25, Fu, fx_to(fx_mul(fx_split(Fs), k.kS36), kf - 1));
     t.tsum += fx_to(fd, ef + fh - 2102) - Sd * aS;
@@ -1026,7 +1113,7 @@ template <int XBC>
 __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
     k_adjoint_step_fx(const double* __restrict__ A, const double* __restrict__ Lin, double* __restrict__ Lout,
                       const __grid_constant__ Geom g, const __grid_constant__ Phys ph,
-                      const __grid_constant__ AdjConst<double> c, const __grid_constant__ AdjFx k, double* red,
+                      const __grid_constant__ AdjConst<double> c, const __grid_constant__ AdjFx k, const AdjSums sums,
                       const double* __restrict__ inflow_t) {
     const long long S = g.S;
     // This thread's column: mu_f (0..18), mu_g (19..37), then h_g and later
@@ -1287,7 +1374,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         }
         zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
     }
-    warp_partials<double>(tau_acc, bin0, bin1, bin2, has_b, red);
+    block_sums<double, XBC == XBC_INFLOW_OUTFLOW>(tau_acc, bin0, bin1, bin2, has_b, sums);
 }
 
 // Eight lanes per cell (lattices of at most 32 cells per SM, two warps per
@@ -1299,7 +1386,7 @@ template <int XBC>
 __global__ void __launch_bounds__(128)
     k_adjoint_step_fx_split(const double* __restrict__ A, const double* __restrict__ Lin, double* __restrict__ Lout,
                             const __grid_constant__ Geom g, const __grid_constant__ Phys ph,
-                            const __grid_constant__ AdjConst<double> c, const __grid_constant__ AdjFx k, double* red,
+                            const __grid_constant__ AdjConst<double> c, const __grid_constant__ AdjFx k, const AdjSums sums,
                             const double* __restrict__ inflow_t) {
     const unsigned full = 0xffffffffu;
     const long long S = g.S;
@@ -1472,7 +1559,7 @@ __global__ void __launch_bounds__(128)
             }
         }
     }
-    warp_partials<double>(tau_acc, bin0, bin1, bin2, XBC == XBC_INFLOW_OUTFLOW, red);
+    block_sums<double, XBC == XBC_INFLOW_OUTFLOW>(tau_acc, bin0, bin1, bin2, true, sums);
 }
 
 // ---------------------------------------------------------------------------
@@ -2262,17 +2349,17 @@ static AdjFxShape adj_fx_shape(long long N, int nsm) {
 }
 
 static void launch_adjoint_fx(const Geom& g, const Phys& ph, const AdjConst<double>& c, const double* A,
-                              const double* Li, double* Lo, double* red, const AdjFxShape& sh, const double* inflow_t,
+                              const double* Li, double* Lo, const AdjSums& sums, const AdjFxShape& sh, const double* inflow_t,
                               cudaStream_t st) {
     AdjFx k;
     double qh, ql;
     fx_div2(5.0, 3.0, qh, ql);
     k.kS1 = fx_const(qh, ql, 62);
     fx_div2(1.0, 36.0, qh, ql);
-    k.kS36 = fx_const(qh, ql, 65);
+    k.kS36 = fx_const_w(qh, ql, 65);
     k.kE1 = ph.fx.kE1;
     k.kE0 = ph.fx.kE0;
-    auto go = [&](auto kern) { kern<<<sh.grid, sh.threads, 0, st>>>(A, Li, Lo, g, ph, c, k, red, inflow_t); };
+    auto go = [&](auto kern) { kern<<<sh.grid, sh.threads, 0, st>>>(A, Li, Lo, g, ph, c, k, sums, inflow_t); };
     switch (g.xbc) {
         case XBC_PERIODIC:
             sh.split ? go(k_adjoint_step_fx_split<XBC_PERIODIC>) : go(k_adjoint_step_fx<XBC_PERIODIC>);
@@ -2287,7 +2374,7 @@ static void launch_adjoint_fx(const Geom& g, const Phys& ph, const AdjConst<doub
 }
 
 template <typename T>
-static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li, T* Lo, double* red, int nb,
+static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li, T* Lo, const AdjSums& sums, int nb,
                           const double* inflow_d, cudaStream_t st) {
     const AdjConst<T> c = make_adj_const<T>(ph);
     const T* inflow_t = inflow_table<T>(inflow_d);
@@ -2301,11 +2388,12 @@ static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li
         const int pg = nsm * minb;
         return pg < nb ? pg : nb;
     };
-    // each launcher returns the number of warps whose partial sums it wrote
+    // returns the number of warps whose partial sums are left for k_finalize
+    // (0: a kernel that adds up its own)
     auto go = [&](auto kern, bool pipe, int minb) {
         const int grid = pipe ? persistent_grid(minb) : nb;
-        kern<<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, red, inflow_t);
-        return grid * 4;
+        kern<<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, sums, inflow_t);
+        return pipe ? 0 : grid * 4;
     };
     int warps = 0;
     if constexpr (sizeof(T) == 4) {
@@ -2320,7 +2408,7 @@ static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li
             auto staged = [&](auto kern) {
                 smem_opt_in((const void*)kern, (int)kStageSmemBytes);  // a failure shows at the launch
                 const int grid = persistent_grid(3);
-                kern<<<grid, kStageThreads, kStageSmemBytes, st>>>(A, Li, Lo, g, ph, c, red, inflow_t, tab);
+                kern<<<grid, kStageThreads, kStageSmemBytes, st>>>(A, Li, Lo, g, ph, c, sums.red, inflow_t, tab);
                 return grid * (kStageThreads / 32);
             };
             // 16-byte copies of lambda_t+1: the buffer must be 16-byte aligned
@@ -2343,8 +2431,8 @@ static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li
         if (ph.fx_on) {
             persistent_grid(1);  // the SM count
             const AdjFxShape sh = adj_fx_shape(g.N, nsm);
-            launch_adjoint_fx(g, ph, c, A, Li, Lo, red, sh, inflow_t, st);
-            return sh.warps();
+            launch_adjoint_fx(g, ph, c, A, Li, Lo, sums, sh, inflow_t, st);
+            return 0;
         }
         switch (g.xbc) {
             case XBC_PERIODIC: warps = go(k_adjoint_step<T, XBC_PERIODIC, 2, true>, true, 2); break;
@@ -2368,18 +2456,19 @@ static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li
 }
 
 cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const void* A, const void* lam_in,
-                                void* lam_out, double* red, const double* inflow_d, double* dtau, double* dbeta_in,
-                                cudaStream_t st) {
+                                void* lam_out, double* red, unsigned* ticket, const double* inflow_d, double* dtau,
+                                double* dbeta_in, cudaStream_t st) {
     const int nb = adj_blocks(g.N);
-    set_last_launch_count(2);
+    const AdjSums sums{red, ticket, dtau, dbeta_in};
     int warps;
     if (prec == 0)
-        warps = adjoint_step_t<double>(g, ph, (const double*)A, (const double*)lam_in, (double*)lam_out, red, nb,
+        warps = adjoint_step_t<double>(g, ph, (const double*)A, (const double*)lam_in, (double*)lam_out, sums, nb,
                                        inflow_d, st);
     else
-        warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, red, nb,
+        warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, sums, nb,
                                       inflow_d, st);
-    k_finalize<<<1, 1024, 0, st>>>(red, warps, dtau, dbeta_in);
+    if (warps) k_finalize<<<g.xbc == XBC_INFLOW_OUTFLOW ? 4 : 1, 256, 0, st>>>(red, warps, dtau, dbeta_in);
+    set_last_launch_count(warps ? 2 : 1);
     return cudaGetLastError();
 }
 
@@ -2394,7 +2483,11 @@ cudaError_t launch_adjoint_fields(int prec, const Geom& g, const Phys& ph, const
     else
         k_adjoint_fields<float><<<nb, 128, 0, st>>>(n0, eps0, beta0, (const float*)A0, (const float*)lam0, dn0, deps0,
                                                     dbeta0, g, ph, red);
-    k_finalize<<<1, 1024, 0, st>>>(red, nb, nullptr, dbeta_in);
+    // without an inflow plane every dL/dbeta_in term is zero
+    if (g.xbc == XBC_INFLOW_OUTFLOW)
+        k_finalize<<<4, 256, 0, st>>>(red, nb, nullptr, dbeta_in);
+    else
+        set_last_launch_count(1);
     return cudaGetLastError();
 }
 
@@ -2408,12 +2501,14 @@ cudaError_t launch_adjoint_fields(int prec, const Geom& g, const Phys& ph, const
 // race.
 // ---------------------------------------------------------------------------
 static __device__ __align__(256) double g_adj_scratch[kAdjScratchDoubles];
+static __device__ unsigned g_adj_ticket;
 
 namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mu;
 struct ScratchSetup {
     double* ptr;    // device address of g_adj_scratch in the context below
+    unsigned* ticket;  // and of g_adj_ticket
     int nsm;        // SM count of the device
     CUcontext ctx;  // the context the set-up was made in
 };
@@ -2425,7 +2520,7 @@ ScratchSetup g_scratch[kMaxDevices];
 // not loaded yet), so that no later call loads code, which can allocate.
 // Redone when the device's context is not the one it was made in (after
 // cudaDeviceReset the old address is stale).
-cudaError_t scratch_for_device(int dev, double** ptr, int* nsm) {
+cudaError_t scratch_for_device(int dev, double** ptr, unsigned** ticket, int* nsm) {
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     const CUcontext ctx = current_context();
     std::lock_guard<std::mutex> lock(g_scratch_mu);
@@ -2434,6 +2529,8 @@ cudaError_t scratch_for_device(int dev, double** ptr, int* nsm) {
         s.ptr = nullptr;
         double* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress((void**)&p, g_adj_scratch);
+        if (e != cudaSuccess) return e;
+        e = cudaGetSymbolAddress((void**)&s.ticket, g_adj_ticket);
         if (e != cudaSuccess) return e;
         int n = 0;
         e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
@@ -2476,26 +2573,25 @@ cudaError_t scratch_for_device(int dev, double** ptr, int* nsm) {
         s.ptr = p;
     }
     *ptr = s.ptr;
+    *ticket = s.ticket;
     *nsm = s.nsm;
     return cudaSuccess;
 }
 
 template <typename T, int MINB>
-int adjoint_step_noalloc_t(const Geom& g, const Phys& ph, const T* A, const T* Li, T* Lo, double* red, int grid,
+int adjoint_step_noalloc_t(const Geom& g, const Phys& ph, const T* A, const T* Li, T* Lo, const AdjSums& sums, int grid,
                            const double* inflow_d, cudaStream_t st) {
     const AdjConst<T> c = make_adj_const<T>(ph);
     const T* inflow_t = inflow_table<T>(inflow_d);
     switch (g.xbc) {
         case XBC_PERIODIC:
-            k_adjoint_step<T, XBC_PERIODIC, MINB, true><<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, red, inflow_t);
+            k_adjoint_step<T, XBC_PERIODIC, MINB, true><<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, sums, inflow_t);
             break;
         case XBC_INFLOW_OUTFLOW:
-            k_adjoint_step<T, XBC_INFLOW_OUTFLOW, MINB, true><<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, red,
-                                                                                   inflow_t);
+            k_adjoint_step<T, XBC_INFLOW_OUTFLOW, MINB, true><<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, sums, inflow_t);
             break;
         default:
-            k_adjoint_step<T, XBC_OUTFLOW_BOTH, MINB, true><<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, red,
-                                                                                 inflow_t);
+            k_adjoint_step<T, XBC_OUTFLOW_BOTH, MINB, true><<<grid, 128, 0, st>>>(A, Li, Lo, g, ph, c, sums, inflow_t);
             break;
     }
     return grid;
@@ -2511,7 +2607,9 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
     if (e != cudaSuccess) return e;
     double* red = nullptr;
     int nsm = 0;
-    e = scratch_for_device(dev, &red, &nsm);
+    unsigned* ticket = nullptr;
+    e = scratch_for_device(dev, &red, &ticket, &nsm);
+    const AdjSums sums{red, ticket, dtau, dbeta_in};
     if (e != cudaSuccess) return e;
     const int nb = adj_blocks(g.N);
     if (prec == 0 && ph.fx_on) {
@@ -2519,10 +2617,9 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
         const long long need = 4ll * sh.warps();
         if (need_doubles) *need_doubles = need;
         if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
-        set_last_launch_count(2);
+        set_last_launch_count(1);
         launch_adjoint_fx(g, ph, make_adj_const<double>(ph), (const double*)A, (const double*)lam_in, (double*)lam_out,
-                          red, sh, inflow_table<double>(inflow_d), st);
-        k_finalize<<<1, 1024, 0, st>>>(red, sh.warps(), dtau, dbeta_in);
+                          sums, sh, inflow_table<double>(inflow_d), st);
         return cudaGetLastError();
     }
     if (prec != 0 && g.adj_pipe == 2) {
@@ -2532,10 +2629,10 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
         const long long need = 16ll * grid3;
         if (need_doubles) *need_doubles = need;
         if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
-        set_last_launch_count(2);
-        const int warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, red, nb,
+        const int warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, sums, nb,
                                                 inflow_d, st);
-        k_finalize<<<1, 1024, 0, st>>>(red, warps, dtau, dbeta_in);
+        k_finalize<<<g.xbc == XBC_INFLOW_OUTFLOW ? 4 : 1, 256, 0, st>>>(red, warps, dtau, dbeta_in);
+        set_last_launch_count(2);
         return cudaGetLastError();
     }
     const int minb = prec == 0 ? 2 : 4;
@@ -2543,14 +2640,13 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
     const long long need = 16ll * grid;  // 4 warps x 4 partial sums per block
     if (need_doubles) *need_doubles = need;
     if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
-    set_last_launch_count(2);
+    set_last_launch_count(1);
     if (prec == 0)
-        adjoint_step_noalloc_t<double, 2>(g, ph, (const double*)A, (const double*)lam_in, (double*)lam_out, red, grid,
+        adjoint_step_noalloc_t<double, 2>(g, ph, (const double*)A, (const double*)lam_in, (double*)lam_out, sums, grid,
                                           inflow_d, st);
     else
-        adjoint_step_noalloc_t<float, 4>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, red, grid,
+        adjoint_step_noalloc_t<float, 4>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, sums, grid,
                                          inflow_d, st);
-    k_finalize<<<1, 1024, 0, st>>>(red, grid * 4, dtau, dbeta_in);
     return cudaGetLastError();
 }
 

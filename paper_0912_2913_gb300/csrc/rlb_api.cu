@@ -133,7 +133,7 @@ void layout(const rlb_params* p, long long* S, int* elem, size_t* state_bytes) {
 }
 
 size_t counters_bytes() {
-    return align_up(sizeof(unsigned long long) * (2 * kCounterSlots + 3), kAlign) + align_up((sizeof(double) + sizeof(float)) * kInflowTable, kAlign);
+    return align_up(sizeof(unsigned long long) * (2 * kCounterSlots + 4), kAlign) + align_up((sizeof(double) + sizeof(float)) * kInflowTable, kAlign);
 }
 size_t red_bytes(const rlb_params* p) {
     return align_up(sizeof(double) * adj_red_doubles((long long)p->nx * p->ny * p->nz), kAlign);
@@ -302,9 +302,14 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
     c->cnt.first_bad = c->cnt.slots + 2 * kCounterSlots;
     c->cnt.macro_bad = c->cnt.first_bad + 1;
     c->cnt.pipe_err = c->cnt.first_bad + 2;
-    c->inflow_d = (double*)(base + 2 * sb + align_up(sizeof(unsigned long long) * (2 * kCounterSlots + 3), kAlign));
+    c->cnt.adj_ticket = (unsigned*)(c->cnt.first_bad + 3);
+    c->inflow_d = (double*)(base + 2 * sb + align_up(sizeof(unsigned long long) * (2 * kCounterSlots + 4), kAlign));
     c->red = (double*)(base + 2 * sb + counters_bytes());
     s = reset_counters(c);
+    if (s == RLB_OK) {
+        e = cudaMemsetAsync(c->cnt.adj_ticket, 0, sizeof(unsigned long long), c->stream);
+        if (e != cudaSuccess) s = cuda_fail(c, e, "reset ticket");
+    }
     if (s == RLB_OK) s = after_launch(c, launch_inflow_derivs(c->ph, c->inflow_d, c->stream), "inflow table");
     if (s != RLB_OK) {
         rlb_destroy(c);
@@ -587,7 +592,7 @@ rlb_status rlb_adjoint_step(rlb_ctx* c, const void* state_t, const void* lam_in,
     if (c->g.zhalo) return fail(c, RLB_ERR_ARG, "the discrete adjoint covers whole lattices (no z slabs)");
     if (!state_t || !lam_in || !lam_out || lam_in == lam_out) return fail(c, RLB_ERR_ARG, "bad buffers");
     if (!dL_dtau_accum || !dL_dbeta_in_accum) return fail(c, RLB_ERR_ARG, "accumulators are required");
-    return after_launch(c, launch_adjoint_step(c->p.prec, c->g, c->ph, state_t, lam_in, lam_out, c->red, c->inflow_d,
+    return after_launch(c, launch_adjoint_step(c->p.prec, c->g, c->ph, state_t, lam_in, lam_out, c->red, c->cnt.adj_ticket, c->inflow_d,
                                                dL_dtau_accum, dL_dbeta_in_accum, c->stream),
                         "adjoint_step");
 }

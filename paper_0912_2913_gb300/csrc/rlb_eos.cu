@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(128, 4)
             // units of 2^-61 of the scale (g_0: 2^-59)
             const int eb = m.k - 61;
             const double rw8 = rW * k.om8;  // omega / (8 W), below 1/4
-            const FxSplit r = fx_split(fx_fixed(rw8, 64));
+            const FxSplit r = fx_split(fx_weight(fx_fixed(rw8, 64)));
             const FxSplit sx = fx_split(m.dx), sy = fx_split(m.dy), sz = fx_split(m.dz);
             const FxSplit wx = fx_split(fx_mul(sx, r) << 3), wy = fx_split(fx_mul(sy, r) << 3),
                           wz = fx_split(fx_mul(sz, r) << 3);  // omega u / 8, x 2^64
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(128, 6) k_init_eos(const double* __restrict__ 
         t.uz = fx_mul(vz, c.kU) << c.sU;
         const int64_t X = t.Pxx + t.Pyy + t.Pzz, Pi = fx_scaled(P, we, 61);
         t.A = fx_mul(fx_split(Pi), k.kP) - fx_mul(fx_split(X << 1), k.k3);
-        const int64_t g0 = ((xw - Pi + 2) >> 2) - fx_mul(fx_split(Pi << 1), k.kc2) - ((X + 1) >> 1);
+        const int64_t g0 = fx_weight((xw - Pi + 2) >> 2) - fx_mul(fx_split(Pi << 1), k.kc2) - ((X + 1) >> 1);
         const int gb = we - 1085, fb = se - 1085;
         put(19, fx_to(g0, gb + 3));
         const FxSplit s12 = fx_split(fx_mul(xs, c.kS12) << 2);
@@ -631,7 +631,7 @@ FxConst over_c2(const Phys& ph, double num, double den, int s) {
     double qh, ql;
     fx_div2(num, den, qh, ql);
     const double th = qh / c2, tl = (fma(-th, c2, qh) + (ql - th * c2l)) / c2;
-    return fx_const(th, tl, s);
+    return fx_const_w(th, tl, s);
 }
 
 FxEosInit make_fx_eos_init(const Phys& ph) {
@@ -651,11 +651,11 @@ FxEos make_fx_eos(const Phys& ph) {
     double qh, ql;
     k.kP = over_c2(ph, om, 12.0, 64);
     k.kP0 = over_c2(ph, om, 1.0, 62);
-    k.kE0 = fx_const(om, 0.0, 62);
+    k.kE0 = fx_const_w(om, 0.0, 62);
     fx_div2(om, 12.0, qh, ql);
-    k.kU = fx_const(qh, ql, 64);
+    k.kU = fx_const_w(qh, ql, 64);
     fx_div2(om, 36.0, qh, ql);
-    k.kS = fx_const(qh, ql, 64);
+    k.kS = fx_const_w(qh, ql, 64);
     fx_div2(1.0, 3.0, qh, ql);
     k.k3 = fx_const(qh, ql, 63);
     fx_div2(2.0, 3.0, qh, ql);

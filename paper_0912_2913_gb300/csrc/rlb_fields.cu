@@ -376,7 +376,7 @@ FxInit make_fx_init(const Phys& ph, int prec) {
         double qh, ql;
         fx_div2(num, den, qh, ql);
         const double th = qh / c2, tl = (fma(-th, c2, qh) + (ql - th * c2l)) / c2;
-        return fx_const(th, tl, s);
+        return fx_const_w(th, tl, s);
     };
     // FP64 populations lose low bits with c_l (see k_step_f64_fx); binary32
     // ones are rounded far above them
@@ -401,11 +401,11 @@ FxInit make_fx_init(const Phys& ph, int prec) {
     double oh, ol;
     fx_div2(1.0, 3.0, oh, ol);
     const double dh = oh - th, de = (oh - (dh + th)) + (ol - tl);
-    k.k0 = fx_const(dh, de, 64);
+    k.k0 = fx_const_w(dh, de, 64);
     fx_div2(1.0, 36.0, qh, ql);
-    k.kS = fx_const(qh, ql, 65);
+    k.kS = fx_const_w(qh, ql, 65);
     fx_div2(1.0, 12.0 * c, qh, ql);
-    k.kS12 = fx_const(qh, ql, 65);
+    k.kS12 = fx_const_w(qh, ql, 65);
     // exponents (high words) that leave every product and the output in range
     k.lo = (prec == 0 ? 200 : 1023 - 110) << 20;
     k.hi = (prec == 0 ? 1800 : 1023 + 110) << 20;

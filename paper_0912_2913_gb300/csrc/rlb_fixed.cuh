@@ -26,6 +26,11 @@
 //   g_0 = w_0 [E (3 - 2 / c_l^2) + 1.5 d.u],
 // which needs neither gamma^2 nor a subtraction of nearly equal terms.
 //
+// Weights: the lattice weights are the binary64 numbers nearest 1/3, 1/18 and
+// 1/36, as in the binary64 kernels.  All three are (1 - 2^-54) of the
+// fraction, so the equilibria carry that factor: over thousands of steps a
+// scheme with the exact fractions would drift away from them by 2^-54 a step.
+//
 // Everything here is integer or explicitly rounded, so the kernels that use
 // it (one cell per thread, eight lanes per cell) give the same values.  The
 // functions compile for the host as well (checks of the arithmetic).
@@ -160,6 +165,9 @@ RLB_FX int64_t fx_from(double v, int emax) {
     return (int64_t)((x ^ (uint64_t)s) - (uint64_t)s);
 }
 
+// the factor (1 - 2^-54) of the binary64 weights
+RLB_FX int64_t fx_weight(int64_t v) { return v - (v >> 54); }
+
 // v 2^s for v >= 0 with v 2^s < 2^63 (truncated)
 RLB_FX int64_t fx_fixed(double v, int s) {
     const uint32_t hi = (uint32_t)fx_hi(v), lo = fx_lo(v);
@@ -185,6 +193,20 @@ RLB_FX double fx_to(int64_t t, int eb) {
     }
     a = (a << n) + 512u;  // leading bit at 62; round half up in the 53rd bit
     const uint64_t m = a >> 10;
+    const uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(1084 + eb - n) << 20);
+    return fx_double(hi | ((uint32_t)s & 0x80000000u), (uint32_t)m);
+}
+
+// fx_to with ties to even: for sums of binary64 values, whose few excess bits
+// make ties common (near rest, rounding them up is a bias of 2^-55 a cell).
+RLB_FX double fx_to_even(int64_t t, int eb) {
+    const int32_t s = (int32_t)(t >> 63);
+    uint64_t a = (uint64_t)((t ^ (int64_t)s) - (int64_t)s);
+    const uint32_t ah = (uint32_t)(a >> 32);
+    if (a == 0) return 0.0;
+    const int n = ah != 0u ? fx_clz(ah) - 1 : 31 + fx_clz((uint32_t)a);
+    a <<= n;
+    const uint64_t m = (a + 511u + ((uint32_t)(a >> 10) & 1u)) >> 10;
     const uint32_t hi = (uint32_t)(m >> 32) + ((uint32_t)(1084 + eb - n) << 20);
     return fx_double(hi | ((uint32_t)s & 0x80000000u), (uint32_t)m);
 }
@@ -301,7 +323,7 @@ RLB_FX bool fx_g_terms(int64_t E, int64_t dx, int64_t dy, int64_t dz, int emax, 
     double D;
     r_d = fx_reciprocal_D(Ed, u_d[0], u_d[1], u_d[2], k, D);
     const double rW = r_d * k.om4;  // (omega / 4) / D
-    const FxSplit r = fx_split(fx_fixed(rW, 65));
+    const FxSplit r = fx_split(fx_weight(fx_fixed(rW, 65)));
     const FxSplit sx = fx_split(dx), sy = fx_split(dy), sz = fx_split(dz);
     // w = d r: (d 2^61)(rW 2^65) 2^-64 = w 2^62, then x 8
     t.wx = fx_split(fx_mul(sx, r) << 3);

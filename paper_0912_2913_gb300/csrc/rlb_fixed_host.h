@@ -14,3 +14,8 @@ inline FxConst fx_const(int64_t v) {
 inline FxConst fx_const(double hi, double lo, int s) {
     return fx_const((int64_t)ldexp(hi, s) + (int64_t)llrint(ldexp(lo, s)));
 }
+// (hi + lo) 2^s times the factor (1 - 2^-54) of the binary64 weights
+inline FxConst fx_const_w(double hi, double lo, int s) {
+    const int64_t v = (int64_t)ldexp(hi, s) + (int64_t)llrint(ldexp(lo, s));
+    return fx_const(v - (v >> 54));
+}

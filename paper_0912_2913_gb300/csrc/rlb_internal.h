@@ -80,6 +80,7 @@ struct Counters {
     unsigned long long* slots;      // [2][kCounterSlots]: unphysical, non-positive equilibria
     unsigned long long* first_bad;  // min over flagged updates of step*N + cell
     unsigned long long* macro_bad;  // cells flagged by the last macro evaluation
+    unsigned* adj_ticket;           // blocks of an adjoint kernel that have left their sums (0 between launches)
     unsigned long long* pipe_err;   // set when a staged kernel gave up waiting for its copies
 };
 
@@ -125,8 +126,8 @@ inline long long adj_red_doubles(long long N) { return N <= kAdjSplitCells ? N +
 cudaError_t launch_adjoint_macro(int prec, const Geom& g, const Phys& ph, const void* A, const double* dn,
                                  const double* deps, const double* dbeta, void* lam, cudaStream_t stream);
 cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const void* A, const void* lam_in,
-                                void* lam_out, double* red, const double* inflow_d, double* dtau, double* dbeta_in,
-                                cudaStream_t stream);
+                                void* lam_out, double* red, unsigned* ticket, const double* inflow_d, double* dtau,
+                                double* dbeta_in, cudaStream_t stream);
 // Allocation-free variant of launch_adjoint_step (same kernels, persistent
 // grid): partial sums in a static device array of kAdjScratchDoubles doubles,
 // set up once per device on first use.  Needs 16 doubles per block of the

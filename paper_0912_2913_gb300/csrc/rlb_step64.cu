@@ -730,20 +730,20 @@ FxRun make_fx_run(double omega, double c_l) {
     fx_div2(omega, 36.0, qh, ql);
     th = qh / c2h;
     tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
-    k.kE = fx_const(th, tl, 65);
-    k.kS = fx_const(qh, ql, 65);
+    k.kE = fx_const_w(th, tl, 65);
+    k.kS = fx_const_w(qh, ql, 65);
     fx_div2(omega, 12.0, qh, ql);
-    k.kU = fx_const(qh, ql, 65);
+    k.kU = fx_const_w(qh, ql, 65);
     // omega (1 - 2 / (3 c_l^2)) = omega - 24 omega / (36 c_l^2)
     const int64_t kE65 = (int64_t)ldexp(th, 65) + (int64_t)llrint(ldexp(tl, 65));
     const int64_t v = (int64_t)ldexp(omega, 62) - 3 * kE65;
-    k.k0 = fx_const(v);
+    k.k0 = fx_const(v - (v >> 54));
     fx_div2(1.0, 36.0, qh, ql);
     th = qh / c2h;
     tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
-    k.kE1 = fx_const(th, tl, 65);
+    k.kE1 = fx_const_w(th, tl, 65);
     // (3 - 2 / c_l^2) / 3 = 1 - 24 / (36 c_l^2)
-    k.kE0 = fx_const(1.0 - 24.0 * th, fma(-24.0, th, 1.0) - (1.0 - 24.0 * th) - 24.0 * tl, 62);
+    k.kE0 = fx_const_w(1.0 - 24.0 * th, fma(-24.0, th, 1.0) - (1.0 - 24.0 * th) - 24.0 * tl, 62);
     fx_div2(5.0, 9.0, qh, ql);
     k.kQ = fx_const(qh, ql, 63);
     fx_div2(1.0, 6.0, qh, ql);
