@@ -324,8 +324,7 @@ __device__ __forceinline__ bool eos_moments(const double* g, int em, EosMoments&
     if (n > 12 || !(xf * xf + yf * yf + zf * zf < Ef * Ef)) return false;
     m.E = E << n, m.dx = dx << n, m.dy = dy << n, m.dz = dz << n;
     m.k = em - 1018 - n;
-    const int64_t Er = (m.E + 256) >> 9;
-    m.Ed = fx_double((uint32_t)(Er >> 32) + (1022u << 20), (uint32_t)Er);
+    m.Ed = fx_unit(m.E);
     m.x = fx_to(m.dx, -61), m.y = fx_to(m.dy, -61), m.z = fx_to(m.dz, -61);
     return true;
 }
@@ -347,6 +346,7 @@ struct FxEos {
     FxConst kS;   // omega / 36          x 2^64
     FxConst k3;   // 1 / 3               x 2^63
     FxConst k23;  // 2 / 3               x 2^63
+    int64_t om57;     // omega x 2^57
     double om8, omw;  // omega / 8, 1 - omega
 };
 
@@ -411,8 +411,15 @@ __global__ void __launch_bounds__(128, 4)
         if (ok) {
             // units of 2^-61 of the scale (g_0: 2^-59)
             const int eb = m.k - 61;
-            const double rw8 = rW * k.om8;  // omega / (8 W), below 1/4
-            const FxSplit r = fx_split(fx_weight(fx_fixed(rw8, 64)));
+            // omega / (8 W), below 1/4, x 2^64, with the residual of the sum
+            // E + P in fixed point: without it the roundings of W, of 1/W and
+            // of this product are common to every term that is linear in u
+            // (and are most of the error of a population that they cancel in)
+            const int64_t Pi = fx_fixed(P, 61);
+            int64_t r8 = fx_fixed(rW * k.om8, 64);
+            const int64_t rest = k.om57 - fx_mul(fx_split((int64_t)((uint64_t)(m.E + Pi) >> 1)), fx_split(r8));
+            r8 += (int64_t)__float2int_rn((float)(int32_t)rest * 16.0f * fx_seed_f32(rW));
+            const FxSplit r = fx_split(fx_weight(r8));
             const FxSplit sx = fx_split(m.dx), sy = fx_split(m.dy), sz = fx_split(m.dz);
             const FxSplit wx = fx_split(fx_mul(sx, r) << 3), wy = fx_split(fx_mul(sy, r) << 3),
                           wz = fx_split(fx_mul(sz, r) << 3);  // omega u / 8, x 2^64
@@ -426,7 +433,7 @@ __global__ void __launch_bounds__(128, 4)
             t.ux = fx_mul(sx, k.kU);
             t.uy = fx_mul(sy, k.kU);
             t.uz = fx_mul(sz, k.kU);
-            const int64_t X = t.Pxx + t.Pyy + t.Pzz, Pi = fx_fixed(P, 61);
+            const int64_t X = t.Pxx + t.Pyy + t.Pzz;
             t.A = fx_mul(fx_split(Pi), k.kP) - fx_mul(fx_split(X << 1), k.k3);
             const int64_t g0 = fx_mul(fx_split(m.E), k.kE0) - fx_mul(fx_split(Pi << 1), k.kP0) - X;
             int64_t low = g0 - 1;  // negative when an equilibrium is not positive
@@ -509,7 +516,10 @@ __global__ void __launch_bounds__(128, 6) k_init_eos(const double* __restrict__ 
     if (c.on && oh > 0x3F900000 && oh < 0x3FF00001 && nh > c.lo && nh < c.hi && eh > c.lo && eh < c.hi &&
         Ph > eh - (10 << 20) && Ph <= eh + (1 << 20)) {
         const double gam = rsqrt_unit(omb2);
-        const double W = (ee + P) * (gam * gam), sn = nn * gam;
+        // gamma^2 and gamma to their last bit: an error here is common to all
+        // populations of a cell, and stays in its conserved moments
+        const double g2 = gam * gam, gh = fma(-omb2, g2, 1.0);
+        const double W = (ee + P) * fma(g2, gh, g2), sn = nn * fma(0.5 * gh, gam, gam);
         int we, se;
         const int64_t xw = fx_mantissa(W, we);
         const FxSplit xs = fx_split(fx_mantissa(sn, se));
@@ -660,6 +670,7 @@ FxEos make_fx_eos(const Phys& ph) {
     k.k3 = fx_const(qh, ql, 63);
     fx_div2(2.0, 3.0, qh, ql);
     k.k23 = fx_const(qh, ql, 63);
+    k.om57 = (int64_t)(om * 0x1p57);
     k.om8 = 0.125 * om;
     k.omw = 1.0 - om;
     return k;

@@ -211,6 +211,12 @@ RLB_FX double fx_to_even(int64_t t, int eb) {
     return fx_double(hi | ((uint32_t)s & 0x80000000u), (uint32_t)m);
 }
 
+// x 2^-61 for x in [2^61, 2^62), ties to even
+RLB_FX double fx_unit(int64_t x) {
+    const int64_t r = (x + 255 + ((x >> 9) & 1)) >> 9;
+    return fx_double((uint32_t)(r >> 32) + (1022u << 20), (uint32_t)r);
+}
+
 // a split for products: value = h 2^32 + 2 l (the lowest bit dropped)
 struct FxSplit {
     int32_t h, l;
@@ -315,8 +321,7 @@ RLB_FX bool fx_g_terms(int64_t E, int64_t dx, int64_t dy, int64_t dz, int emax, 
     dy <<= n;
     dz <<= n;
     t.eb = emax - 1080 - n;  // 2^-62 of the scaled value: 2^(emax-1023) 2^(61-56-n) 2^-62
-    const int64_t Er = (E + 256) >> 9;
-    const double Ed = fx_double((uint32_t)(Er >> 32) + (1022u << 20), (uint32_t)Er);
+    const double Ed = fx_unit(E);
     u_d[0] = fx_to(dx, -61);
     u_d[1] = fx_to(dy, -61);
     u_d[2] = fx_to(dz, -61);
