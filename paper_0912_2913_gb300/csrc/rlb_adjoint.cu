@@ -270,7 +270,7 @@ __device__ __forceinline__ void block_sums(double tau, double b0, double b1, dou
 __global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ red, int nslots, double* dtau,
                                                   double* dbeta_in) {
     __shared__ double sm[256];
-    const int k = blockIdx.x, t = threadIdx.x;
+    const int k = blockIdx.x, t = dependent_begin(threadIdx.x);
     if (k == 0 && !dtau) return;
     // four independent partial sums so that four loads are in flight; the
     // grouping depends only on nslots (deterministic)
@@ -1126,7 +1126,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
     double bin0 = 0.0, bin1 = 0.0, bin2 = 0.0;
     bool has_b = false;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long li = (long long)blockIdx.x * blockDim.x + tid; li < g.N; li += stride) {
+    for (long long li = dependent_begin(blockIdx.x * blockDim.x + tid); li < g.N; li += stride) {
         const int idx = (int)li;
         int x, y, z;
         cell_coords(g, idx, x, y, z);
@@ -1390,7 +1390,7 @@ __global__ void __launch_bounds__(128)
                             const double* __restrict__ inflow_t) {
     const unsigned full = 0xffffffffu;
     const long long S = g.S;
-    const long long t8 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int t8 = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);
     const int j = threadIdx.x & 7, base = threadIdx.x & 24;  // lane of the group, its first lane in the warp
     const bool live = (t8 >> 3) < g.N;
     const int idx = live ? (int)(t8 >> 3) : 0;
@@ -1620,7 +1620,7 @@ __global__ void __launch_bounds__(kStageThreads, 3)
     double bin0 = 0.0, bin1 = 0.0, bin2 = 0.0;
     bool has_b = false;
     // 64-bit loop counter: li + stride cannot wrap for any accepted N
-    long long li = (long long)blockIdx.x * blockDim.x + tid;
+    long long li = dependent_begin(blockIdx.x * blockDim.x + tid);
     int idx = li < g.N ? (int)li : 0;
     int x = 0, y = 0, z = 0;
     PullOffsets o{};
@@ -1782,7 +1782,7 @@ __global__ void __launch_bounds__(kStageThreads, 3)
     bool has_b = false;
     // block-uniform loop over the block's cells [cb, cb + 128) (every thread
     // reaches every barrier); 64-bit: cb + stride cannot wrap
-    long long cb = (long long)blockIdx.x * blockDim.x;
+    long long cb = dependent_begin(blockIdx.x * blockDim.x);
     long long li = cb + tid;
     int idx = li < g.N ? (int)li : 0;
     int x = 0, y = 0, z = 0;
@@ -2359,7 +2359,7 @@ static void launch_adjoint_fx(const Geom& g, const Phys& ph, const AdjConst<doub
     k.kS36 = fx_const_w(qh, ql, 65);
     k.kE1 = ph.fx.kE1;
     k.kE0 = ph.fx.kE0;
-    auto go = [&](auto kern) { kern<<<sh.grid, sh.threads, 0, st>>>(A, Li, Lo, g, ph, c, k, sums, inflow_t); };
+    auto go = [&](auto kern) { launch_dependent(kern, sh.grid, sh.threads, 0, st, A, Li, Lo, g, ph, c, k, sums, inflow_t); };
     switch (g.xbc) {
         case XBC_PERIODIC:
             sh.split ? go(k_adjoint_step_fx_split<XBC_PERIODIC>) : go(k_adjoint_step_fx<XBC_PERIODIC>);
@@ -2408,7 +2408,7 @@ static int adjoint_step_t(const Geom& g, const Phys& ph, const T* A, const T* Li
             auto staged = [&](auto kern) {
                 smem_opt_in((const void*)kern, (int)kStageSmemBytes);  // a failure shows at the launch
                 const int grid = persistent_grid(3);
-                kern<<<grid, kStageThreads, kStageSmemBytes, st>>>(A, Li, Lo, g, ph, c, sums.red, inflow_t, tab);
+                launch_dependent(kern, grid, kStageThreads, kStageSmemBytes, st, A, Li, Lo, g, ph, c, sums.red, inflow_t, tab);
                 return grid * (kStageThreads / 32);
             };
             // 16-byte copies of lambda_t+1: the buffer must be 16-byte aligned
@@ -2467,7 +2467,7 @@ cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const v
     else
         warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, sums, nb,
                                       inflow_d, st);
-    if (warps) k_finalize<<<g.xbc == XBC_INFLOW_OUTFLOW ? 4 : 1, 256, 0, st>>>(red, warps, dtau, dbeta_in);
+    if (warps) launch_dependent(k_finalize, g.xbc == XBC_INFLOW_OUTFLOW ? 4 : 1, 256, 0, st, red, warps, dtau, dbeta_in);
     set_last_launch_count(warps ? 2 : 1);
     return cudaGetLastError();
 }
@@ -2485,7 +2485,7 @@ cudaError_t launch_adjoint_fields(int prec, const Geom& g, const Phys& ph, const
                                                     dbeta0, g, ph, red);
     // without an inflow plane every dL/dbeta_in term is zero
     if (g.xbc == XBC_INFLOW_OUTFLOW)
-        k_finalize<<<4, 256, 0, st>>>(red, nb, nullptr, dbeta_in);
+        launch_dependent(k_finalize, 4, 256, 0, st, red, nb, (double*)nullptr, dbeta_in);
     else
         set_last_launch_count(1);
     return cudaGetLastError();
@@ -2631,7 +2631,7 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
         if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
         const int warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, sums, nb,
                                                 inflow_d, st);
-        k_finalize<<<g.xbc == XBC_INFLOW_OUTFLOW ? 4 : 1, 256, 0, st>>>(red, warps, dtau, dbeta_in);
+        launch_dependent(k_finalize, g.xbc == XBC_INFLOW_OUTFLOW ? 4 : 1, 256, 0, st, red, warps, dtau, dbeta_in);
         set_last_launch_count(2);
         return cudaGetLastError();
     }

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(128, 4)
     k_step_eos_fx(const double* __restrict__ A, double* __restrict__ B, const __grid_constant__ Geom g,
                   const __grid_constant__ Phys ph, Counters cnt, int count, long long step_index,
                   const __grid_constant__ FxEos k) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);
     if (idx >= g.N) return;
     int x, y, z;
     cell_coords(g, idx, x, y, z);
@@ -695,7 +695,9 @@ cudaError_t launch_step_eos(const Geom& g, const Phys& ph, const void* A, void* 
     const int cs = count ? 1 : 0;
     if (eos_fx_on(ph)) {
         const FxEos k = make_fx_eos(ph);
-        auto go = [&](auto kern) { kern<<<nb, 128, 0, st>>>((const double*)A, (double*)B, g, ph, cnt, cs, step_index, k); };
+        auto go = [&](auto kern) {
+            launch_dependent(kern, nb, 128, 0, st, (const double*)A, (double*)B, g, ph, cnt, cs, step_index, k);
+        };
         switch (g.xbc) {
             case XBC_PERIODIC: go(k_step_eos_fx<XBC_PERIODIC>); break;
             case XBC_INFLOW_OUTFLOW: go(k_step_eos_fx<XBC_INFLOW_OUTFLOW>); break;

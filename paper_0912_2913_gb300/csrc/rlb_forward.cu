@@ -60,7 +60,7 @@ template <int XBC, bool SOLID, int MINB, bool PREF, typename I = long long, bool
           int TB = 256>
 __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__ A, float* __restrict__ B, Geom g,
                                                        Dev32 c, Counters cnt, int count, long long step_index) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);
     if (idx >= g.N) return;
     int x, y, z;
     cell_coords(g, idx, x, y, z);
@@ -321,13 +321,13 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
             // lattice speeds above 1: the compensated collision (one launch
             // shape; the TMA-staged and tuning variants use the binary32 one)
             if (idx32)
-                k_step_f32<XBC, SOLID, 2, false, int, true><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs,
+                launch_dependent(k_step_f32<XBC, SOLID, 2, false, int, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs,
                                                                                  step_index);
             else if (split32)
-                k_step_f32<XBC, SOLID, 2, false, unsigned, true><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt,
+                launch_dependent(k_step_f32<XBC, SOLID, 2, false, unsigned, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt,
                                                                                       cs, step_index);
             else
-                k_step_f32<XBC, SOLID, 2, false, long long, true><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c,
+                launch_dependent(k_step_f32<XBC, SOLID, 2, false, long long, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c,
                                                                                        cnt, cs, step_index);
             return;
         }
@@ -335,26 +335,26 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
             return;
         cudaGetLastError();
         switch (g.variant) {
-            case 0: k_step_f32<XBC, SOLID, 3, false><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
+            case 0: launch_dependent(k_step_f32<XBC, SOLID, 3, false>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
             case 1:
                 if (idx32)
-                    k_step_f32<XBC, SOLID, 3, true, int><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);
+                    launch_dependent(k_step_f32<XBC, SOLID, 3, true, int>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index);
                 else if (split32)
-                    k_step_f32<XBC, SOLID, 3, true, unsigned><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs,
+                    launch_dependent(k_step_f32<XBC, SOLID, 3, true, unsigned>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs,
                                                                                step_index);
                 else
-                    k_step_f32<XBC, SOLID, 3, true><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);
+                    launch_dependent(k_step_f32<XBC, SOLID, 3, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index);
                 break;
             case 2:
                 if (idx32)
-                    k_step_f32<XBC, SOLID, 4, false, int><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);
+                    launch_dependent(k_step_f32<XBC, SOLID, 4, false, int>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index);
                 else if (split32)
-                    k_step_f32<XBC, SOLID, 4, false, unsigned><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs,
+                    launch_dependent(k_step_f32<XBC, SOLID, 4, false, unsigned>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs,
                                                                                 step_index);
                 else
-                    k_step_f32<XBC, SOLID, 4, false><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);
+                    launch_dependent(k_step_f32<XBC, SOLID, 4, false>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index);
                 break;
-            case 3: k_step_f32<XBC, SOLID, 4, true><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
+            case 3: launch_dependent(k_step_f32<XBC, SOLID, 4, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
             case 6:
             case 7:
             case 8: {
@@ -368,9 +368,9 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
                 const unsigned n = blocks_for(g.N, t);
 #define RLB_EARLY_LAUNCH(MB, TBK)                                                                                        \
     do {                                                                                                                 \
-        if (idx32) k_step_f32<XBC, SOLID, MB, false, int, false, true, TBK><<<n, t, 0, st>>>(a, b, g, c, cnt, cs, step_index); \
-        else if (split32) k_step_f32<XBC, SOLID, MB, false, unsigned, false, true, TBK><<<n, t, 0, st>>>(a, b, g, c, cnt, cs, step_index); \
-        else k_step_f32<XBC, SOLID, MB, false, long long, false, true, TBK><<<n, t, 0, st>>>(a, b, g, c, cnt, cs, step_index); \
+        if (idx32) launch_dependent(k_step_f32<XBC, SOLID, MB, false, int, false, true, TBK>, n, t, 0, st, a, b, g, c, cnt, cs, step_index); \
+        else if (split32) launch_dependent(k_step_f32<XBC, SOLID, MB, false, unsigned, false, true, TBK>, n, t, 0, st, a, b, g, c, cnt, cs, step_index); \
+        else launch_dependent(k_step_f32<XBC, SOLID, MB, false, long long, false, true, TBK>, n, t, 0, st, a, b, g, c, cnt, cs, step_index); \
     } while (0)
                 if (v == 6) RLB_EARLY_LAUNCH(6, 128);
                 else if (v == 7) RLB_EARLY_LAUNCH(7, 128);
@@ -388,7 +388,7 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
                     k_step_f32_pipe<XBC, SOLID, true><<<grid, 256, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);
                 break;
             }
-            default: k_step_f32<XBC, SOLID, 3, true><<<nb, tb, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
+            default: launch_dependent(k_step_f32<XBC, SOLID, 3, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
         }
     }
 }

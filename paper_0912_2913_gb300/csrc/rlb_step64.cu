@@ -7,10 +7,6 @@
 #include "rlb_device.cuh"
 #include "rlb_fixed.cuh"
 
-#ifndef RLB_FXB
-#define RLB_FXB 5
-#endif
-
 namespace rlb {
 
 // ---------------------------------------------------------------------------
@@ -423,7 +419,7 @@ __global__ void __launch_bounds__(128, MINB)
     k_step_f64_fx(const double* __restrict__ A, double* __restrict__ B, const __grid_constant__ Geom g,
                   const __grid_constant__ Phys ph, Counters cnt, int count, long long step_index,
                   const __grid_constant__ PlaneTab64 tab) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);
     if (idx >= g.N) return;
     int x, y, z;
     cell_coords(g, idx, x, y, z);
@@ -530,11 +526,11 @@ __global__ void __launch_bounds__(128)
     k_step_f64_fx_split(const double* __restrict__ A, double* __restrict__ B, const __grid_constant__ Geom g,
                         const __grid_constant__ Phys ph, Counters cnt, int count, long long step_index) {
     const unsigned full = 0xffffffffu;
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int tid = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);  // 8 N < 2^31 (small lattices; tests)
     const int j = threadIdx.x & 7;  // lane of the cell's group
-    const long long cell = tid >> 3;
+    const int cell = (int)((unsigned)tid >> 3);
     const bool live = cell < g.N;
-    const int idx = live ? (int)cell : 0;
+    const int idx = live ? cell : 0;
     int x, y, z;
     cell_coords(g, idx, x, y, z);
     const bool halo = g.zhalo && (z == 0 || z == g.nz - 1);  // filled by the exchange
@@ -699,10 +695,10 @@ void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B
     // (N <= 16 x SMs), unless RLB_F64_SPLIT says otherwise; same values.  The
     // 1600-cell tube, issued on the stream: 10.24 us per step in binary64, 8.20
     // in fixed point (20 instead of 103 FP64 instructions per warp).
-    const bool split = g.f64split == 1 || (g.f64split < 0 && g.N <= 16ll * nsm);
+    const bool split = (g.f64split == 1 && g.N < (1 << 27)) || (g.f64split < 0 && g.N <= 16ll * nsm);
     if (ph.fx_on) {
         if (split) {
-            k_step_f64_fx_split<XBC><<<blocks(8ll * g.N, 128), 128, 0, st>>>(A, B, g, ph, cnt, c, step_index);
+            launch_dependent(k_step_f64_fx_split<XBC>, blocks(8ll * g.N, 128), 128, 0, st, A, B, g, ph, cnt, c, step_index);
             return;
         }
         PlaneTab64 tab;
@@ -712,7 +708,7 @@ void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B
         }
         // small lattices spread over more SMs in 32-thread blocks
         const int tb = blocks(g.N, 128) < (unsigned)nsm ? 32 : 128;
-        k_step_f64_fx<XBC, RLB_FXB><<<blocks(g.N, tb), tb, 0, st>>>(A, B, g, ph, cnt, c, step_index, tab);
+        launch_dependent(k_step_f64_fx<XBC, 5>, blocks(g.N, tb), tb, 0, st, A, B, g, ph, cnt, c, step_index, tab);
         return;
     }
     if (split) {
