@@ -142,10 +142,8 @@ RLB_API rlb_status rlb_init_fields(rlb_ctx* ctx, const double* n, const double* 
  * (fused pull streaming with link bounce-back, moments, eps = 3P recovery,
  * equilibria Eqs. (equil1s, equil2as, equil2bs), BGK relaxation, boundary
  * planes; under RLB_EOS_GAMMA_LAW the Newton recovery and Eqs. (equil1,
- * equil2a, equil2b)).  Asynchronous, except that the first call on an RLB_FP32_DEV
- * context times its launch variants (bit-identical results) on the
- * context's second buffer and synchronises once; make that first call
- * before any stream capture.  nsteps >= 0.                                  */
+ * equil2a, equil2b)).  Asynchronous; the first call on a device loads its
+ * kernel: make it before any stream capture.  nsteps >= 0.                  */
 RLB_API rlb_status rlb_step(rlb_ctx* ctx, int32_t nsteps);
 
 /* One time step from the device state src into the device state dst (both

@@ -230,7 +230,7 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
         const char* t = getenv("RLB_TMA");
         g.tma = (t && t[0] == '1' && !g.zhalo) ? 1 : 0;  // the TMA-staged step updates every z plane
         const char* v = getenv("RLB_F32_VARIANT");
-        g.variant = v ? atoi(v) : -1;  // -1: chosen by timing at the first step
+        g.variant = v ? atoi(v) : -1;  // -1: by the number of cells (launch_step)
         const char* ap = getenv("RLB_ADJ_PIPE");
         g.adj_pipe = ap ? atoi(ap) : 2;
         const char* ac = getenv("RLB_ADJ_COOP");
@@ -389,60 +389,11 @@ rlb_status rlb_init_fields(rlb_ctx* c, const double* n, const double* eps, const
     return RLB_OK;
 }
 
-// Launch variants of the FP32 step compute bit-identical results; which one
-// is fastest depends on the lattice.  The candidates: 2 (256-thread blocks,
-// 64 registers), 7 and 8 (the f populations loaded before the g arithmetic,
-// 128 x 7 blocks at 72 registers, 64 x 12 at 80; measured fastest on the
-// 512^3 box and the 200x100x100 sphere).  The first FP32 rlb_step times
-// each on the context's second buffer (which the step then overwrites) and
-// keeps the fastest.  This first call synchronises the stream once.
-static rlb_status autotune_f32(rlb_ctx* c) {
-    const int cand[3] = {2, 7, 8};
-    float best = 1e30f;
-    int pick = 2;
-    cudaEvent_t e0, e1;
-    RLB_CUDA(c, cudaEventCreate(&e0), "event");
-    RLB_CUDA(c, cudaEventCreate(&e1), "event");
-    for (int k = 0; k < 3; ++k) {
-        c->g.variant = cand[k];
-        cudaError_t e = launch_step(c->p.prec, c->g, c->ph, c->A, c->B, c->cnt, false, 0, c->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < 3 && e == cudaSuccess; ++r)
-            e = launch_step(c->p.prec, c->g, c->ph, c->A, c->B, c->cnt, false, 0, c->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        float ms = 0.f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e != cudaSuccess) {
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            return cuda_fail(c, e, "autotune");
-        }
-        c->launches += 4;
-        if (ms < best) {
-            best = ms;
-            pick = cand[k];
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    c->g.variant = pick;
-    return RLB_OK;
-}
-
 rlb_status rlb_step(rlb_ctx* c, int32_t nsteps) {
     Nvtx nvtx_("rlb_step");
     RLB_LATCHED(c);
     if (nsteps < 0) return fail(c, RLB_ERR_ARG, "nsteps must be >= 0");
     if (!c->inited) return fail(c, RLB_ERR_STATE, "rlb_step before rlb_init_fields");
-    if (c->g.variant < 0 && nsteps > 0) {
-        if (c->p.prec == RLB_FP32_DEV && !c->g.tma) {
-            rlb_status s = autotune_f32(c);
-            if (s != RLB_OK) return s;
-        } else {
-            c->g.variant = 7;
-        }
-    }
     for (int32_t t = 0; t < nsteps; ++t) {
         rlb_status s = after_launch(c,
                                     c->ph.eos ? launch_step_eos(c->g, c->ph, c->A, c->B, c->cnt, true, c->steps, c->stream)
@@ -462,7 +413,6 @@ rlb_status rlb_step_into(rlb_ctx* c, const void* src, void* dst) {
     Nvtx nvtx_("rlb_step_into");
     RLB_LATCHED(c);
     if (!src || !dst || src == dst) return fail(c, RLB_ERR_ARG, "src and dst must be distinct device buffers");
-    if (c->g.variant < 0) c->g.variant = 7;  // untuned: the shape measured fastest on the benchmark lattices
     return after_launch(c,
                         c->ph.eos ? launch_step_eos(c->g, c->ph, src, dst, c->cnt, false, 0, c->stream)
                                   : launch_step(c->p.prec, c->g, c->ph, src, dst, c->cnt, false, 0, c->stream),
@@ -474,7 +424,6 @@ rlb_status rlb_step_into_counted(rlb_ctx* c, const void* src, void* dst) {
     RLB_LATCHED(c);
     if (!src || !dst || src == dst) return fail(c, RLB_ERR_ARG, "src and dst must be distinct device buffers");
     if (!c->inited) return fail(c, RLB_ERR_STATE, "rlb_step_into_counted before rlb_init_fields");
-    if (c->g.variant < 0) c->g.variant = 7;  // untuned: the shape measured fastest on the benchmark lattices
     rlb_status s = after_launch(c,
                                 c->ph.eos ? launch_step_eos(c->g, c->ph, src, dst, c->cnt, true, c->steps, c->stream)
                                           : launch_step(c->p.prec, c->g, c->ph, src, dst, c->cnt, true, c->steps,

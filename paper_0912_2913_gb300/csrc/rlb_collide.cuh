@@ -23,12 +23,14 @@ namespace rlb {
 // fetch(q, i): the population of plane q (velocity i = q mod 19) pulled from
 // x - e_i, as stored (a solid neighbour yields the solid marker);
 // bounce(q, i): the cell's own population of the opposite velocity, the link
-// bounce-back value; put(q, v): store the post-collision value.
+// bounce-back value; put(q, v, old): store the post-collision value (old: the
+// gathered one).
 // A pulled marker is a NaN, so the sum of a phase's 19 values is NaN exactly
 // when a marker (or a non-finite population) is among them: the per-value
 // marker tests run only then.
+// Returns false when v[0], the cell's own population, is the marker.
 template <bool SOLID, class Fetch, class Bounce>
-__device__ __forceinline__ void gather_phase(float* v, int base, Fetch fetch, Bounce bounce) {
+__device__ __forceinline__ bool gather_phase(float* v, int base, Fetch fetch, Bounce bounce) {
 #pragma unroll
     for (int i = 0; i < 19; ++i) v[i] = fetch(base + i, i);
     if (SOLID) {
@@ -36,18 +38,21 @@ __device__ __forceinline__ void gather_phase(float* v, int base, Fetch fetch, Bo
 #pragma unroll
         for (int i = 1; i < 19; ++i) s += v[i];
         if (isnan(s)) {
+            if (is_solid(v[0])) return false;
 #pragma unroll
             for (int i = 1; i < 19; ++i)
                 if (is_solid(v[i])) v[i] = bounce(base + i, i);
         }
     }
+    return true;
 }
 
 // EARLYF: the f populations are loaded into registers before the g phase's
 // arithmetic, so that their loads are in flight during it (the same values,
 // the same arithmetic; more registers per thread).
+// Returns false, with nothing stored, for a solid cell.
 template <bool SOLID, class Fetch, class Bounce, class Put, bool EARLYF = false>
-__device__ __forceinline__ void collide_cell_f32(Fetch fetch, Bounce bounce, Put put, const Dev32& c, bool& unphys,
+__device__ __forceinline__ bool collide_cell_f32(Fetch fetch, Bounce bounce, Put put, const Dev32& c, bool& unphys,
                                                  bool& nonpos) {
     const float om = c.omega;
     // ---- phase 1: energy-momentum populations g_i (they alone fix eps, beta) ----
@@ -57,7 +62,7 @@ __device__ __forceinline__ void collide_cell_f32(Fetch fetch, Bounce bounce, Put
 #pragma unroll
         for (int i = 0; i < 19; ++i) f[i] = fetch(i, i);
     }
-    gather_phase<SOLID>(gg, 19, fetch, bounce);
+    if (!gather_phase<SOLID>(gg, 19, fetch, bounce)) return false;
     float dE = gg[0], d[9];
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
@@ -95,14 +100,14 @@ __device__ __forceinline__ void collide_cell_f32(Fetch fetch, Bounce bounce, Put
         const float k1 = (deps - 2.0f * eg * b2) * c.inv_cl2;
         const float k2 = 6.0f * eg * c.inv_cl2;
         const float k3 = 4.0f * eg * c.inv_cl;
-        put(19, fmaf(om, (float)kW0 * (deps * c.g0a + eg * b2 * c.g0b) - gg[0], gg[0]));
+        put(19, fmaf(om, (float)kW0 * (deps * c.g0a + eg * b2 * c.g0b) - gg[0], gg[0]), gg[0]);
 #pragma unroll
         for (int p = 0; p < 9; ++p) {
             const float w = (float)pair_w(p);
             const float gsym = w * fmaf(k2, qv[p] * qv[p], k1);
             const float gasy = w * k3 * qv[p];
-            put(20 + 2 * p, fmaf(om, (gsym + gasy) - gg[2 * p + 1], gg[2 * p + 1]));
-            put(21 + 2 * p, fmaf(om, (gsym - gasy) - gg[2 * p + 2], gg[2 * p + 2]));
+            put(20 + 2 * p, fmaf(om, (gsym + gasy) - gg[2 * p + 1], gg[2 * p + 1]), gg[2 * p + 1]);
+            put(21 + 2 * p, fmaf(om, (gsym - gasy) - gg[2 * p + 2], gg[2 * p + 2]), gg[2 * p + 2]);
         }
     }
     // ---- phase 2: number populations f_i ----
@@ -125,17 +130,18 @@ __device__ __forceinline__ void collide_cell_f32(Fetch fetch, Bounce bounce, Put
     for (int i = 1; i < 19; ++i) dS += f[i];
     const float sfull = c.n_ref + dS;
     const float fa = 3.0f * sfull * c.inv_cl;
-    put(0, fmaf(om, (float)kW0 * dS - f[0], f[0]));
+    put(0, fmaf(om, (float)kW0 * dS - f[0], f[0]), f[0]);
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
         const float w = (float)pair_w(p);
         const float fsym = w * dS;
         const float fasy = w * fa * qv[p];
-        put(2 * p + 1, fmaf(om, (fsym + fasy) - f[2 * p + 1], f[2 * p + 1]));
-        put(2 * p + 2, fmaf(om, (fsym - fasy) - f[2 * p + 2], f[2 * p + 2]));
+        put(2 * p + 1, fmaf(om, (fsym + fasy) - f[2 * p + 1], f[2 * p + 1]), f[2 * p + 1]);
+        put(2 * p + 2, fmaf(om, (fsym - fasy) - f[2 * p + 2], f[2 * p + 2]), f[2 * p + 2]);
     }
     unphys = !(pos_finite(sfull) && pos_finite(E) && nonneg_finite(d4) && pos_finite(eps) && below_one(b2));
     nonpos = nonpositive_eq(bx, by, bz, c.c_l);
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -166,12 +172,12 @@ __device__ __forceinline__ void collide_cell_f32(Fetch fetch, Bounce bounce, Put
 //     h_i + omega (eq_i - h_i) once more, when it is stored.
 // ---------------------------------------------------------------------------
 template <bool SOLID, class Fetch, class Bounce, class Put>
-__device__ __forceinline__ void collide_cell_f32c(Fetch fetch, Bounce bounce, Put put, const Dev32& c, bool& unphys,
+__device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Put put, const Dev32& c, bool& unphys,
                                                   bool& nonpos) {
     const float om = c.omega;
     // ---- phase 1: energy-momentum populations g_i ----
     float gg[19];
-    gather_phase<SOLID>(gg, 19, fetch, bounce);
+    if (!gather_phase<SOLID>(gg, 19, fetch, bounce)) return false;
     dfl dg[9];
     CSum esum(gg[0]);
 #pragma unroll
@@ -226,14 +232,14 @@ __device__ __forceinline__ void collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     {
         // g_0^eq - g_0^ref = w_0 [deps (3 - 2/c_l^2) + eg b2 (4 - 2/c_l^2)]   (Eq. equil2bs)
         const double g0 = (1.0 / 3.0) * fma(deps, 3.0 - 2.0 * c.inv_cl2_d, eg * b2 * (4.0 - 2.0 * c.inv_cl2_d));
-        put(19, __fmaf_rn(om, df_sub_round(df_of(g0), gg[0]), gg[0]));
+        put(19, __fmaf_rn(om, df_sub_round(df_of(g0), gg[0]), gg[0]), gg[0]);
 #pragma unroll
         for (int p = 0; p < 9; ++p) {
             const int cl = p < 3 ? 0 : 1;
             const dfl gsym = df_add(df_mul(K2[cl], df_mul(qv[p], qv[p])), K1[cl]);
             const dfl gasy = df_mul(A3[cl], ev[p]);
-            put(20 + 2 * p, __fmaf_rn(om, df_sub_round(df_add(gsym, gasy), gg[2 * p + 1]), gg[2 * p + 1]));
-            put(21 + 2 * p, __fmaf_rn(om, df_sub_round(df_add(gsym, df_neg(gasy)), gg[2 * p + 2]), gg[2 * p + 2]));
+            put(20 + 2 * p, __fmaf_rn(om, df_sub_round(df_add(gsym, gasy), gg[2 * p + 1]), gg[2 * p + 1]), gg[2 * p + 1]);
+            put(21 + 2 * p, __fmaf_rn(om, df_sub_round(df_add(gsym, df_neg(gasy)), gg[2 * p + 2]), gg[2 * p + 2]), gg[2 * p + 2]);
         }
     }
     // ---- phase 2: number populations f_i ----
@@ -248,16 +254,17 @@ __device__ __forceinline__ void collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     const dfl FS[2] = {df_of(dS * (1.0 / 18.0)), df_of(dS * (1.0 / 36.0))};
     const double fa = 3.0 * S * c.inv_cl_d;
     const dfl FA[2] = {df_of(fa * (1.0 / 18.0)), df_of(fa * (1.0 / 36.0))};
-    put(0, __fmaf_rn(om, df_sub_round(df_of(dS * (1.0 / 3.0)), f[0]), f[0]));
+    put(0, __fmaf_rn(om, df_sub_round(df_of(dS * (1.0 / 3.0)), f[0]), f[0]), f[0]);
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
         const int cl = p < 3 ? 0 : 1;
         const dfl fasy = df_mul(FA[cl], qv[p]);
-        put(2 * p + 1, __fmaf_rn(om, df_sub_round(df_add(FS[cl], fasy), f[2 * p + 1]), f[2 * p + 1]));
-        put(2 * p + 2, __fmaf_rn(om, df_sub_round(df_add(FS[cl], df_neg(fasy)), f[2 * p + 2]), f[2 * p + 2]));
+        put(2 * p + 1, __fmaf_rn(om, df_sub_round(df_add(FS[cl], fasy), f[2 * p + 1]), f[2 * p + 1]), f[2 * p + 1]);
+        put(2 * p + 2, __fmaf_rn(om, df_sub_round(df_add(FS[cl], df_neg(fasy)), f[2 * p + 2]), f[2 * p + 2]), f[2 * p + 2]);
     }
     unphys = !(pos_finite(S) && pos_finite(E) && nonneg_finite(d4) && pos_finite(eps) && below_one(b2));
     nonpos = nonpositive_eq(d2f(bx), d2f(by), d2f(bz), c.c_l);
+    return true;
 }
 
 }  // namespace rlb

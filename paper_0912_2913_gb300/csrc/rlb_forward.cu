@@ -51,8 +51,8 @@ void set_last_launch_count(int n) { g_last_launches = n; }
 // runs (the default launch: the f loads then hit L2 instead of waiting on
 // HBM, measured +16% on the 200x100x100 sphere).
 // I: type of the element offsets, int when 38 S < 2^31 (fewer address
-// instructions: measured +2 % / +6 % for the two shapes the first step picks
-// from on the 200x100x100 sphere), else long long.
+// instructions: measured +2 % / +6 % for two of the shapes on the
+// 200x100x100 sphere), else long long.
 // COMP: the compensated collision (collide_cell_f32c), run for c_l > 1.
 // EARLY: the f populations are loaded before the g phase's arithmetic.
 // TB: threads per block the register budget is cut for.
@@ -76,19 +76,19 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
     const long long lim = (SPLIT ? 19ll : 38ll) * g.S;  // extent the checked builds test against
     auto pq = [](int q) { return (SPLIT && q >= 19) ? q - 19 : q; };  // plane number within its base
     auto abase = [&](int q) { return (SPLIT && q >= 19) ? Ag : A; };
-    if (XBC != XBC_PERIODIC && (x == 0 || x == g.nx - 1)) {
-        if (XBC == XBC_INFLOW_OUTFLOW && x == 0) {
-#pragma unroll
-            for (int q = 0; q < 38; ++q)
-                ((SPLIT && q >= 19) ? Bg : B)[RLB_CHK(pq(q) * S + idx, lim)] = __ldg(RLB_CHK_PTR(abase(q), pq(q) * S + idx, lim));
-        }
-        return;
-    }
-    const PullOffsets o(g, x, y, z);
+    // The inflow column keeps its populations: its lanes load them through
+    // offsets of zero and store them as loaded, along with their warp (a copy
+    // loop of its own was a second pass over memory for every warp that holds
+    // such a cell: all warps of a lattice 63 cells wide).
+    const bool keep = XBC == XBC_INFLOW_OUTFLOW && x == 0;
+    if (XBC != XBC_PERIODIC && (x == g.nx - 1 || (x == 0 && !keep))) return;
+    PullOffsets o(g, x, y, z);
+    if (keep) o.xm = o.xp = o.ym = o.yp = o.zm = o.zp = 0;
     const int dup = (XBC != XBC_PERIODIC && x == g.nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
     float* Bc = B + idx;
     float* Bgc = Bg + idx;
-    auto put = [&](int q, float v) {
+    auto put = [&](int q, float v, float old) {
+        if (XBC == XBC_INFLOW_OUTFLOW && keep) v = old;
         if constexpr (SPLIT) {
             float* b = q >= 19 ? Bgc : Bc;
             b[RLB_CHK_OFF(pq(q) * S, idx, lim)] = v;
@@ -100,12 +100,6 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
             if (dup) Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
         }
     };
-    if (SOLID && is_solid(__ldg(RLB_CHK_PTR(abase(19), pq(19) * S + idx, lim)))) {  // the cell itself is solid: keep the marker
-        const float m = solid_marker_f();
-#pragma unroll
-        for (int q = 0; q < 38; ++q) ((SPLIT && q >= 19) ? Bgc : Bc)[RLB_CHK_OFF(pq(q) * S, idx, lim)] = m;
-        return;
-    }
     if (PREF) {
 #pragma unroll
         for (int i = 0; i < 19; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(RLB_CHK_PTR(A, i * S + idx + o.src(i), lim)));
@@ -122,13 +116,19 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
         else
             return __ldg(RLB_CHK_PTR(A, (q - i + opp(i)) * S + idx, 38ll * S));
     };
-    bool unphys, nonpos;
+    bool unphys, nonpos, fluid;
     if (COMP)
-        collide_cell_f32c<SOLID>(fetch, bounce, put, c, unphys, nonpos);
+        fluid = collide_cell_f32c<SOLID>(fetch, bounce, put, c, unphys, nonpos);
     else
-        collide_cell_f32<SOLID, decltype(fetch), decltype(bounce), decltype(put), EARLY>(fetch, bounce, put, c, unphys,
-                                                                                        nonpos);
-    if (count) count_flags(cnt, unphys, nonpos, (unsigned long long)step_index * (unsigned long long)g.N + idx);
+        fluid = collide_cell_f32<SOLID, decltype(fetch), decltype(bounce), decltype(put), EARLY>(fetch, bounce, put, c,
+                                                                                                unphys, nonpos);
+    if (!fluid) {  // keep the marker (found among the gathered values: a load of it before them is a round trip more)
+        const float m = solid_marker_f();
+#pragma unroll
+        for (int q = 0; q < 38; ++q) ((SPLIT && q >= 19) ? Bgc : Bc)[RLB_CHK_OFF(pq(q) * S, idx, lim)] = m;
+        return;
+    }
+    if (count && !keep) count_flags(cnt, unphys, nonpos, (unsigned long long)step_index * (unsigned long long)g.N + idx);
 }
 
 // Persistent variant: a grid of (SMs x resident blocks) threads walks the
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256, 3) k_step_f32_pipe(const float* __restric
         const PullOffsets o(g, x, y, z);
         const int dup = (XBC != XBC_PERIODIC && x == g.nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
         float* Bc = B + idx;
-        auto put = [&](int q, float v) {
+        auto put = [&](int q, float v, float) {
             if (CS) {
                 __stcs(Bc + q * S, v);
                 if (dup) __stcs(Bc + q * S + dup, v);
@@ -302,6 +302,20 @@ static int sm_count() {
 // FP64 above all, is then the step's latency).  Results do not depend on it.
 static int step_block(long long N, int full) { return blocks_for(N, full) < (unsigned)sm_count() ? 32 : full; }
 
+// Launch shape of the FP32 step (all give the same bits).  8, f loaded before
+// the g arithmetic in 64-thread blocks x 12 per SM, is the fastest or within
+// 3 % of it from 1600 cells to 512^3 (us a step, shapes 2 / 7 / 8: 47x33x33
+// 5.7 / 4.4 / 4.2; 200x100x100 sphere 102.5 / 93.6 / 91.5; 256^3 844 / 750 /
+// 739; 512^3 6740 / 5982 / 5880), except where the lattice gives every
+// scheduler three to four warps: there two 256-thread blocks spread the warps
+// evenly over an SM's schedulers (63x41x29: 5.8 / 6.9 / 6.3), just below it
+// (48x35x35: 5.8 / 5.0 / 6.2) and just above (64x40x40: 8.8 / 7.0 / 6.6) they
+// lose or gain little.
+static int f32_shape(long long N) {
+    const long long per = 128ll * sm_count();  // one warp on each scheduler
+    return N > 3 * per && N <= 4 * per ? 2 : 8;
+}
+
 template <int XBC, bool SOLID>
 static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A, void* B, Counters cnt, bool count,
                           long long step_index, cudaStream_t st) {
@@ -334,7 +348,8 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
         if (g.tma && launch_step_f32_tma(g, c, (const float*)A, (float*)B, cnt, count, step_index, st) == cudaSuccess)
             return;
         cudaGetLastError();
-        switch (g.variant) {
+        const int variant = g.variant < 0 ? f32_shape(g.N) : g.variant;
+        switch (variant) {
             case 0: launch_dependent(k_step_f32<XBC, SOLID, 3, false>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index); break;
             case 1:
                 if (idx32)
@@ -363,7 +378,7 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
                 // 80 registers)
                 const float* a = (const float*)A;
                 float* b = (float*)B;
-                const int v = g.variant;
+                const int v = variant;
                 const int t = v == 8 ? (tb < 64 ? tb : 64) : (tb < 128 ? tb : 128);
                 const unsigned n = blocks_for(g.N, t);
 #define RLB_EARLY_LAUNCH(MB, TBK)                                                                                        \
@@ -382,7 +397,7 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
             case 5: {
                 unsigned grid = (unsigned)sm_count() * (unsigned)(g.pipe_blocks > 0 ? g.pipe_blocks : 3);
                 if (grid > nb) grid = nb;
-                if (g.variant == 4)
+                if (variant == 4)
                     k_step_f32_pipe<XBC, SOLID, false><<<grid, 256, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);
                 else
                     k_step_f32_pipe<XBC, SOLID, true><<<grid, 256, 0, st>>>((const float*)A, (float*)B, g, c, cnt, cs, step_index);

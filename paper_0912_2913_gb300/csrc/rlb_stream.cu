@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256, MINB)
             auto bounce = [&](int q, int i) { return __ldg(RLB_CHK_PTR(A, (q - i + opp(i)) * S + idx, 38ll * S)); };  // link bounce-back
             const int dup = (XBC != XBC_PERIODIC && x == nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
             float* Bc = B + idx;
-            auto put = [&](int q, float v) {
+            auto put = [&](int q, float v, float) {
                 Bc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v;
                 if (dup) Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
             };
