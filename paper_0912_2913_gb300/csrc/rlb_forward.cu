@@ -111,10 +111,11 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
             return __ldg(RLB_CHK_PTR(A, q * S + idx + o.src(i), 38ll * S));
     };
     auto bounce = [&](int q, int i) {  // link bounce-back
+        const int r = XBC == XBC_INFLOW_OUTFLOW && keep ? q : q - i + opp(i);
         if constexpr (SPLIT)
-            return __ldg(RLB_CHK_PTR(abase(q), (pq(q) - i + opp(i)) * S + idx, lim));
+            return __ldg(RLB_CHK_PTR(abase(q), pq(r) * S + idx, lim));
         else
-            return __ldg(RLB_CHK_PTR(A, (q - i + opp(i)) * S + idx, 38ll * S));
+            return __ldg(RLB_CHK_PTR(A, r * S + idx, 38ll * S));
     };
     bool unphys, nonpos, fluid;
     if (COMP)

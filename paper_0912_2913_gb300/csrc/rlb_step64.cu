@@ -426,14 +426,12 @@ __global__ void __launch_bounds__(128, MINB)
     if (g.zhalo && (z == 0 || z == g.nz - 1)) return;  // z halo planes: filled by the exchange
     const long long S = g.S;
     auto pa = [&](int q, int off) { return __ldg(RLB_CHK_PTR(tab.a[q], (unsigned)off, S)); };
-    if (XBC != XBC_PERIODIC && (x == 0 || x == g.nx - 1)) {
-        if (XBC == XBC_INFLOW_OUTFLOW && x == 0) {
-#pragma unroll
-            for (int q = 0; q < 38; ++q) tab.b[q][RLB_CHK((unsigned)idx, S)] = pa(q, idx);
-        }
-        return;
-    }
-    const PullOffsets o(g, x, y, z);
+    // the inflow column keeps its populations: loaded with the warp's others,
+    // through offsets of zero, and stored as loaded
+    const bool keep = XBC == XBC_INFLOW_OUTFLOW && x == 0;
+    if (XBC != XBC_PERIODIC && (x == g.nx - 1 || (x == 0 && !keep))) return;
+    PullOffsets o(g, x, y, z);
+    if (keep) o.xm = o.xp = o.ym = o.yp = o.zm = o.zp = 0;
     const FxRun& k = ph.fx;
     double h[19];
 #pragma unroll
@@ -451,7 +449,7 @@ __global__ void __launch_bounds__(128, MINB)
         for (int i = 1; i < 19; ++i) {
             if (is_solid(h[i])) {  // link bounce-back
                 bounced |= 1u << i;
-                h[i] = pa(19 + opp(i), idx);
+                h[i] = pa(19 + (XBC == XBC_INFLOW_OUTFLOW && keep ? i : opp(i)), idx);
             }
         }
         em = fx_max_exponent<19>(h);
@@ -479,7 +477,11 @@ __global__ void __launch_bounds__(128, MINB)
                         ((d[2] + d[5]) - d[6]) + (d[7] - d[8]), em, k, t, u, rD);
         if (ok) nonpos = fx_nonpositive(t, u, rD, k);
     }
-    if (ok) {
+    if (XBC == XBC_INFLOW_OUTFLOW && keep) {
+        ok = true, nonpos = false;
+#pragma unroll
+        for (int i = 0; i < 19; ++i) tab.b[19 + i][RLB_CHK((unsigned)idx, S)] = h[i];
+    } else if (ok) {
         put(19, fma(k.omw, h[0], fx_to(t.g0, t.eb + 3)));
 #pragma unroll
         for (int p = 0; p < 9; ++p) {
@@ -488,13 +490,15 @@ __global__ void __launch_bounds__(128, MINB)
             put(20 + 2 * p, fma(k.omw, h[2 * p + 1], fx_to(s + a, t.eb)));
             put(21 + 2 * p, fma(k.omw, h[2 * p + 2], fx_to(s - a, t.eb)));
         }
+    }
+    if (ok) {
         // ---- number populations f_i
 #pragma unroll
         for (int i = 0; i < 19; ++i) h[i] = pa(i, idx + o.src(i));
         if (bounced) {
 #pragma unroll
             for (int i = 1; i < 19; ++i)
-                if ((bounced >> i) & 1u) h[i] = pa(opp(i), idx);
+                if ((bounced >> i) & 1u) h[i] = pa(XBC == XBC_INFLOW_OUTFLOW && keep ? i : opp(i), idx);
         }
         const int ef = fx_max_exponent<19>(h);
         int64_t sum = fx_round4(fx_from(h[0], ef));
@@ -502,7 +506,11 @@ __global__ void __launch_bounds__(128, MINB)
         for (int p = 0; p < 9; ++p) sum += fx_round4(fx_from(h[2 * p + 1], ef) + fx_from(h[2 * p + 2], ef));
         FxF q;
         ok = fx_f_terms(sum, ef, t, k, q);
-        if (ok) {
+        if (XBC == XBC_INFLOW_OUTFLOW && keep) {
+            ok = true;
+#pragma unroll
+            for (int i = 0; i < 19; ++i) tab.b[i][RLB_CHK((unsigned)idx, S)] = h[i];
+        } else if (ok) {
             put(0, fma(k.omw, h[0], fx_to((q.B << 3) + (q.B << 2), q.eb)));
 #pragma unroll
             for (int p = 0; p < 9; ++p) {

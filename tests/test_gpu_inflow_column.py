@@ -48,3 +48,33 @@ def test_inflow_column_and_markers_keep_their_bits(shape, c_l, monkeypatch):
         _, ref, _, _, st_ref = one("4")
         assert torch.equal(b[:, :N], ref[:, :N])
         assert (st["n_unphysical"], st["n_nonpositive_eq"]) == (st_ref["n_unphysical"], st_ref["n_nonpositive_eq"])
+
+
+@pytest.mark.parametrize("eos", ["ultra", "gamma_law"])
+@pytest.mark.parametrize("shape", [(3, 1, 1), (33, 5, 4), (64, 40, 40)], ids=str)
+def test_inflow_column_keeps_its_bits_fp64(shape, eos):
+    from paper_0912_2913_gb300 import RLB
+
+    nx, ny, nz = shape
+    rng = np.random.default_rng(6)
+    n = 1.0 + 0.05 * rng.random((nz, ny, nx))
+    beta = 0.02 * rng.random((3, nz, ny, nx))
+    kw = dict(eos="gamma_law", eos_gamma=1.25, eos_mass=0.1) if eos == "gamma_law" else {}
+    with RLB(nx, ny, nz, 0.8, precision="fp64", xbc="inflow_outflow", beta_in=(0.1, 0.0, 0.0), device="cuda:0",
+             **kw) as sim:
+        sim.init_fields(n, n, beta, None)
+        a, b = sim.state().clone(), sim.new_state()
+        b.fill_(3.0)
+        bits, col = a.view(torch.int64), torch.arange(0, sim.N, nx, device=a.device)
+        if nx > 3:
+            for k, v in ((7, 0x7FF0000000000000), (8, 0x7FF8000012345678), (9, -2 ** 63), (15, 0)):
+                bits[k + 3, col[k]] = v
+        sim.step_into(a, b, counted=True)
+        assert torch.equal(bits[:, col], b.view(torch.int64)[:, col])
+        if nx <= 3:
+            return
+        # away from the column's unusual cells the step is the one of the plain column
+        c, d = sim.state().clone(), sim.new_state()
+        sim.step_into(c, d)
+        inner = torch.arange(sim.N, device=a.device) % nx > 1
+        assert torch.equal(b[:, :sim.N][:, inner], d[:, :sim.N][:, inner])
