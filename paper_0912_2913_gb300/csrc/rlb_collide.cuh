@@ -218,9 +218,11 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     const double deps = eps - c.eps_ref;
     // g^eq_i - g^ref_i = w_i [k1 + k2 q_i^2] +- 3 w_i (e_i . M)/c_l,
     //   k1 = (deps - 2 eg b2)/c_l^2, k2 = 6 eg / c_l^2 (per weight class)
-    const double k1 = (deps - 2.0 * eg * b2) * c.inv_cl2_d, k2 = 6.0 * eg * c.inv_cl2_d;
-    const dfl K1[2] = {df_of(k1 * (1.0 / 18.0)), df_of(k1 * (1.0 / 36.0))};
-    const dfl K2[2] = {df_of(k2 * (1.0 / 18.0)), df_of(k2 * (1.0 / 36.0))};
+    // (the binary64 1/36 is half of the binary64 1/18: so are the products)
+    const double eb2 = eg * b2;
+    const double k1 = fma(-2.0, eb2, deps) * c.inv_cl2_d, k2 = 6.0 * eg * c.inv_cl2_d;
+    const dfl K1a = df_of(k1 * (1.0 / 18.0)), K2a = df_of(k2 * (1.0 / 18.0));
+    const dfl K1[2] = {K1a, df_half(K1a)}, K2[2] = {K2a, df_half(K2a)};
     // 3 w_p as pairs: 1/6 and 1/12
     const dfl A3[2] = {{(float)(1.0 / 6.0), (float)(1.0 / 6.0 - (double)(float)(1.0 / 6.0))},
                        {(float)(1.0 / 12.0), (float)(1.0 / 12.0 - (double)(float)(1.0 / 12.0))}};
@@ -231,7 +233,7 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
                        df_add(Dy, Dz), df_add(Dy, df_neg(Dz))};
     {
         // g_0^eq - g_0^ref = w_0 [deps (3 - 2/c_l^2) + eg b2 (4 - 2/c_l^2)]   (Eq. equil2bs)
-        const double g0 = (1.0 / 3.0) * fma(deps, 3.0 - 2.0 * c.inv_cl2_d, eg * b2 * (4.0 - 2.0 * c.inv_cl2_d));
+        const double g0 = (1.0 / 3.0) * fma(deps, c.g0a_d, eb2 * c.g0b_d);
         put(19, __fmaf_rn(om, df_sub_round(df_of(g0), gg[0]), gg[0]), gg[0]);
 #pragma unroll
         for (int p = 0; p < 9; ++p) {
@@ -251,9 +253,9 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     const double dS = df_dbl(ssum.result());
     const double S = c.n_ref_d + dS;
     // f^eq_i - f^ref_i = w_i dS +- w_i 3 S q_i / c_l   (Eq. equil1s, n gamma = S)
-    const dfl FS[2] = {df_of(dS * (1.0 / 18.0)), df_of(dS * (1.0 / 36.0))};
     const double fa = 3.0 * S * c.inv_cl_d;
-    const dfl FA[2] = {df_of(fa * (1.0 / 18.0)), df_of(fa * (1.0 / 36.0))};
+    const dfl FSa = df_of(dS * (1.0 / 18.0)), FAa = df_of(fa * (1.0 / 18.0));
+    const dfl FS[2] = {FSa, df_half(FSa)}, FA[2] = {FAa, df_half(FAa)};
     put(0, __fmaf_rn(om, df_sub_round(df_of(dS * (1.0 / 3.0)), f[0]), f[0]), f[0]);
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
@@ -263,7 +265,7 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
         put(2 * p + 2, __fmaf_rn(om, df_sub_round(df_add(FS[cl], df_neg(fasy)), f[2 * p + 2]), f[2 * p + 2]), f[2 * p + 2]);
     }
     unphys = !(pos_finite(S) && pos_finite(E) && nonneg_finite(d4) && pos_finite(eps) && below_one(b2));
-    nonpos = nonpositive_eq(d2f(bx), d2f(by), d2f(bz), c.c_l);
+    nonpos = nonpositive_eq(Bx.h, By.h, Bz.h, c.c_l);
     return true;
 }
 

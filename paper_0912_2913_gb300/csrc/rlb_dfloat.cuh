@@ -57,13 +57,6 @@ __device__ __forceinline__ dfl df_mul(dfl x, dfl y) {
     return fast_two_sum(p.h, e);
 }
 
-// Split of a binary64 value: h = x rounded to binary32, l = (x - h) rounded
-// (the conversions on the integer pipe, one FP64 subtraction).
-__device__ __forceinline__ dfl df_of(double x) {
-    const float h = d2f(x);
-    return {h, d2f(x - f2d(h))};
-}
-
 // Split of a binary64 value into a pair on the integer pipe (no FP64
 // instruction): h = x rounded to binary32 (d2f), and the remainder x - h,
 // exact in binary64 as the signed integer R of the 29 mantissa bits below
@@ -86,6 +79,16 @@ __device__ __forceinline__ dfl df_split(double x) {
     const float l = (R == 0 || eb <= 0) ? 0.0f : __uint_as_float(scaled);
     return {h, l};
 }
+
+// As df_split for any x: l = NaN where h overflows (as x - h would be).
+__device__ __forceinline__ dfl df_of(double x) {
+    dfl r = df_split(x);
+    if (isinf(r.h)) r.l = __int_as_float(0x7FFFFFFF);
+    return r;
+}
+
+// half of a pair (exact above the subnormals)
+__device__ __forceinline__ dfl df_half(dfl x) { return {0.5f * x.h, 0.5f * x.l}; }
 
 // h + l in binary64 (exact for a normalised pair).
 __device__ __forceinline__ double df_dbl(dfl x) { return f2d(x.h) + f2d(x.l); }

@@ -284,6 +284,8 @@ Dev32 make_dev32(const Phys& ph) {
     c.c_l_d = ph.c_l;
     c.inv_cl_d = ph.inv_cl;
     c.inv_cl2_d = ph.inv_cl2;
+    c.g0a_d = 3.0 - 2.0 * ph.inv_cl2;
+    c.g0b_d = 4.0 - 2.0 * ph.inv_cl2;
     return c;
 }
 

@@ -72,7 +72,7 @@ struct Dev32 {
     float omega, omw, c_l, inv_cl, inv_cl2, n_ref;
     float g0a, g0b;  // 3 - 2/c_l^2 and 4 - 2/c_l^2
     double eps_ref;
-    double n_ref_d, c_l_d, inv_cl_d, inv_cl2_d;  // binary64 copies (compensated collision)
+    double n_ref_d, c_l_d, inv_cl_d, inv_cl2_d, g0a_d, g0b_d;  // binary64 copies (compensated collision)
 };
 
 // Device-side statistics of a run (see rlb_stats).
