@@ -948,20 +948,6 @@ __global__ void __launch_bounds__(128, MINB)
 // Error against 113-bit references: nu 1.2e-16 (2 to 3e-16 before), the terms
 // of dL/dtau 7.4e-17 rms and below 3e-17 in the mean (1.5e-16 and 7e-17).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async4(uint32_t saddr, const void* gptr) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(gptr) : "memory");
-}
-__device__ __forceinline__ void cp_async8(uint32_t saddr, const void* gptr) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(saddr), "l"(gptr) : "memory");
-}
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gptr) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 struct AdjFx {
     FxConst kS1;  // 5 / 3                        x 2^62

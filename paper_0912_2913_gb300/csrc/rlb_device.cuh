@@ -52,6 +52,22 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigne
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// Per-thread asynchronous copies to shared memory.
+__device__ __forceinline__ void cp_async4(uint32_t saddr, const void* gptr) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(saddr), "l"(gptr) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t saddr, const void* gptr) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(saddr), "l"(gptr) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gptr) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // e_p of the nine pairs: +x, +y, +z, (1,1,0), (1,-1,0), (1,0,1), (1,0,-1), (0,1,1), (0,1,-1).
 __host__ __device__ constexpr int pair_ex(int p) { return (p == 0 || (p >= 3 && p <= 6)) ? 1 : 0; }
 __host__ __device__ constexpr int pair_ey(int p) {

@@ -370,9 +370,9 @@ __global__ void __launch_bounds__(128) k_step_f64_split(const double* __restrict
 // h + omega (eq - h)) beside 2,846 instructions in all, 1,401 of them on the
 // ALU pipe at two clocks each: the two pipes are loaded alike, and a warp's
 // integer and FP64 phases overlap with those of the others.  256^3 box 6.07 ->
-// 2.27 ms, 200x100x100 sphere 0.740 -> 0.333 ms per step.  Resident blocks of
-// 128 threads: 4, 5 and 6 measure alike (2.25, 2.27, 2.32 ms), 3 and 8 (which
-// spills) 2.60 and 2.73 ms.
+// 2.09 ms, 200x100x100 sphere 0.740 -> 0.285 ms per step.  Resident blocks of
+// 128 threads: 4, 5 and 6 measure 2.20, 2.09 and 2.33 ms (0.291, 0.285 and
+// 0.316 for the sphere).
 //
 // Lattice speed: all 19 populations of g share one exponent and the rest
 // population is 9 c_l^2 times the moving ones, so with c_l they lose low bits;
@@ -436,6 +436,16 @@ __global__ void __launch_bounds__(128, MINB)
     double h[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) h[i] = pa(19 + i, idx + o.src(i));
+    // the f populations on their way to shared memory during the g phase, each
+    // thread's into its own slots: loads after that phase were a third of the
+    // stall cycles, and registers for them would cost two of the five blocks
+    // (256^3: 2.34 -> 2.09 ms; 200x100x100 sphere: 300 -> 285 us)
+    __shared__ double staged[19][128];
+    const uint32_t slot = (uint32_t)__cvta_generic_to_shared(&staged[0][threadIdx.x]);
+#pragma unroll
+    for (int i = 0; i < 19; ++i)
+        cp_async8(slot + (uint32_t)(i * 128 * 8), RLB_CHK_PTR(tab.a[i], (unsigned)(idx + o.src(i)), S));
+    cp_async_commit();
     int em = fx_max_exponent<19>(h);
     unsigned bounced = 0u;
     if (em == 0x7FF) {  // a solid marker among them, or a non-finite population
@@ -443,6 +453,7 @@ __global__ void __launch_bounds__(128, MINB)
             const double m = solid_marker_d();
 #pragma unroll
             for (int q = 0; q < 38; ++q) tab.b[q][RLB_CHK((unsigned)idx, S)] = m;
+            cp_async_wait<0>();
             return;
         }
 #pragma unroll
@@ -491,10 +502,11 @@ __global__ void __launch_bounds__(128, MINB)
             put(21 + 2 * p, fma(k.omw, h[2 * p + 2], fx_to(s - a, t.eb)));
         }
     }
+    cp_async_wait<0>();
     if (ok) {
         // ---- number populations f_i
 #pragma unroll
-        for (int i = 0; i < 19; ++i) h[i] = pa(i, idx + o.src(i));
+        for (int i = 0; i < 19; ++i) h[i] = staged[i][threadIdx.x];
         if (bounced) {
 #pragma unroll
             for (int i = 1; i < 19; ++i)
