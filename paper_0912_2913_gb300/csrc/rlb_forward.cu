@@ -336,16 +336,19 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
         const bool split32 = !idx32 && 19 * g.S < (1ll << 32);  // unsigned offsets per population set
         if (ph.c_l > 1.0) {
             // lattice speeds above 1: the compensated collision (one launch
-            // shape; the TMA-staged and tuning variants use the binary32 one)
+            // shape; the TMA-staged and tuning variants use the binary32 one).
+            // 128 threads x 5 per SM; 193x127x161, us a step: 256 x 2 614,
+            // 128 x 5 561, 128 x 6 566, 64 x 12 568, 128 x 7 585
+            const int t = tb < 128 ? tb : 128;
+            const unsigned n = blocks_for(g.N, t);
+            const float* a = (const float*)A;
+            float* b = (float*)B;
             if (idx32)
-                launch_dependent(k_step_f32<XBC, SOLID, 2, false, int, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt, cs,
-                                                                                 step_index);
+                launch_dependent(k_step_f32<XBC, SOLID, 5, false, int, true, false, 128>, n, t, 0, st, a, b, g, c, cnt, cs, step_index);
             else if (split32)
-                launch_dependent(k_step_f32<XBC, SOLID, 2, false, unsigned, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c, cnt,
-                                                                                      cs, step_index);
+                launch_dependent(k_step_f32<XBC, SOLID, 5, false, unsigned, true, false, 128>, n, t, 0, st, a, b, g, c, cnt, cs, step_index);
             else
-                launch_dependent(k_step_f32<XBC, SOLID, 2, false, long long, true>, nb, tb, 0, st, (const float*)A, (float*)B, g, c,
-                                                                                       cnt, cs, step_index);
+                launch_dependent(k_step_f32<XBC, SOLID, 5, false, long long, true, false, 128>, n, t, 0, st, a, b, g, c, cnt, cs, step_index);
             return;
         }
         if (g.tma && launch_step_f32_tma(g, c, (const float*)A, (float*)B, cnt, count, step_index, st) == cudaSuccess)

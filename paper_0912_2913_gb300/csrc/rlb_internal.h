@@ -130,7 +130,7 @@ cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const v
                                 double* dbeta_in, cudaStream_t stream);
 // Allocation-free variant of launch_adjoint_step (same kernels, persistent
 // grid): partial sums in a static device array of kAdjScratchDoubles doubles,
-// set up once per device on first use.  Needs 16 doubles per block of the
+// set up once per device on first use.  Needs 4 doubles per warp of the
 // grid (reported in *need_doubles); returns cudaErrorInvalidValue, launching
 // nothing, when that exceeds the array.
 constexpr long long kAdjScratchDoubles = 32768;  // 256 KiB
