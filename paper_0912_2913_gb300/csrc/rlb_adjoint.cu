@@ -942,7 +942,7 @@ __global__ void __launch_bounds__(128, MINB)
 // are staged in a shared-memory column per thread by asynchronous copies, so
 // that they hold no registers, and the velocity pairs are walked in three
 // rounds by one loop body (a third of the code to fetch).  200x100x100 sphere
-// 1.51 -> 0.85 ms, 192^3 box 5.1 -> 2.35 ms; blocks of 64 threads: 5, 6 and 7
+// 1.51 -> 0.83 ms, 192^3 box 5.1 -> 2.35 ms; blocks of 64 threads: 5, 6 and 7
 // per SM 2.65, 2.35 and 2.49 ms; all values in registers and unrolled, 3
 // blocks of 128: 2.35 ms on the box, 0.854 on the sphere.
 // Error against 113-bit references: nu 1.2e-16 (2 to 3e-16 before), the terms

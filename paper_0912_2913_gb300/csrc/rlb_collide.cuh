@@ -221,12 +221,12 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     // (the binary64 1/36 is half of the binary64 1/18: so are the products)
     const double eb2 = eg * b2;
     const double k1 = fma(-2.0, eb2, deps) * c.inv_cl2_d, k2 = 6.0 * eg * c.inv_cl2_d;
-    const dfl K1a = df_of(k1 * (1.0 / 18.0)), K2a = df_of(k2 * (1.0 / 18.0));
+    const dfl K1a = df_of_alu(k1 * (1.0 / 18.0)), K2a = df_of_alu(k2 * (1.0 / 18.0));
     const dfl K1[2] = {K1a, df_half(K1a)}, K2[2] = {K2a, df_half(K2a)};
     // 3 w_p as pairs: 1/6 and 1/12
     const dfl A3[2] = {{(float)(1.0 / 6.0), (float)(1.0 / 6.0 - (double)(float)(1.0 / 6.0))},
                        {(float)(1.0 / 12.0), (float)(1.0 / 12.0 - (double)(float)(1.0 / 12.0))}};
-    const dfl Bx = df_of(bx), By = df_of(by), Bz = df_of(bz);
+    const dfl Bx = df_of_alu(bx), By = df_of_alu(by), Bz = df_of_alu(bz);
     const dfl qv[9] = {Bx, By, Bz, df_add(Bx, By), df_add(Bx, df_neg(By)), df_add(Bx, Bz), df_add(Bx, df_neg(Bz)),
                        df_add(By, Bz), df_add(By, df_neg(Bz))};
     const dfl ev[9] = {Dx, Dy, Dz, df_add(Dx, Dy), df_add(Dx, df_neg(Dy)), df_add(Dx, Dz), df_add(Dx, df_neg(Dz)),
@@ -234,7 +234,7 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     {
         // g_0^eq - g_0^ref = w_0 [deps (3 - 2/c_l^2) + eg b2 (4 - 2/c_l^2)]   (Eq. equil2bs)
         const double g0 = (1.0 / 3.0) * fma(deps, c.g0a_d, eb2 * c.g0b_d);
-        put(19, __fmaf_rn(om, df_sub_round(df_of(g0), gg[0]), gg[0]), gg[0]);
+        put(19, __fmaf_rn(om, df_sub_round(df_of_alu(g0), gg[0]), gg[0]), gg[0]);
 #pragma unroll
         for (int p = 0; p < 9; ++p) {
             const int cl = p < 3 ? 0 : 1;
@@ -254,9 +254,9 @@ __device__ __forceinline__ bool collide_cell_f32c(Fetch fetch, Bounce bounce, Pu
     const double S = c.n_ref_d + dS;
     // f^eq_i - f^ref_i = w_i dS +- w_i 3 S q_i / c_l   (Eq. equil1s, n gamma = S)
     const double fa = 3.0 * S * c.inv_cl_d;
-    const dfl FSa = df_of(dS * (1.0 / 18.0)), FAa = df_of(fa * (1.0 / 18.0));
+    const dfl FSa = df_of_alu(dS * (1.0 / 18.0)), FAa = df_of_alu(fa * (1.0 / 18.0));
     const dfl FS[2] = {FSa, df_half(FSa)}, FA[2] = {FAa, df_half(FAa)};
-    put(0, __fmaf_rn(om, df_sub_round(df_of(dS * (1.0 / 3.0)), f[0]), f[0]), f[0]);
+    put(0, __fmaf_rn(om, df_sub_round(df_of_alu(dS * (1.0 / 3.0)), f[0]), f[0]), f[0]);
 #pragma unroll
     for (int p = 0; p < 9; ++p) {
         const int cl = p < 3 ? 0 : 1;

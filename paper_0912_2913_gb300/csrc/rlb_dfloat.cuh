@@ -57,6 +57,13 @@ __device__ __forceinline__ dfl df_mul(dfl x, dfl y) {
     return fast_two_sum(p.h, e);
 }
 
+// Split of a binary64 value: h = x rounded to binary32, l = (x - h) rounded
+// (the conversions on the integer pipe, one FP64 subtraction).
+__device__ __forceinline__ dfl df_of(double x) {
+    const float h = d2f(x);
+    return {h, d2f(x - f2d(h))};
+}
+
 // Split of a binary64 value into a pair on the integer pipe (no FP64
 // instruction): h = x rounded to binary32 (d2f), and the remainder x - h,
 // exact in binary64 as the signed integer R of the 29 mantissa bits below
@@ -80,8 +87,11 @@ __device__ __forceinline__ dfl df_split(double x) {
     return {h, l};
 }
 
-// As df_split for any x: l = NaN where h overflows (as x - h would be).
-__device__ __forceinline__ dfl df_of(double x) {
+// df_of without an FP64 instruction: l = NaN where h overflows (as x - h
+// would be).  For kernels whose FP64 pipe is the busy one; in the
+// pair-arithmetic FP64 step, which is bound by its integer and binary32
+// work, it cost 3 %.
+__device__ __forceinline__ dfl df_of_alu(double x) {
     dfl r = df_split(x);
     if (isinf(r.h)) r.l = __int_as_float(0x7FFFFFFF);
     return r;

@@ -231,8 +231,8 @@ __global__ void __launch_bounds__(128) k_step_eos(const double* __restrict__ A, 
 //
 // The binary64 step was bound by some 600 FP64 instructions per cell (65
 // clocks of a scheduler each); 83 remain beside 3,500 in all, the FP64 pipe
-// 71 % busy.  128^3 box, Gamma = 1.2, m = 0.3: step 2.19 -> 0.396 ms,
-// initialisation 0.80 -> 0.149 ms, macroscopic output 1.06 -> 0.26 ms.
+// 71 % busy.  128^3 box, Gamma = 1.2, m = 0.3: step 2.19 -> 0.390 ms,
+// initialisation 0.80 -> 0.152 ms, macroscopic output 1.06 -> 0.26 ms.
 // ---------------------------------------------------------------------------
 
 // On scaled moments (E in [1, 2)): P, 1/W, b = M^2 / W, sq = sqrt(1 - beta^2);

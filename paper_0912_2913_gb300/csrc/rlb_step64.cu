@@ -714,7 +714,8 @@ void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B
     // eight lanes per cell while the lanes fit one warp per scheduler
     // (N <= 16 x SMs), unless RLB_F64_SPLIT says otherwise; same values.  The
     // 1600-cell tube, issued on the stream: 10.24 us per step in binary64, 8.20
-    // in fixed point (20 instead of 103 FP64 instructions per warp).
+    // in fixed point (20 instead of 103 FP64 instructions per warp), 6.25
+    // launched back to back.
     const bool split = (g.f64split == 1 && g.N < (1 << 27)) || (g.f64split < 0 && g.N <= 16ll * nsm);
     if (ph.fx_on) {
         if (split) {
