@@ -154,7 +154,7 @@ __device__ __forceinline__ bool step_cell_f64(const double* __restrict__ A, doub
 template <int XBC, bool SOLID>
 __global__ void __launch_bounds__(128) k_step_f64(const double* __restrict__ A, double* __restrict__ B, Geom g,
                                                   Phys ph, Counters cnt, int count, long long step_index) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int idx = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);
     if (idx >= g.N) return;
     int x, y, z;
     cell_coords(g, idx, x, y, z);
@@ -192,11 +192,11 @@ template <int XBC, bool SOLID>
 __global__ void __launch_bounds__(128) k_step_f64_split(const double* __restrict__ A, double* __restrict__ B, Geom g,
                                                         Phys ph, Counters cnt, int count, long long step_index) {
     const unsigned full = 0xffffffffu;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);  // 8 N < 2^31 (small lattices; tests)
     const int j = threadIdx.x & 7;  // lane of the cell's group
-    const long long cell = t >> 3;
+    const int cell = (int)((unsigned)t >> 3);
     const bool live = cell < g.N;
-    const int idx = live ? (int)cell : 0;
+    const int idx = live ? cell : 0;
     int x, y, z;
     cell_coords(g, idx, x, y, z);
     const bool halo = g.zhalo && (z == 0 || z == g.nz - 1);  // filled by the exchange
@@ -733,11 +733,11 @@ void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B
         return;
     }
     if (split) {
-        k_step_f64_split<XBC, true><<<blocks(8ll * g.N, 128), 128, 0, st>>>(A, B, g, ph, cnt, c, step_index);
+        launch_dependent(k_step_f64_split<XBC, true>, blocks(8ll * g.N, 128), 128, 0, st, A, B, g, ph, cnt, c, step_index);
         return;
     }
     const int tb = blocks(g.N, 128) < (unsigned)nsm ? 32 : 128;
-    k_step_f64<XBC, true><<<blocks(g.N, tb), tb, 0, st>>>(A, B, g, ph, cnt, c, step_index);
+    launch_dependent(k_step_f64<XBC, true>, blocks(g.N, tb), tb, 0, st, A, B, g, ph, cnt, c, step_index);
 }
 }  // namespace
 
