@@ -767,12 +767,6 @@ __device__ __forceinline__ void zero_to_ghost(int x, int nx, int idx, long long 
     }
 }
 
-// mu offset of the outflow ghost that copies x (0 if none)
-template <int XBC>
-__device__ __forceinline__ int dup_of(int x, int nx) {
-    return (XBC != XBC_PERIODIC && x == nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
-}
-
 // Register kernel.  PIPE: persistent grid-stride loop over the cells;
 // otherwise one cell per thread.
 template <typename T, int XBC, int MINB, bool PIPE>

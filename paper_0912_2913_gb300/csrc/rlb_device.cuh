@@ -222,6 +222,17 @@ struct PullOffsets {
     }
 };
 
+// Offset of the outflow ghost that copies x (0 if none), and whether its only
+// fluid plane x = 1 is copied by both ghosts (+1 from dup_of, and -1).
+template <int XBC>
+__device__ __forceinline__ int dup_of(int x, int nx) {
+    return (XBC != XBC_PERIODIC && x == nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
+}
+template <int XBC>
+__device__ __forceinline__ bool dup_both(int nx) {
+    return XBC == XBC_OUTFLOW_BOTH && nx == 3;
+}
+
 // ---------------------------------------------------------------------------
 // Moments in pair form: S = sum f, E = sum g, M = c_l sum g e.
 // ---------------------------------------------------------------------------

@@ -94,10 +94,14 @@ __global__ void __launch_bounds__(128) k_step_f64_df(const double* __restrict__ 
         return;
     }
     const PullOffsets o(g, x, y, z);
-    const int dup = (XBC != XBC_PERIODIC && x == g.nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
+    const int dup = dup_of<XBC>(x, g.nx);
+    const bool both = dup_both<XBC>(g.nx);
     auto put = [&](int q, double v) {
         B[RLB_CHK(q * S + idx, 38ll * S)] = v;
-        if (dup) B[RLB_CHK(q * S + idx + dup, 38ll * S)] = v;
+        if (dup) {
+            B[RLB_CHK(q * S + idx + dup, 38ll * S)] = v;
+            if (both) B[RLB_CHK(q * S + idx - 1, 38ll * S)] = v;
+        }
     };
     // ---- g phase: energy-momentum populations (they alone fix eps, beta) ----
     dfl G[19];

@@ -84,7 +84,8 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
     if (XBC != XBC_PERIODIC && (x == g.nx - 1 || (x == 0 && !keep))) return;
     PullOffsets o(g, x, y, z);
     if (keep) o.xm = o.xp = o.ym = o.yp = o.zm = o.zp = 0;
-    const int dup = (XBC != XBC_PERIODIC && x == g.nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
+    const int dup = dup_of<XBC>(x, g.nx);
+    const bool both = dup_both<XBC>(g.nx);
     float* Bc = B + idx;
     float* Bgc = Bg + idx;
     auto put = [&](int q, float v, float old) {
@@ -94,10 +95,16 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
             b[RLB_CHK_OFF(pq(q) * S, idx, lim)] = v;
             // the outflow copy: dup (+-1) moves the pointer, so that the
             // unsigned offset never has to hold a negative value
-            if (dup) (b + dup)[RLB_CHK_OFF(pq(q) * S, idx + dup, lim)] = v;
+            if (dup) {
+                (b + dup)[RLB_CHK_OFF(pq(q) * S, idx + dup, lim)] = v;
+                if (both) (b - 1)[RLB_CHK_OFF(pq(q) * S, idx - 1, lim)] = v;
+            }
         } else {
             Bc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v;
-            if (dup) Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
+            if (dup) {
+                Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
+                if (both) Bc[RLB_CHK_OFF(q * S - 1, idx, 38ll * S)] = v;
+            }
         }
     };
     if (PREF) {
@@ -171,15 +178,22 @@ __global__ void __launch_bounds__(256, 3) k_step_f32_pipe(const float* __restric
             continue;
         }
         const PullOffsets o(g, x, y, z);
-        const int dup = (XBC != XBC_PERIODIC && x == g.nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
+        const int dup = dup_of<XBC>(x, g.nx);
+        const bool both = dup_both<XBC>(g.nx);
         float* Bc = B + idx;
         auto put = [&](int q, float v, float) {
             if (CS) {
                 __stcs(Bc + q * S, v);
-                if (dup) __stcs(Bc + q * S + dup, v);
+                if (dup) {
+                    __stcs(Bc + q * S + dup, v);
+                    if (both) __stcs(Bc + q * S - 1, v);
+                }
             } else {
                 Bc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v;
-                if (dup) Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
+                if (dup) {
+                    Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
+                    if (both) Bc[RLB_CHK_OFF(q * S - 1, idx, 38ll * S)] = v;
+                }
             }
         };
         if (SOLID && is_solid(__ldg(RLB_CHK_PTR(A, 19 * S + idx, 38ll * S)))) {

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256, MINB)
                 return row[q * plane_elems + (ex > 0 ? xm : (ex < 0 ? xp : x))];
             };
             auto bounce = [&](int q, int i) { return __ldg(RLB_CHK_PTR(A, (q - i + opp(i)) * S + idx, 38ll * S)); };  // link bounce-back
-            const int dup = (XBC != XBC_PERIODIC && x == nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
+            const int dup = dup_of<XBC>(x, nx);  // never both ghosts: nx is a multiple of four here
             float* Bc = B + idx;
             auto put = [&](int q, float v, float) {
                 Bc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v;
