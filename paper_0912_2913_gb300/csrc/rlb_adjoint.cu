@@ -831,6 +831,10 @@ __global__ void __launch_bounds__(128, MINB)
             if (dup) {
 #pragma unroll
                 for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx + dup, 38ll * S)];
+                if (dup_both<XBC>(g.nx)) {
+#pragma unroll
+                    for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx - 1, 38ll * S)];
+                }
             }
         };
         if (!PIPE) {
@@ -965,6 +969,10 @@ __device__ __noinline__ double adjoint_cell_general(const double* A, const doubl
         if (dup) {
 #pragma unroll
             for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx + dup, 38ll * S)];
+            if (dup_both<XBC>(g.nx)) {
+#pragma unroll
+                for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx - 1, 38ll * S)];
+            }
         }
     };
     unsigned bounced = 0u;
@@ -1185,10 +1193,13 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
             for (int i = 0; i < 19; ++i) m = max(m, (uint32_t)__double2hiint(col[base + i][tid]) << 1);
             return (int)(m >> 21);
         };
-        // mu also takes lambda of the outflow ghost that copies x
+        // mu also takes lambda of the outflow ghosts that copy x
         auto add_dup = [&](int base) {
+            for (int off = dup;; off = -1) {
 #pragma unroll 4
-            for (int i = 0; i < 19; ++i) col[base + i][tid] += Lc[RLB_CHK_OFF((base + i) * S + dup, idx, 38ll * S)];
+                for (int i = 0; i < 19; ++i) col[base + i][tid] += Lc[RLB_CHK_OFF((base + i) * S + off, idx, 38ll * S)];
+                if (!dup_both<XBC>(g.nx) || off < 0) break;
+            }
         };
         int eh = max_exp(38);
         unsigned bounced = 0u;
@@ -1398,6 +1409,10 @@ __global__ void __launch_bounds__(128)
                 if (dup) {
                     uf[n] += __ldg(Lin + RLB_CHK(iv[n] * S + idx + dup, 38ll * S));
                     ug[n] += __ldg(Lin + RLB_CHK((19 + iv[n]) * S + idx + dup, 38ll * S));
+                    if (dup_both<XBC>(g.nx)) {
+                        uf[n] += __ldg(Lin + RLB_CHK(iv[n] * S + idx - 1, 38ll * S));
+                        ug[n] += __ldg(Lin + RLB_CHK((19 + iv[n]) * S + idx - 1, 38ll * S));
+                    }
                 }
             }
         }
@@ -1653,6 +1668,10 @@ __global__ void __launch_bounds__(kStageThreads, 3)
                 if (dup) {
 #pragma unroll
                     for (int i = 0; i < 19; ++i) mug[i] += *pl(19 + i, idx + dup);
+                    if (dup_both<XBC>(g.nx)) {
+#pragma unroll
+                        for (int i = 0; i < 19; ++i) mug[i] += *pl(19 + i, idx - 1);
+                    }
                 }
                 cell_g(h, mug, c, r);
             }
@@ -1683,6 +1702,10 @@ __global__ void __launch_bounds__(kStageThreads, 3)
             if (dup) {
 #pragma unroll
                 for (int i = 0; i < 19; ++i) muf[i] += *pl(i, idx + dup);
+                if (dup_both<XBC>(g.nx)) {
+#pragma unroll
+                    for (int i = 0; i < 19; ++i) muf[i] += *pl(i, idx - 1);
+                }
             }
             float tf, aS, fbx, fby, fbz;
             cell_f(h, muf, r, c, tf, aS, fbx, fby, fbz);
@@ -1830,6 +1853,10 @@ __global__ void __launch_bounds__(kStageThreads, 3)
 #pragma unroll
                         for (int i = 0; i < 19; ++i) mug[i] += *pl(19 + i, idx + dup);
                     }
+                    if (dup_both<XBC>(g.nx)) {
+#pragma unroll
+                        for (int i = 0; i < 19; ++i) mug[i] += *pl(19 + i, idx - 1);
+                    }
                 }
                 cell_g(h, mug, c, r);
             }
@@ -1868,6 +1895,10 @@ __global__ void __launch_bounds__(kStageThreads, 3)
                 } else {
 #pragma unroll
                     for (int i = 0; i < 19; ++i) muf[i] += *pl(i, idx + dup);
+                }
+                if (dup_both<XBC>(g.nx)) {
+#pragma unroll
+                    for (int i = 0; i < 19; ++i) muf[i] += *pl(i, idx - 1);
                 }
             }
             float tf, aS, fbx, fby, fbz;

@@ -45,3 +45,51 @@ def test_three_cells_between_outflow_ghosts(prec, env, c_l, monkeypatch):
     n, e, b, ok = sim.macro(where="host")
     sim.close()
     assert ok and max(rel_errors((n, e, b), ref)) <= TOL[prec]
+
+
+def _adjoint_case(w, prec, state=None, lam=None, noalloc=False):
+    """lambda_t, dL/dtau, dL/dbeta_in of one adjoint step and the oracle's; the
+    state (oracle cells) and lambda as the GPU stores them."""
+    from paper_0912_2913_gb300 import RLB
+    from paper_0912_2913_gb300 import _native as N
+
+    p = oracle.Params(**w.params())
+    sim = RLB.from_workload(w, prec, device="cuda:0").init_fields(w.n, w.eps, w.beta, w.solid)
+    rest = 0.0
+    if prec == "fp32":
+        rest = np.stack(oracle.equilibrium(sim.params.n_ref, sim.params.eps_ref, np.zeros(3), w.c_l))
+    st = sim.cells_to_state(_cuda(state - rest))
+    li = sim.cells_to_state(_cuda(lam))
+    lo = torch.full_like(li, float("nan"))
+    acc = torch.zeros(4, dtype=torch.float64, device="cuda")
+    if noalloc:
+        N.rlb_adjoint_step_noalloc(sim.ctx, st, li, lo, acc[0:1], acc[1:4])
+    else:
+        sim.adjoint_step(st, li, lo, acc[0:1], acc[1:4])
+    got = sim.state_to_cells(lo).double().cpu().numpy()
+    lam = sim.state_to_cells(li).double().cpu().numpy()
+    state = sim.state_to_cells(st).double().cpu().numpy() + rest
+    acc = acc.cpu().numpy()
+    sim.close()
+    lam_o, dtau_o, dbin_o = oracle.adjoint_step(p, state, lam, w.solid)
+    return (got, acc[0], acc[1:]), (lam_o, dtau_o, dbin_o)
+
+
+@pytest.mark.parametrize("size", [(3, 4, 5), (3, 41, 43)], ids=["small", "large"])
+@pytest.mark.parametrize("prec,c_l,env", [("fp64", 1.0, {}), ("fp64", 3.0, {}), ("fp32", 1.0, {}),
+                                          ("fp32", 1.0, {"RLB_ADJ_COOP": "0"}), ("fp32", 1.0, {"RLB_ADJ_PIPE": "0"}),
+                                          ("fp32", 1.0, {"RLB_ADJ_PIPE": "1"})])
+def test_adjoint_of_three_cells_between_outflow_ghosts(size, prec, c_l, env, monkeypatch):
+    """The adjoint of that step: mu of x = 1 takes lambda of both ghosts."""
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    w = tiny_workload(*size, 2, seed=8, c_l=c_l)
+    p = oracle.Params(**w.params())
+    st = oracle.init(p, w.n, w.eps, w.beta)
+    oracle.run(p, st, 2)
+    lam = np.random.default_rng(1).normal(size=st.shape)
+    got, ref = _adjoint_case(w, prec, st, lam)
+    tol = 1e-11 if prec == "fp64" else 1e-4
+    big = np.abs(lam).max()
+    assert np.max(np.abs(got[0] - ref[0])) <= tol * np.abs(ref[0]).max()
+    assert abs(got[1] - ref[1]) <= tol * np.prod(size) * big
