@@ -1005,6 +1005,14 @@ __device__ __noinline__ double adjoint_cell_general(const double* A, const doubl
     return (r.tacc + tf) * c.inv_tau2;
 }
 
+// Whether the product sum dot 2^(ea + eb - 2102) of values with block
+// exponents ea and eb can be formed by fx_to, whose result has to be a normal
+// number: otherwise (states of 1e-80 with lambda of 1e-230) the exponent would
+// wrap into the sign, and the cell is left to the binary64 form.
+__device__ __forceinline__ bool dot_in_range(int64_t dot, int ea, int eb) {
+    return dot == 0 || (ea + eb >= 1080 && ea + eb <= 3062);
+}
+
 // What the f phase and the output need of a cell (see the formulas above).
 struct AdjFxCell {
     double x, y, z, E4, rs, rD, ux, uy, uz, yx, yy, yz, uy_, vx, vy, vz, aE;  // d, 4 E, 1/s, 1/D, u, G u, u.y, 36 V, a_E
@@ -1268,6 +1276,8 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                         zf = (float)(int32_t)(dz >> 32);
             ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
         }
+        const int64_t gdot = dot.result(19);
+        ok = ok && dot_in_range(gdot, em, eh);
         if (!ok) {
             cp_async_wait<0>();
             tau_acc += adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
@@ -1275,7 +1285,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
             continue;
         }
         AdjFxCell t;
-        adj_fx_g(E, dx, dy, dz, dot.result(19), m0, Sx, Sy, Sz, Pxy, Pyz, Pzx, Txy, Tyz, Tzx, Vx, Vy, Vz, eh, em, ph, k, t);
+        adj_fx_g(E, dx, dy, dz, gdot, m0, Sx, Sy, Sz, Pxy, Pyz, Pzx, Txy, Tyz, Tzx, Vx, Vy, Vz, eh, em, ph, k, t);
         // ---- f
         cp_async_wait<0>();
         if (bounced) {
@@ -1320,7 +1330,9 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                 Fx += dl, Fy -= dl;
                 rotate3(Fx, Fy, Fz);
             }
-            adj_fx_f(Sf, fd.result(19), Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
+            const int64_t fdot = fd.result(19);
+            ok = ok && dot_in_range(fdot, ef, fh);
+            adj_fx_f(Sf, fdot, Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
         }
         if (!ok) {
             tau_acc += adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
@@ -1490,6 +1502,7 @@ __global__ void __launch_bounds__(128)
     const int32_t Eh = (int32_t)(E >> 32);
     const float Ef = (float)Eh, xf = (float)(int32_t)(dx >> 32), yf = (float)(int32_t)(dy >> 32), zf = (float)(int32_t)(dz >> 32);
     ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
+    ok = ok && dot_in_range(dot, em, eh) && dot_in_range(fd, ef, fh);
     AdjFxCell t;
     int ek = 0;
     if (ok) {

@@ -93,3 +93,26 @@ def test_adjoint_of_three_cells_between_outflow_ghosts(size, prec, c_l, env, mon
     big = np.abs(lam).max()
     assert np.max(np.abs(got[0] - ref[0])) <= tol * np.abs(ref[0]).max()
     assert abs(got[1] - ref[1]) <= tol * np.prod(size) * big
+
+
+@pytest.mark.parametrize("size", [(5, 4, 3), (23, 15, 15)], ids=["eight_lanes", "staged"])
+@pytest.mark.parametrize("sscale,lscale", [(1e-40, 1e-270), (1e-60, 1e-250), (1e-80, 1e-230), (1e60, 1e240)])
+def test_fp64_adjoint_of_tiny_states_and_lambda(size, sscale, lscale):
+    """States and lambda whose products leave the range of binary64 (the terms
+    of dL/dtau underflow to zero) and lambda that loses bits itself: everything
+    finite and equal to the oracle.  Bounds: 1e-11 of the largest values, as at
+    scale one, and 64 smallest subnormals a cell for what underflows (57
+    products of a cell, the oracle's and the kernel's, to half of one each)."""
+    w = tiny_workload(*size, 1, seed=3, bmax=0.5)
+    p = oracle.Params(**w.params())
+    st = oracle.init(p, w.n, w.eps, w.beta)
+    oracle.run(p, st, 2)
+    st *= sscale
+    lam = np.random.default_rng(2).normal(size=st.shape) * lscale
+    lam[:, 0] = 0.0
+    got, ref = _adjoint_case(w, "fp64", st, lam)
+    big, tiny, N = np.abs(lam).max(), 5e-324 * 64, np.prod(size)
+    assert np.isfinite(got[1]) and np.isfinite(got[0]).all()
+    assert np.max(np.abs(got[0] - ref[0])) <= 1e-11 * np.abs(ref[0]).max() + tiny
+    assert abs(got[1] - ref[1]) <= 1e-11 * N * big * np.abs(st).max() + N * tiny
+    assert np.max(np.abs(got[2] - ref[2])) <= 1e-11 * N * big + N * tiny
