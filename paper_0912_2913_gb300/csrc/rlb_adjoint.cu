@@ -943,8 +943,14 @@ __global__ void __launch_bounds__(128, MINB)
 // 1.51 -> 0.83 ms, 192^3 box 5.1 -> 2.35 ms; blocks of 64 threads: 5, 6 and 7
 // per SM 2.65, 2.35 and 2.49 ms; all values in registers and unrolled, 3
 // blocks of 128: 2.35 ms on the box, 0.854 on the sphere.
-// Error against 113-bit references: nu 1.2e-16 (2 to 3e-16 before), the terms
-// of dL/dtau 7.4e-17 rms and below 3e-17 in the mean (1.5e-16 and 7e-17).
+// Error against 113-bit references (1.5e6 cells, |beta_a| up to 0.5, lambda
+// normal): nu 1.2e-16 (2 to 3e-16 in binary64), the terms of dL/dtau 1.1e-16
+// rms (3.0e-16).  What the sum over the lattice sees is their mean, since it
+// counts N times: for lambda of zero mean -7e-20 +- 9e-20 (binary64 -3e-20 +-
+// 2e-19), for binary32 lambda -4e-19, for lambda of one sign -1.3e-17
+// (5.2e-17).  With ties always up, weights floored and a mean in place of the
+// low halves' products these were -2.6e-18, +6.7e-17 and -1.5e-17; without
+// that the 200x100x100 sphere takes 0.83 ms instead of 0.88.
 // ---------------------------------------------------------------------------
 
 struct AdjFx {
@@ -1046,17 +1052,18 @@ __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int6
     const double e2 = fma(-D, r0, 1.0);
     t.rD = fma(r0, fma(e2, e2, e2), r0);
     t.ux = t.x * t.rD, t.uy = t.y * t.rD, t.uz = t.z * t.rD;
-    const FxSplit sp = fx_split((Sx + Sy + Sz) + (Pxy + Pyz + Pzx));
+    const int64_t sp = (Sx + Sy + Sz) + (Pxy + Pyz + Pzx);
     // 8 G: 13.5 / 36 = 3/8; the partial sums may wrap, the result does not
-    const int64_t kap = (m0 << 2) - (fx_mul(sp, k.kS1) << 2) + 4;
-    auto g38 = [](int64_t v, int64_t k8) { return fx_weight((v + (v << 1) + k8) >> 3); };
+    const int64_t kap = (m0 << 2) - (fx_mul_exact(sp, k.kS1) << 2);
+    auto g38 = [](int64_t v, int64_t k8) { return fx_weight_signed(fx_round3_even(v + (v << 1) + k8)); };
+    auto g38_off = [](int64_t v) { return fx_weight_signed((v + (v << 1) + 4) >> 3); };  // u_a u_b has either sign
     const double Gxx = fx_to(g38(Sx + Pxy + Pzx, kap), km), Gyy = fx_to(g38(Sy + Pxy + Pyz, kap), km),
                  Gzz = fx_to(g38(Sz + Pyz + Pzx, kap), km);
-    const double Gxy = fx_to(g38(Txy, 4), km), Gxz = fx_to(g38(Tzx, 4), km), Gyz = fx_to(g38(Tyz, 4), km);
+    const double Gxy = fx_to(g38_off(Txy), km), Gxz = fx_to(g38_off(Tzx), km), Gyz = fx_to(g38_off(Tyz), km);
     t.yx = fma(Gxx, t.ux, fma(Gxy, t.uy, Gxz * t.uz));
     t.yy = fma(Gxy, t.ux, fma(Gyy, t.uy, Gyz * t.uz));
     t.yz = fma(Gxz, t.ux, fma(Gyz, t.uy, Gzz * t.uz));
-    t.aE = fx_to(fx_mul(sp, k.kE1) + fx_mul(fx_split(m0 << 3), k.kE0), km - 1);
+    t.aE = fx_to(fx_mul_exact(sp, k.kE1) + fx_mul_exact(m0 << 3, k.kE0), km - 1);
     t.uy_ = fma(t.ux, t.yx, fma(t.uy, t.yy, t.uz * t.yz));
     t.vx = fx_to(Vx, km), t.vy = fx_to(Vy, km), t.vz = fx_to(Vz, km);
     const double Vd = fma(t.vx, t.x, fma(t.vy, t.y, t.vz * t.z));
@@ -1069,9 +1076,9 @@ __device__ __forceinline__ void adj_fx_f(int64_t Sf, int64_t fd, int64_t Fs, int
                                          int ef, const Phys& ph, const AdjFx& k, AdjFxCell& t) {
     const double Sd = fx_to_even(Sf, fh - 1079);
     const int kf = ef - 1079;
-    const double fx = fx_to(fx_weight(Fx), kf), fy = fx_to(fx_weight(Fy), kf), fz = fx_to(fx_weight(Fz), kf);
+    const double fx = fx_to(fx_weight_signed(Fx), kf), fy = fx_to(fx_weight_signed(Fy), kf), fz = fx_to(fx_weight_signed(Fz), kf);
     const double Fu = fma(fx, t.ux, fma(fy, t.uy, fz * t.uz));
-    const double aS = fma(0.25, Fu, fx_to(fx_mul(fx_split(Fs), k.kS36), kf - 1));
+    const double aS = fma(0.25, Fu, fx_to(fx_mul_exact(Fs, k.kS36), kf - 1));
     t.tsum += fx_to(fd, ef + fh - 2102) - Sd * aS;
     const double sD = (0.25 * Sd) * t.rD;
     const double aD = -fma(sD, Fu, t.uy_);
@@ -1233,31 +1240,31 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         {
             const int64_t h0 = fx_from(col[38][tid], eh), u0 = fx_from(col[19][tid], em);
             E = fx_round4(h0);
-            m0 = fx_round4(u0);
-            dot.add(fx_split(h0), fx_split(u0));
+            m0 = fx_round4_even(u0);
+            dot.add(h0, u0);
 #pragma unroll 1
             for (int r = 0; r < 3; ++r) {
                 const Round v(r);
                 int64_t d, sg, dl;
-                auto pair = [&](int i, int j) {
+                auto pair = [&](int i, int j, int half) {
                     const int64_t a = fx_from(col[38 + i][tid], eh), b = fx_from(col[38 + j][tid], eh);
                     const int64_t ua = fx_from(col[19 + i][tid], em), ub = fx_from(col[19 + j][tid], em);
                     E += fx_round4(a + b);
-                    dot.add(fx_split(a), fx_split(ua));
-                    dot.add(fx_split(b), fx_split(ub));
+                    dot.add(a, ua);
+                    dot.add(b, ub);
                     d = fx_round4(a - b);
-                    sg = fx_round4(ua + ub);
+                    sg = (ua + ub + half) >> 4;
                     dl = fx_round4(ua - ub);
                 };
-                pair(v.ax, v.ax + 1);
+                pair(v.ax, v.ax + 1, 7);  // sigma's ties: down for the axis pairs, up for the others (weights 6 and 6)
                 dx += d;
                 Sx = sg << 1;
                 Vx += dl << 1;
-                pair(v.pp, v.pp + 1);
+                pair(v.pp, v.pp + 1, 8);
                 dx += d, dy += d;
                 Vx += dl, Vy += dl;
                 Pxy = sg, Txy = sg;
-                pair(v.pm, v.mp);
+                pair(v.pm, v.mp, 8);
                 dx += d, dy -= d;
                 Vx += dl, Vy -= dl;
                 Pxy += sg, Txy -= sg;
@@ -1276,7 +1283,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                         zf = (float)(int32_t)(dz >> 32);
             ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
         }
-        const int64_t gdot = dot.result(19);
+        const int64_t gdot = dot.result();
         ok = ok && dot_in_range(gdot, em, eh);
         if (!ok) {
             cp_async_wait<0>();
@@ -1302,35 +1309,35 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
             const int64_t h0 = fx_from(col[38][tid], fh), u0 = fx_from(col[0][tid], ef);
             int64_t Sf = fx_round4(h0);
             FxDot fd{};
-            fd.add(fx_split(h0), fx_split(u0));
-            const int64_t u4 = fx_round4(u0);
+            fd.add(h0, u0);
+            const int64_t u4 = fx_round4_even(u0);
             int64_t Fs = (u4 << 3) + (u4 << 2);  // 36 w0 mu_f0
             int64_t Fx = 0, Fy = 0, Fz = 0;
 #pragma unroll 1
             for (int r = 0; r < 3; ++r) {
                 const Round v(r);
                 int64_t sg, dl;
-                auto pair = [&](int i, int j) {
+                auto pair = [&](int i, int j, int half) {
                     const int64_t a = fx_from(col[38 + i][tid], fh), b = fx_from(col[38 + j][tid], fh);
                     const int64_t ua = fx_from(col[i][tid], ef), ub = fx_from(col[j][tid], ef);
                     Sf += fx_round4(a + b);
-                    fd.add(fx_split(a), fx_split(ua));
-                    fd.add(fx_split(b), fx_split(ub));
-                    sg = fx_round4(ua + ub);
+                    fd.add(a, ua);
+                    fd.add(b, ub);
+                    sg = (ua + ub + half) >> 4;
                     dl = fx_round4(ua - ub);
                 };
-                pair(v.ax, v.ax + 1);
+                pair(v.ax, v.ax + 1, 7);
                 Fs += sg << 1;
                 Fx += dl << 1;
-                pair(v.pp, v.pp + 1);
+                pair(v.pp, v.pp + 1, 8);
                 Fs += sg;
                 Fx += dl, Fy += dl;
-                pair(v.pm, v.mp);
+                pair(v.pm, v.mp, 8);
                 Fs += sg;
                 Fx += dl, Fy -= dl;
                 rotate3(Fx, Fy, Fz);
             }
-            const int64_t fdot = fd.result(19);
+            const int64_t fdot = fd.result();
             ok = ok && dot_in_range(fdot, ef, fh);
             adj_fx_f(Sf, fdot, Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
         }
@@ -1457,18 +1464,19 @@ __global__ void __launch_bounds__(128)
     auto dot4 = [&]() {
         FxDot d{};
 #pragma unroll
-        for (int n = 0; n < 4; ++n) d.add(fx_split(hx[n]), fx_split(ux[n]));
-        return d.result(j == 0 ? 4 : (j == 1 ? 3 : 2));
+        for (int n = 0; n < 4; ++n) d.add(hx[n], ux[n]);
+        return d.result();
     };
     long long E = fx_round4(hx[0] + hx[1]) + fx_round4(hx[2] + hx[3]), dot = dot4();
     const long long d_j = fx_round4(hx[0] - hx[1]), d_8 = fx_round4(hx[2] - hx[3]);
-    const long long s_j = fx_round4(ux[0] + ux[1]), s_8 = fx_round4(ux[2] + ux[3]);  // lane 1's s_8: the rest population
+    const int half = j < 3 ? 7 : 8;  // ties of the axis pairs down, of the others up
+    const long long s_j = (ux[0] + ux[1] + half) >> 4, s_8 = j == 1 ? fx_round4_even(ux[2]) : fx_round4(ux[2] + ux[3]);  // lane 1's s_8: the rest population
     const long long l_j = fx_round4(ux[0] - ux[1]), l_8 = fx_round4(ux[2] - ux[3]);
     // f
 #pragma unroll
     for (int n = 0; n < 4; ++n) hx[n] = fx_from(hf[n], fh), ux[n] = fx_from(uf[n], ef);
     long long Sf = fx_round4(hx[0] + hx[1]) + fx_round4(hx[2] + hx[3]), fd = dot4();
-    const long long sf_j = fx_round4(ux[0] + ux[1]), sf_8 = fx_round4(ux[2] + ux[3]);
+    const long long sf_j = (ux[0] + ux[1] + half) >> 4, sf_8 = j == 1 ? fx_round4_even(ux[2]) : fx_round4(ux[2] + ux[3]);
     const long long lf_j = fx_round4(ux[0] - ux[1]), lf_8 = fx_round4(ux[2] - ux[3]);
     long long Fs = (j < 3 ? sf_j << 1 : sf_j) + (j == 0 ? sf_8 : (j == 1 ? (sf_8 << 3) + (sf_8 << 2) : 0));
 #pragma unroll

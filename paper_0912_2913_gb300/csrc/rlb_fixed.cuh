@@ -165,8 +165,10 @@ RLB_FX int64_t fx_from(double v, int emax) {
     return (int64_t)((x ^ (uint64_t)s) - (uint64_t)s);
 }
 
-// the factor (1 - 2^-54) of the binary64 weights
+// the factor (1 - 2^-54) of the binary64 weights; for signed values, whose
+// rounding must not have a mean, to nearest
 RLB_FX int64_t fx_weight(int64_t v) { return v - (v >> 54); }
+RLB_FX int64_t fx_weight_signed(int64_t v) { return v - ((v + (1ll << 53)) >> 54); }
 
 // v 2^s for v >= 0 with v 2^s < 2^63 (truncated)
 RLB_FX int64_t fx_fixed(double v, int s) {
@@ -177,6 +179,11 @@ RLB_FX int64_t fx_fixed(double v, int s) {
 
 // (x + 8) >> 4: from units of 2^-60 to 2^-56 of the block, rounded to nearest
 RLB_FX int64_t fx_round4(int64_t x) { return (x + 8) >> 4; }
+// Ties always rounded up are an error common to all cells: in signed sums that
+// enter a sum over the lattice they go to even (also (x + 4) >> 3), or down in
+// one half of the terms.
+RLB_FX int64_t fx_round4_even(int64_t x) { return (x + 7 + ((x >> 4) & 1)) >> 4; }
+RLB_FX int64_t fx_round3_even(int64_t x) { return (x + 3 + ((x >> 3) & 1)) >> 3; }
 
 // t 2^eb rounded to nearest binary64, |t| < 2^63; the result is a normal
 // number (eb from the block exponent, at least 100).
@@ -234,15 +241,36 @@ RLB_FX int64_t fx_mul(const FxSplit& a, const FxSplit& b) {
     const int64_t mid = (int64_t)a.h * b.l + ((int64_t)a.l * b.h + 0x60000000ll);
     return (int64_t)a.h * b.h + (mid >> 31);
 }
-// sum of up to 19 products (a b) 2^-64 of values below 2^61, rounded once
+// c + the high word of a b
+RLB_FX uint32_t fx_madhi(uint32_t a, uint32_t b, uint32_t c) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b) + c;
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32) + c;
+#endif
+}
+// The same with the product of the low halves itself (the mean is wrong where
+// they are short: sums of binary32 values), and a's lowest bit rounded to even.
+RLB_FX int64_t fx_mul_exact(int64_t a, const FxConst& b) {
+    const FxSplit s = fx_split(a + ((a >> 1) & a & 1));
+    const uint32_t low = fx_madhi((uint32_t)s.l << 1, (uint32_t)b.l, 1u << 30);
+    const int64_t mid = (int64_t)s.h * b.l + ((int64_t)s.l * b.h + (int64_t)(uint64_t)low);
+    return (int64_t)s.h * b.h + (mid >> 31);
+}
+// sum of up to 19 products (a b) 2^-64 of values below 2^61, rounded once.  The
+// products of the low halves are added too: their mean in their place would
+// be an error common to all cells whose values are short (binary32 lambda,
+// zeros), 25 times the other errors' mean.
 struct FxDot {
     int64_t hh, mid;
-    RLB_FX void add(const FxSplit& a, const FxSplit& b) {
+    uint32_t low;
+    RLB_FX void add(int64_t x, int64_t y) {
+        const FxSplit a = fx_split(x), b = fx_split(y);
         hh += (int64_t)a.h * b.h;
         mid += ((int64_t)a.h * b.l + (int64_t)a.l * b.h) >> 6;
+        low = fx_madhi((uint32_t)x, (uint32_t)b.l >> 6, low);
     }
-    // n: how many of the products have low halves (their mean is added)
-    RLB_FX int64_t result(int n) const { return hh + ((mid + ((int64_t)n << 23) + (1 << 24)) >> 25); }
+    RLB_FX int64_t result() const { return hh + ((mid + (int64_t)low + (1 << 24)) >> 25); }
 };
 
 // What a cell's equilibria are made of, in units of 2^-62 of the normalised
