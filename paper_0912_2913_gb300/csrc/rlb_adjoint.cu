@@ -960,7 +960,20 @@ struct AdjFx {
     FxConst kS36;  // 1 / 36                      x 2^65
 };
 
+// 2^k, |k| <= 1022
+__device__ __forceinline__ double pow2d(int k) { return fx_double((uint32_t)(1023 + k) << 20, 0u); }
+// k such that the largest of N values times 2^k is of order one (non-finite
+// values: 0)
+template <int N>
+__device__ __forceinline__ int unit_shift(const double* v) {
+    const int e = fx_max_exponent<N>(v);
+    return e == 0x7FF ? 0 : max(-1022, min(1022, 1023 - e));
+}
+
 // A cell in binary64 throughout (any state); the terms of dL/dtau returned.
+// lambda_t is linear in lambda and does not depend on the unit of the state,
+// so both are brought to order one first (exactly, by powers of two): products
+// of states of 1e-80 with lambda of 1e-240 lose no bits on the way.
 template <int XBC>
 __device__ __noinline__ double adjoint_cell_general(const double* A, const double* Lin, double* Lout, const Geom& g,
                                                     const AdjConst<double>& c, int idx) {
@@ -969,20 +982,17 @@ __device__ __noinline__ double adjoint_cell_general(const double* A, const doubl
     cell_coords(g, idx, x, y, z);
     const PullOffsets o(g, x, y, z);
     const int dup = dup_of<XBC>(x, g.nx);
-    auto load_mu = [&](double* mu, int base) {
-#pragma unroll
-        for (int i = 0; i < 19; ++i) mu[i] = Lin[RLB_CHK((base + i) * S + idx, 38ll * S)];
-        if (dup) {
-#pragma unroll
-            for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx + dup, 38ll * S)];
-            if (dup_both<XBC>(g.nx)) {
-#pragma unroll
-                for (int i = 0; i < 19; ++i) mu[i] += Lin[RLB_CHK((base + i) * S + idx - 1, 38ll * S)];
-            }
-        }
-    };
+    double h[19], mu[38];
+    double *const muf = mu, *const mug = mu + 19;
+    for (int q = 0; q < 38; ++q) mu[q] = Lin[RLB_CHK(q * S + idx, 38ll * S)];
+    if (dup) {
+        for (int q = 0; q < 38; ++q) mu[q] += Lin[RLB_CHK(q * S + idx + dup, 38ll * S)];
+        if (dup_both<XBC>(g.nx))
+            for (int q = 0; q < 38; ++q) mu[q] += Lin[RLB_CHK(q * S + idx - 1, 38ll * S)];
+    }
+    const int kl = unit_shift<38>(mu);
+    for (int q = 0; q < 38; ++q) mu[q] *= pow2d(kl);
     unsigned bounced = 0u;
-    double h[19], mug[19], muf[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) h[i] = A[RLB_CHK((19 + i) * S + idx + o.src(i), 38ll * S)];
 #pragma unroll
@@ -992,32 +1002,31 @@ __device__ __noinline__ double adjoint_cell_general(const double* A, const doubl
             h[i] = A[RLB_CHK((19 + opp(i)) * S + idx, 38ll * S)];
         }
     }
-    load_mu(mug, 19);
+    const int kh = unit_shift<19>(h);
+    for (int i = 0; i < 19; ++i) h[i] *= pow2d(kh);
     CellG<double> r;
     cell_g64(h, mug, c, r);
 #pragma unroll
     for (int i = 0; i < 19; ++i)
-        h[i] = (bounced >> i) & 1u ? A[RLB_CHK(opp(i) * S + idx, 38ll * S)] : A[RLB_CHK(i * S + idx + o.src(i), 38ll * S)];
-    load_mu(muf, 0);
+        h[i] = ((bounced >> i) & 1u ? A[RLB_CHK(opp(i) * S + idx, 38ll * S)] : A[RLB_CHK(i * S + idx + o.src(i), 38ll * S)]) * pow2d(kh);
     double tf, aS, fbx, fby, fbz, vE, vx, vy, vz;
     cell_f64(h, muf, r, c, tf, aS, fbx, fby, fbz);
     recovery_adjoint64(r.ae, fbx + r.gbx, fby + r.gby, fbz + r.gbz, r, c, vE, vx, vy, vz);
     scatter_cell64(muf, mug, aS, vE, vx, vy, vz, c, [&](int q, int i, double v) {
+        v *= pow2d(-kl);
         if ((bounced >> i) & 1u)
             Lout[RLB_CHK((q - i + opp(i)) * S + idx, 38ll * S)] = v;
         else
             Lout[RLB_CHK(q * S + idx + o.src(i), 38ll * S)] = v;
     });
-    return (r.tacc + tf) * c.inv_tau2;
+    return (r.tacc + tf) * c.inv_tau2 * pow2d(-kh) * pow2d(-kl);
 }
 
-// Whether the product sum dot 2^(ea + eb - 2102) of values with block
-// exponents ea and eb can be formed by fx_to, whose result has to be a normal
+// Whether products of values with block exponents ea and eb can be formed by
+// fx_to (sum mu h, units 2^(ea + eb - 2102)), whose result has to be a normal
 // number: otherwise (states of 1e-80 with lambda of 1e-230) the exponent would
 // wrap into the sign, and the cell is left to the binary64 form.
-__device__ __forceinline__ bool dot_in_range(int64_t dot, int ea, int eb) {
-    return dot == 0 || (ea + eb >= 1080 && ea + eb <= 3062);
-}
+__device__ __forceinline__ bool dot_in_range(int ea, int eb) { return (unsigned)(ea + eb - 1080) <= 1982u; }
 
 // What the f phase and the output need of a cell (see the formulas above).
 struct AdjFxCell {
@@ -1208,6 +1217,18 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
             for (int i = 0; i < 19; ++i) m = max(m, (uint32_t)__double2hiint(col[base + i][tid]) << 1);
             return (int)(m >> 21);
         };
+        // as a block exponent: 1023 for a set of zeros, 0x7FF (left to the
+        // binary64 form) for values all below 2^-923, which would lose bits
+        auto block_exp = [&](int base) {
+            int e = max_exp(base);
+            if (e < 100) {
+                bool any = false;
+#pragma unroll 1
+                for (int i = 0; i < 19; ++i) any |= col[base + i][tid] != 0.0;
+                e = any ? 0x7FF : 1023;
+            }
+            return e;
+        };
         // mu also takes lambda of the outflow ghosts that copy x
         auto add_dup = [&](int base) {
             for (int off = dup;; off = -1) {
@@ -1230,9 +1251,8 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         }
         if (dup) add_dup(19);
         // ---- g: moments of h and mu, their dot product
-        int em = max_exp(19);
-        bool ok = eh >= 100 && eh <= 1900 && em <= 1900;
-        em = em < 100 ? 100 : em;
+        const int em = block_exp(19);
+        bool ok = eh >= 600 && eh <= 1400 && em <= 1900 && dot_in_range(em, eh);  // E^2 in range
         int64_t E, dx = 0, dy = 0, dz = 0, m0;
         FxDot dot{};
         // moments of mu: axis sums, plane sums and differences (xy, yz, zx), V
@@ -1283,8 +1303,6 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                         zf = (float)(int32_t)(dz >> 32);
             ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
         }
-        const int64_t gdot = dot.result();
-        ok = ok && dot_in_range(gdot, em, eh);
         if (!ok) {
             cp_async_wait<0>();
             tau_acc += adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
@@ -1292,7 +1310,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
             continue;
         }
         AdjFxCell t;
-        adj_fx_g(E, dx, dy, dz, gdot, m0, Sx, Sy, Sz, Pxy, Pyz, Pzx, Txy, Tyz, Tzx, Vx, Vy, Vz, eh, em, ph, k, t);
+        adj_fx_g(E, dx, dy, dz, dot.result(), m0, Sx, Sy, Sz, Pxy, Pyz, Pzx, Txy, Tyz, Tzx, Vx, Vy, Vz, eh, em, ph, k, t);
         // ---- f
         cp_async_wait<0>();
         if (bounced) {
@@ -1302,10 +1320,8 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         }
         if (dup) add_dup(0);
         {
-            int fh = max_exp(38), ef = max_exp(0);
-            ok = fh <= 1900 && ef <= 1900;
-            fh = fh < 100 ? 100 : fh;
-            ef = ef < 100 ? 100 : ef;
+            const int fh = block_exp(38), ef = block_exp(0);
+            ok = fh <= 1900 && ef <= 1900 && dot_in_range(ef, fh);
             const int64_t h0 = fx_from(col[38][tid], fh), u0 = fx_from(col[0][tid], ef);
             int64_t Sf = fx_round4(h0);
             FxDot fd{};
@@ -1337,9 +1353,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                 Fx += dl, Fy -= dl;
                 rotate3(Fx, Fy, Fz);
             }
-            const int64_t fdot = fd.result();
-            ok = ok && dot_in_range(fdot, ef, fh);
-            adj_fx_f(Sf, fdot, Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
+            adj_fx_f(Sf, fd.result(), Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
         }
         if (!ok) {
             tau_acc += adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
@@ -1348,16 +1362,16 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         }
         tau_acc = fma(t.tsum, c.inv_tau2, tau_acc);
         // ---- nu = (1 - omega) mu + omega (...), scattered.  omega (v_E +
-        // e_i.v_d) as integers of one exponent; values beyond its range
-        // (ek >= 1900) are non-finite or about to overflow
+        // e_i.v_d) as integers of one exponent; values beyond its range are
+        // non-finite, about to overflow (ek >= 1900) or about to underflow
         const double nuE = t.nuE, nuS = t.nuS, kv[4] = {t.nuE, t.tx, t.ty, t.tz};
         int ek = fx_max_exponent<4>(kv);
+        if (ek < 100) ek = kv[0] == 0.0 && kv[1] == 0.0 && kv[2] == 0.0 && kv[3] == 0.0 ? 1023 : 1900;
         if (ek >= 1900) {
             adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
             zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
             continue;
         }
-        ek = ek < 100 ? 100 : ek;
         const int64_t kE = fx_from(nuE, ek);
         int64_t ka = fx_from(t.tx, ek), kb = fx_from(t.ty, ek), kc = fx_from(t.tz, ek);
         double* Lo = Lout + idx;
@@ -1447,7 +1461,13 @@ __global__ void __launch_bounds__(128)
             hg[n] = __ldg(A + RLB_CHK((19 + opp_rt(iv[n])) * S + idx, 38ll * S));
         }
     }
-    int eh = fx_max_exponent<4>(hg), em = fx_max_exponent<4>(ug), fh = fx_max_exponent<4>(hf), ef = fx_max_exponent<4>(uf);
+    // block exponents as in the kernel above: here 1 where values all below
+    // 2^-923 are, 0 for zeros
+    auto lane_exp = [](const double* v) {
+        const int e = fx_max_exponent<4>(v);
+        return e >= 100 ? e : (v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || v[3] != 0.0 ? 1 : 0);
+    };
+    int eh = fx_max_exponent<4>(hg), em = lane_exp(ug), fh = lane_exp(hf), ef = lane_exp(uf);
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) {
         eh = max(eh, __shfl_xor_sync(full, eh, off));
@@ -1455,8 +1475,9 @@ __global__ void __launch_bounds__(128)
         fh = max(fh, __shfl_xor_sync(full, fh, off));
         ef = max(ef, __shfl_xor_sync(full, ef, off));
     }
-    bool ok = eh >= 100 && eh <= 1900 && em <= 1900 && fh <= 1900 && ef <= 1900;
-    eh = max(eh, 100), em = max(em, 100), fh = max(fh, 100), ef = max(ef, 100);
+    auto block_exp = [](int e) { return e >= 100 ? e : (e ? 0x7FF : 1023); };
+    em = block_exp(em), fh = block_exp(fh), ef = block_exp(ef);
+    bool ok = eh >= 600 && eh <= 1400 && em <= 1900 && fh <= 1900 && ef <= 1900 && dot_in_range(em, eh) && dot_in_range(ef, fh);
     long long hx[4], ux[4];
     // g
 #pragma unroll
@@ -1510,7 +1531,6 @@ __global__ void __launch_bounds__(128)
     const int32_t Eh = (int32_t)(E >> 32);
     const float Ef = (float)Eh, xf = (float)(int32_t)(dx >> 32), yf = (float)(int32_t)(dy >> 32), zf = (float)(int32_t)(dz >> 32);
     ok = ok && Eh > 0 && fx_clz((uint32_t)Eh) <= 14 && xf * xf + yf * yf + zf * zf < ph.fx.m_max * (Ef * Ef);
-    ok = ok && dot_in_range(dot, em, eh) && dot_in_range(fd, ef, fh);
     AdjFxCell t;
     int ek = 0;
     if (ok) {
@@ -1519,8 +1539,8 @@ __global__ void __launch_bounds__(128)
         adj_fx_f(Sf, fd, Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
         const double kv[4] = {t.nuE, t.tx, t.ty, t.tz};
         ek = fx_max_exponent<4>(kv);
+        if (ek < 100) ek = kv[0] == 0.0 && kv[1] == 0.0 && kv[2] == 0.0 && kv[3] == 0.0 ? 1023 : 1900;
         ok = ek < 1900;
-        ek = max(ek, 100);
     }
     if (work && ok) {
         const int64_t kE = fx_from(t.nuE, ek), kx = fx_from(t.tx, ek), ky = fx_from(t.ty, ek), kz = fx_from(t.tz, ek);

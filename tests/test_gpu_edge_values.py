@@ -96,21 +96,26 @@ def test_adjoint_of_three_cells_between_outflow_ghosts(size, prec, c_l, env, mon
 
 
 @pytest.mark.parametrize("size", [(5, 4, 3), (23, 15, 15)], ids=["eight_lanes", "staged"])
-@pytest.mark.parametrize("sscale,lscale", [(1e-40, 1e-270), (1e-60, 1e-250), (1e-80, 1e-230), (1e60, 1e240)])
+@pytest.mark.parametrize("sscale,lscale", [(1e-40, 1e-270), (1e-60, 1e-250), (1e-80, 1e-230), (1e60, 1e240),
+                                           (1e-19, 1e-290), (1e-30, 1e-285), (1e-80, 1e-300), (1.0, 1e-290), (1.0, 1e-307),
+                                           (1e-80, 1e-240), (1e-170, 1.0), (1e170, 1e-20)])
 def test_fp64_adjoint_of_tiny_states_and_lambda(size, sscale, lscale):
-    """States and lambda whose products leave the range of binary64 (the terms
-    of dL/dtau underflow to zero) and lambda that loses bits itself: everything
-    finite and equal to the oracle.  Bounds: 1e-11 of the largest values, as at
-    scale one, and 64 smallest subnormals a cell for what underflows (57
-    products of a cell, the oracle's and the kernel's, to half of one each)."""
+    """States and lambda whose products (the terms of dL/dtau) or squares leave
+    the range of binary64, and lambda that loses bits itself.  lambda_t is
+    linear in lambda and does not depend on the unit of the state, so the
+    reference is the oracle's at order one, scaled.  Bounds: 1e-11 of the
+    largest values, as there, and 64 smallest subnormals a cell for what
+    underflows (57 products of a cell, to half of one each)."""
     w = tiny_workload(*size, 1, seed=3, bmax=0.5)
     p = oracle.Params(**w.params())
     st = oracle.init(p, w.n, w.eps, w.beta)
     oracle.run(p, st, 2)
-    st *= sscale
-    lam = np.random.default_rng(2).normal(size=st.shape) * lscale
+    lam = np.random.default_rng(2).normal(size=st.shape)
     lam[:, 0] = 0.0
-    got, ref = _adjoint_case(w, "fp64", st, lam)
+    ref = oracle.adjoint_step(p, st, lam)
+    ref = ref[0] * lscale, ref[1] * lscale * sscale, ref[2] * lscale
+    st, lam = st * sscale, lam * lscale
+    got = _adjoint_case(w, "fp64", st, lam)[0]
     big, tiny, N = np.abs(lam).max(), 5e-324 * 64, np.prod(size)
     assert np.isfinite(got[1]) and np.isfinite(got[0]).all()
     assert np.max(np.abs(got[0] - ref[0])) <= 1e-11 * np.abs(ref[0]).max() + tiny
