@@ -1211,23 +1211,11 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
             for (int q = 0; q < 38; ++q) Lout[RLB_CHK(q * S + idx, 38ll * S)] = col[q][tid];
             continue;
         }
-        auto max_exp = [&](int base) {
+        auto max_word = [&](int base) {
             uint32_t m = 0;
 #pragma unroll 4
             for (int i = 0; i < 19; ++i) m = max(m, (uint32_t)__double2hiint(col[base + i][tid]) << 1);
-            return (int)(m >> 21);
-        };
-        // as a block exponent: 1023 for a set of zeros, 0x7FF (left to the
-        // binary64 form) for values all below 2^-923, which would lose bits
-        auto block_exp = [&](int base) {
-            int e = max_exp(base);
-            if (e < 100) {
-                bool any = false;
-#pragma unroll 1
-                for (int i = 0; i < 19; ++i) any |= col[base + i][tid] != 0.0;
-                e = any ? 0x7FF : 1023;
-            }
-            return e;
+            return m;
         };
         // mu also takes lambda of the outflow ghosts that copy x
         auto add_dup = [&](int base) {
@@ -1237,7 +1225,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                 if (!dup_both<XBC>(g.nx) || off < 0) break;
             }
         };
-        int eh = max_exp(38);
+        int eh = (int)(max_word(38) >> 21);
         unsigned bounced = 0u;
         if (eh == 0x7FF) {  // links to solid cells, or a non-finite population
 #pragma unroll 1
@@ -1247,11 +1235,11 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                     col[38 + i][tid] = Ac[RLB_CHK_OFF((19 + opp_rt(i)) * S, idx, 38ll * S)];
                 }
             }
-            eh = max_exp(38);
+            eh = (int)(max_word(38) >> 21);
         }
         if (dup) add_dup(19);
         // ---- g: moments of h and mu, their dot product
-        const int em = block_exp(19);
+        const int em = fx_block_exponent(max_word(19));
         bool ok = eh >= 600 && eh <= 1400 && em <= 1900 && dot_in_range(em, eh);  // E^2 in range
         int64_t E, dx = 0, dy = 0, dz = 0, m0;
         FxDot dot{};
@@ -1320,7 +1308,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         }
         if (dup) add_dup(0);
         {
-            const int fh = block_exp(38), ef = block_exp(0);
+            const int fh = fx_block_exponent(max_word(38)), ef = fx_block_exponent(max_word(0));
             ok = fh <= 1900 && ef <= 1900 && dot_in_range(ef, fh);
             const int64_t h0 = fx_from(col[38][tid], fh), u0 = fx_from(col[0][tid], ef);
             int64_t Sf = fx_round4(h0);
@@ -1365,8 +1353,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
         // e_i.v_d) as integers of one exponent; values beyond its range are
         // non-finite, about to overflow (ek >= 1900) or about to underflow
         const double nuE = t.nuE, nuS = t.nuS, kv[4] = {t.nuE, t.tx, t.ty, t.tz};
-        int ek = fx_max_exponent<4>(kv);
-        if (ek < 100) ek = kv[0] == 0.0 && kv[1] == 0.0 && kv[2] == 0.0 && kv[3] == 0.0 ? 1023 : 1900;
+        const int ek = fx_block_exponent(fx_max_word<4>(kv));
         if (ek >= 1900) {
             adjoint_cell_general<XBC>(A, Lin, Lout, g, c, idx);
             zero_to_ghost<double, XBC>(x, g.nx, idx, S, Lout);
@@ -1461,22 +1448,15 @@ __global__ void __launch_bounds__(128)
             hg[n] = __ldg(A + RLB_CHK((19 + opp_rt(iv[n])) * S + idx, 38ll * S));
         }
     }
-    // block exponents as in the kernel above: here 1 where values all below
-    // 2^-923 are, 0 for zeros
-    auto lane_exp = [](const double* v) {
-        const int e = fx_max_exponent<4>(v);
-        return e >= 100 ? e : (v[0] != 0.0 || v[1] != 0.0 || v[2] != 0.0 || v[3] != 0.0 ? 1 : 0);
-    };
-    int eh = fx_max_exponent<4>(hg), em = lane_exp(ug), fh = lane_exp(hf), ef = lane_exp(uf);
+    uint32_t wh = fx_max_word<4>(hg), wm = fx_max_word<4>(ug), vh = fx_max_word<4>(hf), vm = fx_max_word<4>(uf);
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) {
-        eh = max(eh, __shfl_xor_sync(full, eh, off));
-        em = max(em, __shfl_xor_sync(full, em, off));
-        fh = max(fh, __shfl_xor_sync(full, fh, off));
-        ef = max(ef, __shfl_xor_sync(full, ef, off));
+        wh = max(wh, __shfl_xor_sync(full, wh, off));
+        wm = max(wm, __shfl_xor_sync(full, wm, off));
+        vh = max(vh, __shfl_xor_sync(full, vh, off));
+        vm = max(vm, __shfl_xor_sync(full, vm, off));
     }
-    auto block_exp = [](int e) { return e >= 100 ? e : (e ? 0x7FF : 1023); };
-    em = block_exp(em), fh = block_exp(fh), ef = block_exp(ef);
+    const int eh = (int)(wh >> 21), em = fx_block_exponent(wm), fh = fx_block_exponent(vh), ef = fx_block_exponent(vm);
     bool ok = eh >= 600 && eh <= 1400 && em <= 1900 && fh <= 1900 && ef <= 1900 && dot_in_range(em, eh) && dot_in_range(ef, fh);
     long long hx[4], ux[4];
     // g
@@ -1538,8 +1518,7 @@ __global__ void __launch_bounds__(128)
                  v[7] - v[8], v[5] - v[6], Vx, Vy, Vz, eh, em, ph, k, t);
         adj_fx_f(Sf, fd, Fs, Fx, Fy, Fz, fh, ef, ph, k, t);
         const double kv[4] = {t.nuE, t.tx, t.ty, t.tz};
-        ek = fx_max_exponent<4>(kv);
-        if (ek < 100) ek = kv[0] == 0.0 && kv[1] == 0.0 && kv[2] == 0.0 && kv[3] == 0.0 ? 1023 : 1900;
+        ek = fx_block_exponent(fx_max_word<4>(kv));
         ok = ek < 1900;
     }
     if (work && ok) {

@@ -139,9 +139,10 @@ RLB_FX uint64_t fx_shr(uint64_t v, uint32_t s) {
 #endif
 }
 
-// Largest binary64 exponent field of n values; 0x7FF when one is not finite.
+// Largest high word of N values without the sign, times 2; the binary64
+// exponent field of the largest (0x7FF when one is not finite).
 template <int N>
-RLB_FX int fx_max_exponent(const double* v) {
+RLB_FX uint32_t fx_max_word(const double* v) {
     uint32_t m = 0;
 #ifdef __CUDA_ARCH__
 #pragma unroll
@@ -150,8 +151,16 @@ RLB_FX int fx_max_exponent(const double* v) {
         const uint32_t t = (uint32_t)fx_hi(v[i]) << 1;
         m = t > m ? t : m;
     }
-    return (int)(m >> 21);
+    return m;
 }
+template <int N>
+RLB_FX int fx_max_exponent(const double* v) {
+    return (int)(fx_max_word<N>(v) >> 21);
+}
+// The block exponent of values with the largest word m: 1023 for zeros (values
+// below 2^-1042 count as zero), and 0x7FF, as for non-finite ones, when all lie
+// below 2^-923, where fx_from would keep too few of their bits.
+RLB_FX int fx_block_exponent(uint32_t m) { return m >= 100u << 21 ? (int)(m >> 21) : (m ? 0x7FF : 1023); }
 
 // v 2^60 / 2^(emax - 1023), truncated towards zero; |result| < 2^61.
 RLB_FX int64_t fx_from(double v, int emax) {
