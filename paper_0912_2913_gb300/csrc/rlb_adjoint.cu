@@ -2233,15 +2233,14 @@ __global__ void __launch_bounds__(128, 4) k_adjoint_fields(const double* __restr
             for (int i = 0; i < 19; ++i) lg[i] = __ldg(RLB_CHK_PTR(lam, (19 + i) * S + idx, 38ll * S));
 #pragma unroll
             for (int i = 0; i < 19; ++i) lf[i] = __ldg(RLB_CHK_PTR(lam, i * S + idx, 38ll * S));
-            constexpr int BIAS = sizeof(T) == 4 ? 127 : 1023, LO = sizeof(T) == 4 ? 64 : 100, HI = sizeof(T) == 4 ? 250 : 1900;
-            int em = fx_max_exponent<19>(lg), ef = fx_max_exponent<19>(lf);
+            constexpr int BIAS = sizeof(T) == 4 ? 127 : 1023, HI = sizeof(T) == 4 ? 250 : 1900;
+            int um, uf;
+            const int em = fx_block_exponent<19>(lg, um), ef = fx_block_exponent<19>(lf, uf);
             const double b2 = fma(bx, bx, fma(by, by, bz * bz));
             const double omb2 = 1.0 - b2;
             const int oh = __double2hiint(omb2);
             if (em <= HI && ef <= HI && oh > 0x3F900000 && oh < 0x3FF00001) {
-                em = em < LO ? LO : em;
-                ef = ef < LO ? LO : ef;
-                const int km = em - BIAS - 56, kf = ef - BIAS - 56;
+                const int km = em - BIAS - 56 - um, kf = ef - BIAS - 56 - uf;
                 int64_t Sx = 0, Sy = 0, Sz = 0, Pxy = 0, Pxz = 0, Pyz = 0, Txy = 0, Txz = 0, Tyz = 0, Vx = 0, Vy = 0, Vz = 0;
                 int64_t Fx = 0, Fy = 0, Fz = 0;
                 const int64_t m0 = fx_round4(fx_from(lg[0], em)), u0 = fx_round4(fx_from(lf[0], ef));
@@ -2288,7 +2287,10 @@ __global__ void __launch_bounds__(128, 4) k_adjoint_fields(const double* __restr
                 az = fma(cy, yz, fma(cv, vz, fma(ng, fz, cs * bz)));
             } else {
                 double df[19], dg[19];
-                for (int i = 0; i < 19; ++i) df[i] = (double)lf[i], dg[i] = (double)lg[i];
+                for (int i = 0; i < 19; ++i) {
+                    df[i] = (double)lf[i] * (uf ? 0x1p-96 : 1.0);
+                    dg[i] = (double)lg[i] * (um ? 0x1p-96 : 1.0);
+                }
                 eq_fields_adjoint(df, dg, n, e, bx, by, bz, ph, an, ae, ax, ay, az);
             }
             if (inflow) {

@@ -494,14 +494,38 @@ __device__ __forceinline__ int64_t fx_from(float v, int emax) {
     return (int64_t)((x ^ (uint64_t)s) - (uint64_t)s);
 }
 template <int N>
-__device__ __forceinline__ int fx_max_exponent(const float* v) {
+__device__ __forceinline__ uint32_t fx_max_word(const float* v) {
     uint32_t m = 0;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const uint32_t t = __float_as_uint(v[i]) << 1;
         m = t > m ? t : m;
     }
-    return (int)(m >> 24);
+    return m;
+}
+template <int N>
+__device__ __forceinline__ int fx_max_exponent(const float* v) {
+    return (int)(fx_max_word<N>(v) >> 24);
+}
+// The block exponent of N binary32 values for fx_from, which reads subnormals
+// as normal numbers and shifts zeros out from an exponent of 61 on only: values
+// all below 2^-63 are brought up by 2^96 (exactly) and `lift` says so.
+template <int N>
+__device__ __forceinline__ int fx_block_exponent(float* v, int& lift) {
+    int e = fx_max_exponent<N>(v);
+    lift = 0;
+    if (e < 64) {
+        lift = 96;
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] *= 0x1p96f;
+        e = max(fx_max_exponent<N>(v), 64);
+    }
+    return e;
+}
+template <int N>
+__device__ __forceinline__ int fx_block_exponent(double* v, int& lift) {
+    lift = 0;
+    return fx_block_exponent(fx_max_word<N>(v));
 }
 
 // The moments of a stored state's cell: E, S and d = M / c_l in binary64 (d

@@ -163,3 +163,34 @@ def test_dtau_has_no_common_rounding_error():
         want = math.fsum([want] + t.ravel().tolist())
     sigma = U * np.sqrt(2 * 40 / 12) * np.sqrt(((lam * st) ** 2).sum())
     assert abs(got - want) <= 4 * sigma, (got - want, sigma)
+
+
+@pytest.mark.parametrize("prec,lscale", [("fp32", 1e-20), ("fp32", 1e-29), ("fp32", 1e-34), ("fp32", 1e-37), ("fp32", 1e-40),
+                                         ("fp64", 1e-279), ("fp64", 1e-290), ("fp64", 1e-305), ("fp64", 1e-312)])
+def test_field_adjoints_of_tiny_lambda(prec, lscale):
+    """Gradients of the initial fields for lambda far below one, zero in part
+    of the lattice, and one cell whose f lambdas alone are tiny; bounds as at
+    scale one (64 roundings times gamma^2), and 64 smallest subnormals."""
+    from paper_0912_2913_gb300 import RLB
+
+    rng = np.random.default_rng(9)
+    shape = (3, 5, 41)
+    w = tiny_workload(41, 5, 3, 1, seed=9, bmax=0.5)
+    p = oracle.Params(**w.params())
+    sim = RLB.from_workload(w, prec, device="cuda:0").init_fields(w.n, w.eps, w.beta)
+    l0 = rng.normal(size=shape + (2, 19)) * lscale
+    l0[0, 1] = 0.0
+    l0[1, 1, 7, 1] = rng.normal(size=19)
+    ls = sim.cells_to_state(_cuda(l0))
+    l0 = sim.state_to_cells(ls).double().cpu().numpy()
+    outs = [torch.empty(shape, dtype=torch.float64, device="cuda") for _ in range(2)]
+    db, acc = torch.empty((3,) + shape, dtype=torch.float64, device="cuda"), torch.zeros(3, dtype=torch.float64, device="cuda")
+    sim.adjoint_fields(_cuda(w.n), _cuda(w.eps), _cuda(w.beta), ls, outs[0], outs[1], db, acc)
+    ref = oracle.adjoint_fields(p, w.n, w.eps, w.beta, np.ascontiguousarray(l0))
+    sim.close()
+    gam2 = 1 / (1 - (w.beta * w.beta).sum(0))
+    big, bigf, tiny = np.abs(l0).max((-1, -2)) * gam2, np.abs(l0[..., 0, :]).max(-1) * gam2, 5e-324 * 64
+    assert np.all(np.abs(outs[0].cpu().numpy() - ref[0]) <= 64 * U * gam2 * bigf + tiny)
+    assert np.all(np.abs(outs[1].cpu().numpy() - ref[1]) <= 64 * U * gam2 * big * 8 + tiny)
+    assert np.all(np.abs(db.cpu().numpy() - ref[2]) <= 64 * U * gam2 ** 2 * big * 16 * (w.n + w.eps) + tiny)
+    assert np.all(np.abs(acc.cpu().numpy() - ref[3]) <= 64 * U * 41 * 15 * np.abs(l0).max() * 16 * 4 + tiny * 615)
