@@ -2096,7 +2096,7 @@ __global__ void __launch_bounds__(128, 6) k_adjoint_macro(const T* __restrict__ 
     T h[19], f[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) f[i] = __ldg(RLB_CHK_PTR(A, i * S + idx, 38ll * S));
-    if (is_solid(f[0]) || (gn == 0.0 && ge == 0.0 && gx == 0.0 && gy == 0.0 && gz == 0.0)) {
+    if (is_solid(f[0])) {
 #pragma unroll
         for (int q = 0; q < 38; ++q) put(q, (T)0);
         return;
@@ -2105,6 +2105,11 @@ __global__ void __launch_bounds__(128, 6) k_adjoint_macro(const T* __restrict__ 
     for (int i = 0; i < 19; ++i) h[i] = __ldg(RLB_CHK_PTR(A, (19 + i) * S + idx, 38ll * S));
     FxMoments m;
     if (fx_moments(h, f, ph.fx.m3cl2, ph.n_ref, ph.eps_ref, m)) {
+        if (gn == 0.0 && ge == 0.0 && gx == 0.0 && gy == 0.0 && gz == 0.0) {  // zero only where the fields exist
+#pragma unroll
+            for (int q = 0; q < 38; ++q) put(q, (T)0);
+            return;
+        }
         const double E2 = m.E + m.E;
         double ys, hs;
         rsqrt_seed(m.disc, ys, hs);

@@ -194,3 +194,28 @@ def test_field_adjoints_of_tiny_lambda(prec, lscale):
     assert np.all(np.abs(outs[1].cpu().numpy() - ref[1]) <= 64 * U * gam2 * big * 8 + tiny)
     assert np.all(np.abs(db.cpu().numpy() - ref[2]) <= 64 * U * gam2 ** 2 * big * 16 * (w.n + w.eps) + tiny)
     assert np.all(np.abs(acc.cpu().numpy() - ref[3]) <= 64 * U * 41 * 15 * np.abs(l0).max() * 16 * 4 + tiny * 615)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_macro_adjoint_of_cells_without_a_gradient(prec):
+    """A cell with zero output gradients: lambda is zero where the fields exist
+    and not a number where they do not (a non-finite population, |M| > 2E /
+    sqrt 3), as zero times the undefined derivative is."""
+    from paper_0912_2913_gb300 import RLB
+
+    w = tiny_workload(9, 4, 3, 0, seed=4)
+    sim = RLB.from_workload(w, prec, device="cuda:0").init_fields(w.n, w.eps, w.beta)
+    s = sim.state()
+    s[19 + 3, 5] = float("nan")
+    s[19 + 4, 20] = float("inf")
+    s[19 + 1, 33], s[19 + 2, 33] = 40.0, -40.0  # |M| beyond E
+    s[2, 50] = float("nan")
+    z = torch.zeros((3, 4, 9), dtype=torch.float64, device="cuda")
+    zb = torch.zeros((3, 3, 4, 9), dtype=torch.float64, device="cuda")
+    lam = sim.new_state()
+    sim.adjoint_macro(s, z, z, zb, lam)
+    nan = torch.isnan(lam[:, :sim.N]).any(0).cpu().numpy()
+    rest = lam[:, :sim.N][:, torch.from_numpy(~nan).cuda()]
+    sim.close()
+    assert set(np.nonzero(nan)[0]) == {5, 20, 33, 50}
+    assert bool((rest == 0).all())
