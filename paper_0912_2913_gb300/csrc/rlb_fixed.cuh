@@ -72,6 +72,7 @@ struct FxRun {
     double three_cl;
     float m_max;  // largest |M|^2 / (c_l^2 E^2) of the fast path
     float q_scale;  // beta = q_scale x (high word of w)
+    float q_margin;  // of the positivity decision on that beta
     float c_l;
 };
 

@@ -219,3 +219,37 @@ def test_macro_adjoint_of_cells_without_a_gradient(prec):
     sim.close()
     assert set(np.nonzero(nan)[0]) == {5, 20, 33, 50}
     assert bool((rest == 0).all())
+
+
+@pytest.mark.parametrize("tau", [1e4, 1e6, 1e9])
+@pytest.mark.parametrize("split", ["0", "1"])
+def test_positivity_count_at_large_tau(tau, split, monkeypatch):
+    """The positivity decision in binary32 near its threshold at |q| = 1/3, for
+    relaxation times far above the usual ones."""
+    from paper_0912_2913_gb300 import RLB
+
+    monkeypatch.setenv("RLB_F64_SPLIT", split)
+    shape = (4, 8, 64)
+    N = int(np.prod(shape))
+    rng = np.random.default_rng(3)
+    b = np.zeros((3, N))
+    grid = np.linspace(0.31, 0.36, N)
+    b[0] = grid
+    b[:, ::2] = rng.normal(size=(3, N))[:, ::2]
+    b[:, ::2] *= grid[::2] / np.abs(b[:, ::2]).sum(0)
+    n, e, b = np.ones(shape), np.ones(shape), b.reshape((3,) + shape)
+    p = oracle.Params(nx=64, ny=8, nz=4, tau=tau)
+    a = oracle.init(p, n, e, b)
+    ev = np.asarray(oracle.lattice()[0], int)
+    s = np.empty_like(a)
+    for i in range(19):
+        s[..., i] = np.roll(a[..., i], tuple(-ev[i][c] for c in (2, 1, 0)), axis=(0, 1, 2))
+    stats = oracle.Stats()
+    oracle.step(p, s, stats=stats)
+    sim = RLB(64, 8, 4, tau, precision="fp64", device="cuda:0")
+    sim.load_state(sim.cells_to_state(_cuda(s)))
+    sim.step(1)
+    got = sim.stats()["n_nonpositive_eq"]
+    sim.close()
+    assert 0.1 * N < stats.n_nonpositive_eq < 0.9 * N
+    assert got == stats.n_nonpositive_eq
