@@ -219,15 +219,17 @@ RLB_API rlb_status rlb_adjoint_step(rlb_ctx* ctx, const void* state_t, const voi
  * capped at the lattice's block count.  The per-warp partial sums live in one static
  * device array of 32768 doubles (256 KiB) per device: a launch that would
  * need more (4 doubles per warp) returns RLB_ERR_ARG and enqueues nothing;
- * every launch writes all the slots it reads, so nothing needs to start at
- * zero.  The first call on each device (and the first after the device's
+ * every launch writes all the slots it reads.  The counter by which the blocks
+ * of an FP64 launch find the last of them is the context's own; rlb_create and
+ * rlb_init_fields set it to zero and every launch leaves it there.  The first call on each device (and the first after the device's
  * context was reset) does the set-up: it takes the array's address and loads
  * every kernel this entry point launches, which may allocate and
  * synchronise, so make that first call before any stream capture and before
  * the code that must not allocate; later calls allocate nothing.  The
  * context's device must be current.  Calls that overlap in time on one
- * device (different streams or contexts) share the array and race:
- * serialise them.                                                          */
+ * device (different contexts) share the array and race: serialise them.  What
+ * they spoil is their own sums; replays of one context's captured calls that
+ * overlap can leave its counter off until the next rlb_init_fields.         */
 RLB_API rlb_status rlb_adjoint_step_noalloc(rlb_ctx* ctx, const void* state_t, const void* lam_in, void* lam_out,
                                             double* dL_dtau_accum, double* dL_dbeta_in_accum);
 

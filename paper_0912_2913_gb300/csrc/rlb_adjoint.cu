@@ -181,7 +181,9 @@ __device__ __forceinline__ void block_reduce4(double v0, double v1, double v2, d
 
 // Where a persistent adjoint kernel leaves its sums: red[block*4 + k], then,
 // by the last block to arrive at the ticket (which it resets to 0), the sum
-// over the blocks added to the accumulators.
+// over the blocks added to the accumulators.  The ticket is the context's, also
+// where red is shared by all contexts of a device: launches of two contexts
+// that overlap spoil their own sums, not those of later ones.
 struct AdjSums {
     double* red;
     unsigned* ticket;
@@ -2539,14 +2541,12 @@ cudaError_t launch_adjoint_fields(int prec, const Geom& g, const Phys& ph, const
 // race.
 // ---------------------------------------------------------------------------
 static __device__ __align__(256) double g_adj_scratch[kAdjScratchDoubles];
-static __device__ unsigned g_adj_ticket;
 
 namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mu;
 struct ScratchSetup {
     double* ptr;    // device address of g_adj_scratch in the context below
-    unsigned* ticket;  // and of g_adj_ticket
     int nsm;        // SM count of the device
     CUcontext ctx;  // the context the set-up was made in
 };
@@ -2558,7 +2558,7 @@ ScratchSetup g_scratch[kMaxDevices];
 // not loaded yet), so that no later call loads code, which can allocate.
 // Redone when the device's context is not the one it was made in (after
 // cudaDeviceReset the old address is stale).
-cudaError_t scratch_for_device(int dev, double** ptr, unsigned** ticket, int* nsm) {
+cudaError_t scratch_for_device(int dev, double** ptr, int* nsm) {
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     const CUcontext ctx = current_context();
     std::lock_guard<std::mutex> lock(g_scratch_mu);
@@ -2567,8 +2567,6 @@ cudaError_t scratch_for_device(int dev, double** ptr, unsigned** ticket, int* ns
         s.ptr = nullptr;
         double* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress((void**)&p, g_adj_scratch);
-        if (e != cudaSuccess) return e;
-        e = cudaGetSymbolAddress((void**)&s.ticket, g_adj_ticket);
         if (e != cudaSuccess) return e;
         int n = 0;
         e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
@@ -2611,7 +2609,6 @@ cudaError_t scratch_for_device(int dev, double** ptr, unsigned** ticket, int* ns
         s.ptr = p;
     }
     *ptr = s.ptr;
-    *ticket = s.ticket;
     *nsm = s.nsm;
     return cudaSuccess;
 }
@@ -2637,16 +2634,15 @@ int adjoint_step_noalloc_t(const Geom& g, const Phys& ph, const T* A, const T* L
 }  // namespace
 
 cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph, const void* A, const void* lam_in,
-                                        void* lam_out, const double* inflow_d, double* dtau, double* dbeta_in,
-                                        cudaStream_t st, long long* need_doubles) {
+                                        void* lam_out, unsigned* ticket, const double* inflow_d, double* dtau,
+                                        double* dbeta_in, cudaStream_t st, long long* need_doubles) {
     set_last_launch_count(0);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     double* red = nullptr;
     int nsm = 0;
-    unsigned* ticket = nullptr;
-    e = scratch_for_device(dev, &red, &ticket, &nsm);
+    e = scratch_for_device(dev, &red, &nsm);
     const AdjSums sums{red, ticket, dtau, dbeta_in};
     if (e != cudaSuccess) return e;
     const int nb = adj_blocks(g.N);

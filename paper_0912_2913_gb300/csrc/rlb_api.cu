@@ -151,7 +151,8 @@ rlb_status reset_counters(rlb_ctx* c) {
     RLB_CUDA(c, cudaMemsetAsync(c->cnt.slots, 0, sizeof(unsigned long long) * 2 * kCounterSlots, c->stream),
              "reset counters");
     RLB_CUDA(c, cudaMemsetAsync(c->cnt.first_bad, 0xff, sizeof(unsigned long long), c->stream), "reset counters");
-    RLB_CUDA(c, cudaMemsetAsync(c->cnt.macro_bad, 0, 2 * sizeof(unsigned long long), c->stream), "reset counters");
+    // macro_bad, pipe_err and the adjoint's ticket follow one another
+    RLB_CUDA(c, cudaMemsetAsync(c->cnt.macro_bad, 0, 3 * sizeof(unsigned long long), c->stream), "reset counters");
     return RLB_OK;
 }
 
@@ -306,10 +307,6 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
     c->inflow_d = (double*)(base + 2 * sb + align_up(sizeof(unsigned long long) * (2 * kCounterSlots + 4), kAlign));
     c->red = (double*)(base + 2 * sb + counters_bytes());
     s = reset_counters(c);
-    if (s == RLB_OK) {
-        e = cudaMemsetAsync(c->cnt.adj_ticket, 0, sizeof(unsigned long long), c->stream);
-        if (e != cudaSuccess) s = cuda_fail(c, e, "reset ticket");
-    }
     if (s == RLB_OK) s = after_launch(c, launch_inflow_derivs(c->ph, c->inflow_d, c->stream), "inflow table");
     if (s != RLB_OK) {
         rlb_destroy(c);
@@ -560,8 +557,8 @@ rlb_status rlb_adjoint_step_noalloc(rlb_ctx* c, const void* state_t, const void*
         return fail(c, RLB_ERR_STATE, "rlb_adjoint_step_noalloc: the context's device %d is not current (%d is)",
                     c->device, dev);
     long long need = 0;
-    e = launch_adjoint_step_noalloc(c->p.prec, c->g, c->ph, state_t, lam_in, lam_out, c->inflow_d, dL_dtau_accum,
-                                    dL_dbeta_in_accum, c->stream, &need);
+    e = launch_adjoint_step_noalloc(c->p.prec, c->g, c->ph, state_t, lam_in, lam_out, c->cnt.adj_ticket, c->inflow_d,
+                                    dL_dtau_accum, dL_dbeta_in_accum, c->stream, &need);
     if (e == cudaErrorInvalidValue && need > kAdjScratchDoubles)
         return fail(c, RLB_ERR_ARG,
                     "rlb_adjoint_step_noalloc: the launch needs %lld scratch doubles, the static maximum is %lld",

@@ -135,8 +135,8 @@ cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const v
 // nothing, when that exceeds the array.
 constexpr long long kAdjScratchDoubles = 32768;  // 256 KiB
 cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph, const void* A, const void* lam_in,
-                                        void* lam_out, const double* inflow_d, double* dtau, double* dbeta_in,
-                                        cudaStream_t stream, long long* need_doubles);
+                                        void* lam_out, unsigned* ticket, const double* inflow_d, double* dtau,
+                                        double* dbeta_in, cudaStream_t stream, long long* need_doubles);
 // d eq_in / d beta_in table of the inflow state: kInflowTable doubles
 // followed by the same kInflowTable values rounded to binary32 (the FP32
 // adjoint kernels read the float copy, so their ghost cells convert nothing).

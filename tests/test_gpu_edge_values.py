@@ -253,3 +253,34 @@ def test_positivity_count_at_large_tau(tau, split, monkeypatch):
     sim.close()
     assert 0.1 * N < stats.n_nonpositive_eq < 0.9 * N
     assert got == stats.n_nonpositive_eq
+
+
+def test_a_stale_adjoint_ticket_ends_with_the_next_initialisation():
+    """The blocks of an FP64 adjoint step draw a ticket of their own context;
+    whatever an interrupted or overlapped launch left in it, rlb_init_fields
+    starts it afresh, and another context never sees it."""
+    from paper_0912_2913_gb300 import RLB
+    from paper_0912_2913_gb300 import _native as N
+
+    w = tiny_workload(23, 15, 15, 1, seed=6)
+    sims = [RLB.from_workload(w, "fp64", device="cuda:0").init_fields(w.n, w.eps, w.beta) for _ in range(2)]
+    lam = [torch.randn(sims[0].state().shape, dtype=torch.float64, device="cuda") for _ in range(2)]
+
+    def sums(sim, noalloc):
+        acc = torch.zeros(4, dtype=torch.float64, device="cuda")
+        f = (lambda *a: N.rlb_adjoint_step_noalloc(sim.ctx, *a)) if noalloc else sim.adjoint_step
+        f(sim.state(), lam[0], lam[1], acc[0:1], acc[1:4])
+        return acc.cpu()
+
+    want = [sums(sims[0], k) for k in (False, True)]
+    assert torch.equal(*want)
+    # the ticket is the fourth word behind the 2 x 4096 statistics slots
+    at = 2 * ((sims[0].state_bytes + 255) // 256 * 256) + 8 * (2 * 4096 + 3)
+    sims[0].ws[at] = 3
+    for k in (False, True):
+        assert torch.equal(sums(sims[1], k), want[0])
+    sims[0].init_fields(w.n, w.eps, w.beta)
+    for k in (False, True):
+        assert torch.equal(sums(sims[0], k), want[0])
+    for s in sims:
+        s.close()
