@@ -274,10 +274,10 @@ rlb_status rlb_create(const rlb_params* p, void* stream, void* workspace, size_t
     ph.three_cl = 3.0 * p->c_l;
     ph.fx = make_fx_run(ph.omega, p->c_l);
     ph.fi = make_fx_init(ph, p->prec);
-    // the fixed-point FP64 step: measured closer to the exact values than the
-    // binary64 one for lattice speeds up to 3 (rlb_fixed.cuh); its cell
-    // offsets are 32-bit byte counts
-    ph.fx_on = p->eos == RLB_EOS_ULTRA && p->c_l >= 1.0 && p->c_l <= 2.0 && S < (1ll << 29) ? 1 : 0;
+    // the fixed-point FP64 step: closer to the exact values than the binary64
+    // one at these lattice speeds (k_step_f64_fx); its cell offsets are 32-bit
+    // byte counts
+    ph.fx_on = p->eos == RLB_EOS_ULTRA && fx_covers(p->c_l) && S < (1ll << 29) ? 1 : 0;
     ph.eos = p->eos;
     ph.eos_gamma = p->eos == RLB_EOS_GAMMA_LAW ? p->eos_gamma : 4.0 / 3.0;
     ph.eos_mass = p->eos == RLB_EOS_GAMMA_LAW ? p->eos_mass : 0.0;

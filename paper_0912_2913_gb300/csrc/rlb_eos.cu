@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(128, 5) k_macro_eos(const double* __restrict__
 }
 
 // The fixed-point kernels cover 1 <= c_l <= 2 (see k_step_f64_fx).
-bool eos_fx_on(const Phys& ph) { return ph.c_l >= 1.0 && ph.c_l <= 2.0; }
+bool eos_fx_on(const Phys& ph) { return fx_covers(ph.c_l); }
 
 // num / (den c_l^2) x 2^s
 FxConst over_c2(const Phys& ph, double num, double den, int s) {
@@ -645,7 +645,8 @@ FxConst over_c2(const Phys& ph, double num, double den, int s) {
 }
 
 FxEosInit make_fx_eos_init(const Phys& ph) {
-    FxEosInit k;
+    FxEosInit k{};
+    if (!ph.fi.on) return k;
     k.k8 = over_c2(ph, 1.0, 8.0, 65);
     k.kP = over_c2(ph, 1.0, 12.0, 65);
     k.kc2 = over_c2(ph, 1.0, 1.0, 62);

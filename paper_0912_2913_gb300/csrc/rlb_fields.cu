@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(128, 6) k_macro(const T* __restrict__ A, doubl
 // Launchers
 // ---------------------------------------------------------------------------
 FxInit make_fx_init(const Phys& ph, int prec) {
-    FxInit k;
+    FxInit k{};
     const double c = ph.c_l, c2 = c * c, c2l = fma(c, c, -c2);
     // num / (den c_l^2) and num / (den c_l) as constants times 2^s
     auto over_c2 = [&](double num, double den, int s) {

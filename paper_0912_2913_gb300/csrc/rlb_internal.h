@@ -94,8 +94,6 @@ cudaError_t launch_macro(int prec, const Geom& g, const Phys& ph, const void* A,
 // FP64 step (rlb_step64.cu).
 cudaError_t launch_step_f64(const Geom& g, const Phys& ph, const void* A, void* B, Counters cnt, bool count,
                             long long step_index, cudaStream_t stream);
-// Constants of the fixed-point FP64 step.
-FxRun make_fx_run(double omega, double c_l);
 // Constants of the fixed-point initialisation (c_l and the reference of ph).
 FxInit make_fx_init(const Phys& ph, int prec);
 // FP64 step with its arithmetic in compensated binary32 pairs (rlb_f64df.cu).

@@ -743,41 +743,6 @@ void launch_step_f64_t(const Geom& g, const Phys& ph, const double* A, double* B
 }
 }  // namespace
 
-FxRun make_fx_run(double omega, double c_l) {
-    FxRun k;
-    double qh, ql, th, tl, c2h = c_l * c_l, c2l = fma(c_l, c_l, -c2h);
-    fx_div2(omega, 36.0, qh, ql);
-    th = qh / c2h;
-    tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
-    k.kE = fx_const_w(th, tl, 65);
-    k.kS = fx_const_w(qh, ql, 65);
-    fx_div2(omega, 12.0, qh, ql);
-    k.kU = fx_const_w(qh, ql, 65);
-    // omega (1 - 2 / (3 c_l^2)) = omega - 24 omega / (36 c_l^2)
-    const int64_t kE65 = (int64_t)ldexp(th, 65) + (int64_t)llrint(ldexp(tl, 65));
-    const int64_t v = (int64_t)ldexp(omega, 62) - 3 * kE65;
-    k.k0 = fx_const(v - (v >> 54));
-    fx_div2(1.0, 36.0, qh, ql);
-    th = qh / c2h;
-    tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
-    k.kE1 = fx_const_w(th, tl, 65);
-    // (3 - 2 / c_l^2) / 3 = 1 - 24 / (36 c_l^2)
-    k.kE0 = fx_const_w(1.0 - 24.0 * th, fma(-24.0, th, 1.0) - (1.0 - 24.0 * th) - 24.0 * tl, 62);
-    fx_div2(5.0, 9.0, qh, ql);
-    k.kQ = fx_const(qh, ql, 63);
-    fx_div2(1.0, 6.0, qh, ql);
-    k.kG = fx_const(qh, ql, 63);
-    k.om4 = 0.25 * omega;
-    k.omw = 1.0 - omega;
-    k.m3cl2 = -3.0 * c_l * c_l;
-    k.three_cl = 3.0 * c_l;
-    k.m_max = (float)(0.98 / (c_l * c_l));
-    k.q_scale = (float)ldexp(12.0 * c_l / omega, -33);
-    k.q_margin = 1e-4f + 68.0f * k.q_scale;
-    k.c_l = (float)c_l;
-    return k;
-}
-
 cudaError_t launch_step_f64(const Geom& g, const Phys& ph, const void* A, void* B, Counters cnt, bool count,
                             long long step_index, cudaStream_t st) {
     const double* a = (const double*)A;
