@@ -400,7 +400,7 @@ FxInit make_fx_init(const Phys& ph, int prec) {
     const double th = qh / c2, tl = (fma(-th, c2, qh) + (ql - th * c2l)) / c2;
     double oh, ol;
     fx_div2(1.0, 3.0, oh, ol);
-    const double dh = oh - th, de = (oh - (dh + th)) + (ol - tl);
+    const double dh = oh - th, de = ((oh - dh) - th) + (ol - tl);
     k.k0 = fx_const_w(dh, de, 64);
     fx_div2(1.0, 36.0, qh, ql);
     k.kS = fx_const_w(qh, ql, 65);

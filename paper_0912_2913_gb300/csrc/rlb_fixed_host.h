@@ -50,7 +50,8 @@ inline FxRun make_fx_run(double omega, double c_l) {
     tl = (fma(-th, c2h, qh) + (ql - th * c2l)) / c2h;
     k.kE1 = fx_const_w(th, tl, 65);
     // (3 - 2 / c_l^2) / 3 = 1 - 24 / (36 c_l^2)
-    k.kE0 = fx_const_w(1.0 - 24.0 * th, fma(-24.0, th, 1.0) - (1.0 - 24.0 * th) - 24.0 * tl, 62);
+    const double ph = 24.0 * th, hi = 1.0 - ph;
+    k.kE0 = fx_const_w(hi, ((1.0 - hi) - ph) - fma(24.0, th, -ph) - 24.0 * tl, 62);
     fx_div2(5.0, 9.0, qh, ql);
     k.kQ = fx_const(qh, ql, 63);
     fx_div2(1.0, 6.0, qh, ql);

@@ -15,7 +15,7 @@ static void check(const rlb::FxConst& k, long double want, int s) {
 
 int main() {
     const double taus[] = {0.5000000000000001, 0.51, 0.8, 1.0, 30.0, 1e6, 1e12};
-    const double speeds[] = {1e-150, 0.01, 0.3, 0.57, 0.99, 1.0, 1.3, 2.0, 2.1, 10.0, 1e6, 1e150};
+    const double speeds[] = {1e-150, 0.01, 0.3, 0.57, 0.99, 1.0, 1.1, 1.3, 1.5, 1.7320508, 2.0, 2.1, 10.0, 1e6, 1e150};
     const long double w = 1.0L - ldexpl(1.0L, -54);  // the binary64 weights
     for (double tau : taus)
         for (double c : speeds) {
@@ -32,6 +32,7 @@ int main() {
             check(k.kS, w * om / 36, 65);
             check(k.k0, w * om * (1 - 2 / (3 * c2)), 62);
             check(k.kE1, w / (36 * c2), 65);
+            check(k.kE0, w * (3 - 2 / c2) / 3, 62);
             check(k.kQ, 5.0L / 9, 63);
             check(k.kG, 1.0L / 6, 63);
         }
