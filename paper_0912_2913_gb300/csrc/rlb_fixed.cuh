@@ -545,9 +545,10 @@ __device__ __forceinline__ bool fx_moments(const T* h, const T* f, double m3cl2,
     // the moving populations share an exponent; FP64: the rest population,
     // 9 c_l^2 times larger, is added in binary64; FP32: it shares it too (its
     // deviation carries 24 bits)
-    const int em = DEV ? fx_max_exponent<19>(h) : fx_max_exponent<18>(h + 1);
-    const int ef = fx_max_exponent<19>(f);
-    bool ok = ((DEV && em == 0) || em > LO) && em < HI && ((DEV && ef == 0) || ef > LO) && ef < HI;
+    const uint32_t wm = DEV ? fx_max_word<19>(h) : fx_max_word<18>(h + 1), wf = fx_max_word<19>(f);
+    const int em = (int)(wm >> (DEV ? 24 : 21)), ef = (int)(wf >> (DEV ? 24 : 21));
+    // deviations that are all zero, but not subnormal ones
+    bool ok = ((DEV && wm == 0) || em > LO) && em < HI && ((DEV && wf == 0) || ef > LO) && ef < HI;
     double E = 0, sf = 0, dx = 0, dy = 0, dz = 0;
     if (!ok) return false;
     {

@@ -284,3 +284,25 @@ def test_a_stale_adjoint_ticket_ends_with_the_next_initialisation():
         assert torch.equal(sums(sims[0], k), want[0])
     for s in sims:
         s.close()
+
+
+def test_macro_of_subnormal_deviations():
+    """FP32 states whose deviations are binary32 subnormals beside a tiny
+    reference: the fields carry them."""
+    from paper_0912_2913_gb300 import RLB
+
+    ref = 1e-30
+    sim = RLB(16, 2, 1, 0.8, precision="fp32", n_ref=ref, eps_ref=ref, device="cuda:0")
+    rng = np.random.default_rng(0)
+    d = (rng.uniform(-1, 1, (1, 2, 16, 2, 19)) * 1e-38).astype(np.float32)
+    st = sim.cells_to_state(_cuda(d))
+    d = sim.state_to_cells(st).double().cpu().numpy()
+    assert np.abs(d).max() > 5e-39
+    rest = np.stack(oracle.equilibrium(ref, ref, np.zeros(3), 1.0))
+    n, e, b, _ = sim.macro(state=st, where="host")
+    want = oracle.macro(oracle.Params(nx=16, ny=2, nz=1, tau=0.8), np.ascontiguousarray(d + rest))
+    sim.close()
+    # the sums of a cell, 19 terms of 1e-30 in the oracle's binary64
+    assert np.all(np.abs(n - want[0]) <= 64 * U * ref)
+    assert np.all(np.abs(e - want[1]) <= 64 * U * ref)
+    assert np.all(np.abs(b - want[2]) <= 64 * U)
