@@ -264,16 +264,19 @@ def test_a_stale_adjoint_ticket_ends_with_the_next_initialisation():
 
     w = tiny_workload(23, 15, 15, 1, seed=6)
     sims = [RLB.from_workload(w, "fp64", device="cuda:0").init_fields(w.n, w.eps, w.beta) for _ in range(2)]
-    lam = [torch.randn(sims[0].state().shape, dtype=torch.float64, device="cuda") for _ in range(2)]
+    lam = [torch.randn(sims[0].state().shape, dtype=torch.float64, device="cuda") for _ in range(3)]
 
-    def sums(sim, noalloc):
+    def sums(sim, noalloc, k=0):
         acc = torch.zeros(4, dtype=torch.float64, device="cuda")
         f = (lambda *a: N.rlb_adjoint_step_noalloc(sim.ctx, *a)) if noalloc else sim.adjoint_step
-        f(sim.state(), lam[0], lam[1], acc[0:1], acc[1:4])
+        f(sim.state(), lam[k], lam[2], acc[0:1], acc[1:4])
         return acc.cpu()
 
     want = [sums(sims[0], k) for k in (False, True)]
     assert torch.equal(*want)
+    for sim in sims:  # other block sums in the arrays
+        assert not torch.equal(sums(sim, False, 1), want[0])
+        assert not torch.equal(sums(sim, True, 1), want[0])
     # the ticket is the fourth word behind the 2 x 4096 statistics slots
     at = 2 * ((sims[0].state_bytes + 255) // 256 * 256) + 8 * (2 * 4096 + 3)
     sims[0].ws[at] = 3
