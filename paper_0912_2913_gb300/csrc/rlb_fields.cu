@@ -406,8 +406,10 @@ FxInit make_fx_init(const Phys& ph, int prec) {
     k.kS = fx_const_w(qh, ql, 65);
     fx_div2(1.0, 12.0 * c, qh, ql);
     k.kS12 = fx_const_w(qh, ql, 65);
-    // exponents (high words) that leave every product and the output in range
-    k.lo = (prec == 0 ? 200 : 1023 - 110) << 20;
+    // exponents (high words) that leave every product and the output in range:
+    // a deviation that fx_to_f32 decides is at least 2^-29 of its cell's
+    // scale, and below 2^-126 it would be rounded a second time
+    k.lo = (prec == 0 ? 200 : 1023 - 96) << 20;
     k.hi = (prec == 0 ? 1800 : 1023 + 110) << 20;
     k.rf = ph.n_ref / 36.0;
     k.rg = ph.eps_ref / 36.0 * ph.inv_cl2;

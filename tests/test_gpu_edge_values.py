@@ -309,3 +309,35 @@ def test_macro_of_subnormal_deviations():
     assert np.all(np.abs(n - want[0]) <= 64 * U * ref)
     assert np.all(np.abs(e - want[1]) <= 64 * U * ref)
     assert np.all(np.abs(b - want[2]) <= 64 * U)
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -115, 2.0 ** -108, 2.0 ** -95])
+def test_fp32_init_of_deviations_near_the_subnormals(scale):
+    """Initial deviations rounded once to binary32, also where they end among
+    the subnormals (binary64 form restated in numpy, operation by operation)."""
+    from paper_0912_2913_gb300 import RLB
+
+    rng = np.random.default_rng(2)
+    shape, c = (4, 8, 64), 16.0
+    n, e = scale * np.exp(rng.uniform(-0.01, 0.01, (2,) + shape))
+    b = rng.uniform(-1e-3, 1e-3, (3,) + shape)
+    sim = RLB(64, 8, 4, 0.8, c_l=c, precision="fp32", n_ref=scale, eps_ref=scale, device="cuda:0").init_fields(n, e, b)
+    got = sim.state_to_cells(sim.state()).cpu().numpy()
+    sim.close()
+    bx, by, bz = b
+    i1, i2 = 1.0 / c, 1.0 / (c * c)
+    b2 = bx * bx + by * by + bz * bz
+    gam2 = 1.0 / (1.0 - b2)
+    ng, eg = n * np.sqrt(gam2), e * gam2
+    want = np.empty(shape + (2, 19), np.float32)
+    w0 = 1.0 / 3.0
+    want[..., 0, 0] = w0 * ng - w0 * scale
+    want[..., 1, 0] = w0 * (4.0 * eg - e * (2.0 * i2 + 1.0) - 2.0 * eg * b2 * i2) - w0 * scale * (3.0 - 2.0 * i2)
+    for p, q in enumerate((bx, by, bz, bx + by, bx - by, bx + bz, bx - bz, by + bz, by - bz)):
+        w = 1.0 / 18.0 if p < 3 else 1.0 / 36.0
+        fa = 3.0 * q * i1
+        gs, ga = e * i2 + eg * (6.0 * q * q - 2.0 * b2) * i2, eg * 4.0 * q * i1
+        for s, i in ((1, 2 * p + 1), (-1, 2 * p + 2)):
+            want[..., 0, i] = w * ng * (1.0 + s * fa) - w * scale
+            want[..., 1, i] = w * (gs + s * ga) - w * scale * i2
+    assert np.array_equal(got.view(np.int32), want.view(np.int32))
