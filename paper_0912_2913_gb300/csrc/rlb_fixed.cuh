@@ -71,8 +71,7 @@ struct FxRun {
     double m3cl2; // -3 c_l^2
     double three_cl;
     float m_max;  // largest |M|^2 / (c_l^2 E^2) of the fast path
-    float q_scale;  // beta = q_scale x (high word of w)
-    float q_margin;  // of the positivity decision on that beta
+    float q_scale;  // beta = q_scale x (high word of w); NaN where that is too coarse
     float c_l;
 };
 

@@ -30,7 +30,7 @@ inline FxRun make_fx_run(double omega, double c_l) {
     k.three_cl = 3.0 * c_l;
     k.m_max = (float)(0.98 / (c_l * c_l));
     k.q_scale = (float)ldexp(12.0 * c_l / omega, -33);
-    k.q_margin = 1e-4f + 68.0f * k.q_scale;
+    if (!(68.0f * k.q_scale < 9e-5f)) k.q_scale = NAN;  // (fx_nonpositive)
     k.c_l = (float)c_l;
     if (!fx_covers(c_l)) return k;
     double qh, ql, th, tl, c2h = c_l * c_l, c2l = fma(c_l, c_l, -c2h);

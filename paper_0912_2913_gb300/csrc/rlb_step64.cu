@@ -392,17 +392,19 @@ struct PlaneTab64 {
 // The positivity decision of nonpositive_eq.  The flag depends on the largest
 // |q_p| alone (the g bracket falls with |q| up to c_l / 3, beyond which the f
 // bracket is negative), so beta in binary32 decides unless a bracket lies
-// within q_margin of zero; then beta is formed in binary64 and rounded, as the
-// general path does.  The margin is 1e-4 and what the step of this beta,
-// q_scale (12 c_l tau 2^-33: 1e-4 at tau = 7e4), can move a bracket by: q by
-// two steps times |12 q - 4 c_l| <= 25, b2 by at most 3 times six.
+// within 1e-4 of zero; then beta is formed in binary64 and rounded, as the
+// general path does.  The step of this beta is q_scale = 12 c_l tau 2^-33, and a
+// bracket can move by 68 of them (q by two steps times |12 q - 4 c_l| <= 25, b2
+// by at most 3 times six): for tau c_l beyond 950 q_scale is NaN, which sends
+// every cell to binary64.  (A margin that grows with tau, read from the
+// constants instead of an immediate: 256^3 2.09 -> 2.17 ms.)
 __device__ __forceinline__ bool fx_nonpositive(const FxG& t, const double* u, double rD, const FxRun& k) {
     const float bx = k.q_scale * (float)t.wx.h, by = k.q_scale * (float)t.wy.h, bz = k.q_scale * (float)t.wz.h;
     const float ax = fabsf(bx), ay = fabsf(by), az = fabsf(bz);
     const float q = fmaxf(ax + ay, fmaxf(ax + az, ay + az));
     const float b2 = fmaf(bx, bx, fmaf(by, by, bz * bz));
     const float m = fminf(fmaf(-3.0f, q, k.c_l), fmaf(q, fmaf(6.0f, q, -4.0f * k.c_l), fmaf(-3.0f, b2, 1.0f)));
-    if (fabsf(m) > k.q_margin) return m < 0.0f;
+    if (fabsf(m) > 1e-4f) return m < 0.0f;
     const double r3 = rD * k.three_cl;
     return nonpositive_eq(d2f(u[0] * r3), d2f(u[1] * r3), d2f(u[2] * r3), k.c_l);
 }

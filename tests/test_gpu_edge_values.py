@@ -221,7 +221,7 @@ def test_macro_adjoint_of_cells_without_a_gradient(prec):
     assert bool((rest == 0).all())
 
 
-@pytest.mark.parametrize("tau", [1e4, 1e6, 1e9])
+@pytest.mark.parametrize("tau", [900.0, 1e4, 1e6, 1e9])
 @pytest.mark.parametrize("split", ["0", "1"])
 def test_positivity_count_at_large_tau(tau, split, monkeypatch):
     """The positivity decision in binary32 near its threshold at |q| = 1/3, for
