@@ -540,7 +540,8 @@ struct FxMoments {
 template <typename T>
 __device__ __forceinline__ bool fx_moments(const T* h, const T* f, double m3cl2, double n_ref, double eps_ref, FxMoments& m) {
     constexpr bool DEV = sizeof(T) == 4;
-    constexpr int BIAS = DEV ? 127 : 1023, LO = DEV ? 64 : 128, HI = DEV ? 250 : 1900;
+    // LO: with E below 2^477 the quotients M / E stay above 2^-900 (fx_to)
+    constexpr int BIAS = DEV ? 127 : 1023, LO = DEV ? 64 : 624, HI = DEV ? 250 : 1900;
     // the moving populations share an exponent; FP64: the rest population,
     // 9 c_l^2 times larger, is added in binary64; FP32: it shares it too (its
     // deviation carries 24 bits)

@@ -341,3 +341,20 @@ def test_fp32_init_of_deviations_near_the_subnormals(scale):
             want[..., 0, i] = w * ng * (1.0 + s * fa) - w * scale
             want[..., 1, i] = w * (gs + s * ga) - w * scale * i2
     assert np.array_equal(got.view(np.int32), want.view(np.int32))
+
+
+def test_macro_of_a_rest_population_far_above_the_others():
+    """Moving populations 2^-1000 times the rest one: beta underflows instead
+    of wrapping."""
+    from paper_0912_2913_gb300 import RLB
+
+    p = oracle.Params(nx=4, ny=1, nz=1, tau=0.8)
+    a = oracle.init(p, np.ones((1, 1, 4)), np.ones((1, 1, 4)), np.full((3, 1, 1, 4), 0.1))
+    a[..., 1, 1:] *= 2.0 ** np.array([0, -400, -760, -800])[:, None]
+    a[..., 1, 0] *= 2.0 ** np.array([0, 200, 300, 400])
+    sim = RLB(4, 1, 1, 0.8, precision="fp64", device="cuda:0")
+    n, e, b, _ = sim.macro(state=sim.cells_to_state(_cuda(a)), where="host")
+    want = oracle.macro(p, a)
+    sim.close()
+    assert np.all(np.abs(e - want[1]) <= 64 * U * want[1])
+    assert np.all(np.abs(b - want[2]) <= 64 * U * np.abs(want[2]) + 5e-324 * 64)
