@@ -319,18 +319,27 @@ static int sm_count() {
 // FP64 above all, is then the step's latency).  Results do not depend on it.
 static int step_block(long long N, int full) { return blocks_for(N, full) < (unsigned)sm_count() ? 32 : full; }
 
-// Launch shape of the FP32 step (all give the same bits).  8, f loaded before
-// the g arithmetic in 64-thread blocks x 12 per SM, is the fastest or within
-// 3 % of it from 1600 cells to 512^3 (us a step, shapes 2 / 7 / 8: 47x33x33
-// 5.7 / 4.4 / 4.2; 200x100x100 sphere 102.5 / 93.6 / 91.5; 256^3 844 / 750 /
-// 739; 512^3 6740 / 5982 / 5880), except where the lattice gives every
-// scheduler three to four warps: there two 256-thread blocks spread the warps
-// evenly over an SM's schedulers (63x41x29: 5.8 / 6.9 / 6.3), just below it
-// (48x35x35: 5.8 / 5.0 / 6.2) and just above (64x40x40: 8.8 / 7.0 / 6.6) they
-// lose or gain little.
+// Launch shape of the FP32 step (all give the same bits), by how the lattice
+// fills the chip: r = cells per SM / 128, one warp on each scheduler per unit.
+// Shape 8, f loaded before the g arithmetic in 64-thread blocks x 12 per SM, is
+// the fastest where blocks are many (us a step, shapes 2 / 7 / 8: 200x100x100
+// sphere 102.5 / 93.6 / 91.5; 256^3 844 / 750 / 739; 512^3 6740 / 5982 / 5880)
+// or fit easily (r = 0.5: 3.8 / 3.2 / 3.0; 2.5: 5.7 / 4.3 / 4.1).  In between a
+// shape takes a step up where another block goes on the busiest SM (2 of 256
+// threads at r = 4, 7 of 128 at 3.5, 8 of 64 at 3) and where its resident
+// blocks are used up (7 at r = 7 and 14, 8 at 6 and 12), the same for
+// 1D, 3D, periodic and inflow lattices:
+//   r = 3.0    5.9 / 4.2 / 4.2     r = 3.01   5.8 / 4.7 / 6.1     r = 3.5    5.8 / 5.1 / 6.3
+//   r = 3.51   5.8 / 6.8 / 6.3     r = 4.0    5.8 / 6.8 / 6.4     r = 4.01   8.7 / 6.8 / 6.4
+//   r = 5.98   9.3 / 7.1 / 6.3     r = 6.1    9.4 / 7.1 / 7.2     r = 7.0    9.4 / 6.9 / 7.8
+//   r = 8.0    9.3 / 8.4 / 8.5     r = 8.9   10.9 / 9.0 / 9.0     r = 11.9  12.9 / 10.7 / 10.8
+//   r = 12.5  14.0 / 11.2 / 11.7   r = 14.0  15.0 / 12.6 / 13.2   r = 14.9  16.6 / 13.8 / 14.2
+//   r = 16.0  17.5 / 15.4 / 15.2   r = 18.8  21.8 / 18.7 / 18.2   r = 32    35.8 / 33.3 / 31.0
 static int f32_shape(long long N) {
-    const long long per = 128ll * sm_count();  // one warp on each scheduler
-    return N > 3 * per && N <= 4 * per ? 2 : 8;
+    const long long r2 = (N + 64ll * sm_count() - 1) / (64ll * sm_count());  // 2 r, rounded up
+    if (r2 == 7) return 7;
+    if (r2 == 8) return 2;
+    return (r2 > 12 && r2 <= 17) || (r2 > 24 && r2 <= 30) ? 7 : 8;
 }
 
 template <int XBC, bool SOLID>
