@@ -216,13 +216,14 @@ RLB_API rlb_status rlb_adjoint_step(rlb_ctx* ctx, const void* state_t, const voi
  * kernel, SMs x 2 blocks of 128), FP32 the
  * persistent shared-memory staged kernel (SMs x 3 blocks of 128; with
  * RLB_ADJ_PIPE=0 or 1 the persistent register kernel, SMs x 4 blocks), grids
- * capped at the lattice's block count.  The per-warp partial sums live in one static
+ * capped at the lattice's block count.  The partial sums live in one static
  * device array of 32768 doubles (256 KiB) per device: a launch that would
- * need more (4 doubles per warp) returns RLB_ERR_ARG and enqueues nothing;
- * every launch writes all the slots it reads.  The counter by which the blocks
- * of an FP64 launch find the last of them is the context's own; rlb_create and
- * rlb_init_fields set it to zero and every launch leaves it there.  The first call on each device (and the first after the device's
- * context was reset) does the set-up: it takes the array's address and loads
+ * need more (4 doubles per block, in the staged kernel per warp) returns
+ * RLB_ERR_ARG and enqueues nothing; every launch writes all the slots it
+ * reads.  The counter by which the blocks of a launch find the last of them
+ * (all kernels but the staged one) is the context's own; rlb_create and
+ * rlb_init_fields set it to zero and every launch leaves it there.  The first
+ * call on each device (and the first after the device's context was reset) does the set-up: it takes the array's address and loads
  * every kernel this entry point launches, which may allocate and
  * synchronise, so make that first call before any stream capture and before
  * the code that must not allocate; later calls allocate nothing.  The

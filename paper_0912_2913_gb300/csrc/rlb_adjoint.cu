@@ -2376,11 +2376,9 @@ cudaError_t smem_opt_in(const void* kern, int bytes) {
 
 // Launch of the fixed-point FP64 adjoint: eight lanes per cell while the
 // lanes fit two warps per scheduler, else persistent blocks of 64 threads.
-// warps(): how many write partial sums (4 each).
 struct AdjFxShape {
     bool split;
     int grid, threads;
-    int warps() const { return grid * (threads / 32); }
 };
 static AdjFxShape adj_fx_shape(long long N, int nsm) {
     if (N <= kAdjSplitCells && N <= 32ll * nsm) return {true, (int)((8 * N + 127) / 128), 128};
@@ -2534,11 +2532,11 @@ cudaError_t launch_adjoint_fields(int prec, const Geom& g, const Phys& ph, const
 // ---------------------------------------------------------------------------
 // Allocation-free adjoint step.  Same kernels as launch_adjoint_step, always
 // as the persistent grid-stride launch (grid = SMs x resident blocks, capped
-// at the block count), with the per-warp partial sums in a fixed static
-// device array instead of the context workspace.  Every launch writes all
-// grid*16 slots it reads, so the array needs no zeroing; two launches that
-// overlap in time on one device (other streams, other contexts) share it and
-// race.
+// at the block count), with the partial sums in a fixed static device array
+// instead of the context workspace.  Every launch writes all the slots it
+// reads (4 per block, in the staged kernel per warp), so the array needs no
+// zeroing; two launches that overlap in time on one device (other contexts)
+// share it and race, for their own sums only (AdjSums).
 // ---------------------------------------------------------------------------
 static __device__ __align__(256) double g_adj_scratch[kAdjScratchDoubles];
 
@@ -2648,7 +2646,7 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
     const int nb = adj_blocks(g.N);
     if (prec == 0 && ph.fx_on) {
         const AdjFxShape sh = adj_fx_shape(g.N, nsm);
-        const long long need = 4ll * sh.warps();
+        const long long need = 4ll * sh.grid;  // 4 partial sums per block (block_sums)
         if (need_doubles) *need_doubles = need;
         if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
         set_last_launch_count(1);
@@ -2660,7 +2658,7 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
         // FP32 with the default kernel choice: the staged kernel that
         // rlb_adjoint_step runs (persistent, SMs x 3 blocks of 128)
         const int grid3 = nsm * 3 < nb ? nsm * 3 : nb;
-        const long long need = 16ll * grid3;
+        const long long need = 16ll * grid3;  // 4 partial sums per warp (k_finalize adds them up)
         if (need_doubles) *need_doubles = need;
         if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
         const int warps = adjoint_step_t<float>(g, ph, (const float*)A, (const float*)lam_in, (float*)lam_out, sums, nb,
@@ -2671,7 +2669,7 @@ cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph,
     }
     const int minb = prec == 0 ? 2 : 4;
     const int grid = nsm * minb < nb ? nsm * minb : nb;
-    const long long need = 16ll * grid;  // 4 warps x 4 partial sums per block
+    const long long need = 4ll * grid;  // 4 partial sums per block (block_sums)
     if (need_doubles) *need_doubles = need;
     if (need > kAdjScratchDoubles) return cudaErrorInvalidValue;
     set_last_launch_count(1);

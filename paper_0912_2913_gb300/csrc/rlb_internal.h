@@ -117,8 +117,9 @@ cudaError_t launch_check_solid_planes(const Geom& g, const uint8_t* solid, unsig
 cudaError_t launch_halo_exchange(int elem, long long nxy, void* lower, long long S_lower, int nz_lower, void* upper,
                                  long long S_upper, cudaStream_t stream);
 
-// Adjoint.  'red' holds 4 doubles of partial sums per warp: of 32 cells, or
-// of 4 in the eight-lane form of small lattices (at most kAdjSplitCells).
+// Adjoint.  'red' holds 4 doubles of partial sums per warp of 32 cells, or per
+// block of a kernel that adds up its own (in the eight-lane form of small
+// lattices, at most kAdjSplitCells, blocks of 16 cells).
 constexpr long long kAdjSplitCells = 8192;
 inline long long adj_red_doubles(long long N) { return N <= kAdjSplitCells ? N + 64 : 4 * 4 * ((N + 127) / 128); }
 cudaError_t launch_adjoint_macro(int prec, const Geom& g, const Phys& ph, const void* A, const double* dn,
@@ -128,8 +129,8 @@ cudaError_t launch_adjoint_step(int prec, const Geom& g, const Phys& ph, const v
                                 double* dbeta_in, cudaStream_t stream);
 // Allocation-free variant of launch_adjoint_step (same kernels, persistent
 // grid): partial sums in a static device array of kAdjScratchDoubles doubles,
-// set up once per device on first use.  Needs 4 doubles per warp of the
-// grid (reported in *need_doubles); returns cudaErrorInvalidValue, launching
+// set up once per device on first use.  Needs 4 doubles per block of the grid,
+// in the staged FP32 kernel per warp (reported in *need_doubles); returns cudaErrorInvalidValue, launching
 // nothing, when that exceeds the array.
 constexpr long long kAdjScratchDoubles = 32768;  // 256 KiB
 cudaError_t launch_adjoint_step_noalloc(int prec, const Geom& g, const Phys& ph, const void* A, const void* lam_in,
