@@ -1037,7 +1037,9 @@ struct AdjFxCell {
     double nuE, nuS, tx, ty, tz;      // omega v_E, omega a_S, omega v_d
 };
 
-// Recovery and the g moments of mu in binary64.  S*, P*, T*: the sums of
+// Recovery and the g moments of mu in binary64 (ties to even throughout: sums
+// of equal values, as of lambda next to a boundary, meet them often, and an
+// error that every step repeats adds up in lambda).  S*, P*, T*: the sums of
 // sigma_p over the axis pairs (doubled), and over each plane's two diagonal
 // pairs and their difference; units 2^-56 of the block exponents eh, em.
 __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int64_t dz, int64_t dot, int64_t m0, int64_t Sx,
@@ -1046,7 +1048,7 @@ __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int6
                                          const Phys& ph, const AdjFx& k, AdjFxCell& t) {
     const int kh = eh - 1079, km = em - 1079;
     const double Ed = fx_to_even(E, kh);
-    t.x = fx_to(dx, kh), t.y = fx_to(dy, kh), t.z = fx_to(dz, kh);
+    t.x = fx_to_even(dx, kh), t.y = fx_to_even(dy, kh), t.z = fx_to_even(dz, kh);
     const double E2 = Ed + Ed;
     t.E4 = E2 + E2;
     const double dd = fma(t.x, t.x, fma(t.y, t.y, t.z * t.z));
@@ -1068,17 +1070,17 @@ __device__ __forceinline__ void adj_fx_g(int64_t E, int64_t dx, int64_t dy, int6
     const int64_t kap = (m0 << 2) - (fx_mul_exact(sp, k.kS1) << 2);
     auto g38 = [](int64_t v, int64_t k8) { return fx_weight_signed(fx_round3_even(v + (v << 1) + k8)); };
     auto g38_off = [](int64_t v) { return fx_weight_signed((v + (v << 1) + 4) >> 3); };  // u_a u_b has either sign
-    const double Gxx = fx_to(g38(Sx + Pxy + Pzx, kap), km), Gyy = fx_to(g38(Sy + Pxy + Pyz, kap), km),
-                 Gzz = fx_to(g38(Sz + Pyz + Pzx, kap), km);
-    const double Gxy = fx_to(g38_off(Txy), km), Gxz = fx_to(g38_off(Tzx), km), Gyz = fx_to(g38_off(Tyz), km);
+    const double Gxx = fx_to_even(g38(Sx + Pxy + Pzx, kap), km), Gyy = fx_to_even(g38(Sy + Pxy + Pyz, kap), km),
+                 Gzz = fx_to_even(g38(Sz + Pyz + Pzx, kap), km);
+    const double Gxy = fx_to_even(g38_off(Txy), km), Gxz = fx_to_even(g38_off(Tzx), km), Gyz = fx_to_even(g38_off(Tyz), km);
     t.yx = fma(Gxx, t.ux, fma(Gxy, t.uy, Gxz * t.uz));
     t.yy = fma(Gxy, t.ux, fma(Gyy, t.uy, Gyz * t.uz));
     t.yz = fma(Gxz, t.ux, fma(Gyz, t.uy, Gzz * t.uz));
-    t.aE = fx_to(fx_mul_exact(sp, k.kE1) + fx_mul_exact(m0 << 3, k.kE0), km - 1);
+    t.aE = fx_to_even(fx_mul_exact(sp, k.kE1) + fx_mul_exact(m0 << 3, k.kE0), km - 1);
     t.uy_ = fma(t.ux, t.yx, fma(t.uy, t.yy, t.uz * t.yz));
-    t.vx = fx_to(Vx, km), t.vy = fx_to(Vy, km), t.vz = fx_to(Vz, km);
+    t.vx = fx_to_even(Vx, km), t.vy = fx_to_even(Vy, km), t.vz = fx_to_even(Vz, km);
     const double Vd = fma(t.vx, t.x, fma(t.vy, t.y, t.vz * t.z));
-    t.tsum = fx_to(dot, em + eh - 2102) - fma(Ed, t.aE, fma(D, t.uy_, Vd * (1.0 / 12.0)));
+    t.tsum = fx_to_even(dot, em + eh - 2102) - fma(Ed, t.aE, fma(D, t.uy_, Vd * (1.0 / 12.0)));
 }
 
 // The f moments (36 w0 mu_f0 + F1 and F times 36, S, the dot product) and the
@@ -1087,10 +1089,10 @@ __device__ __forceinline__ void adj_fx_f(int64_t Sf, int64_t fd, int64_t Fs, int
                                          int ef, const Phys& ph, const AdjFx& k, AdjFxCell& t) {
     const double Sd = fx_to_even(Sf, fh - 1079);
     const int kf = ef - 1079;
-    const double fx = fx_to(fx_weight_signed(Fx), kf), fy = fx_to(fx_weight_signed(Fy), kf), fz = fx_to(fx_weight_signed(Fz), kf);
+    const double fx = fx_to_even(fx_weight_signed(Fx), kf), fy = fx_to_even(fx_weight_signed(Fy), kf), fz = fx_to_even(fx_weight_signed(Fz), kf);
     const double Fu = fma(fx, t.ux, fma(fy, t.uy, fz * t.uz));
-    const double aS = fma(0.25, Fu, fx_to(fx_mul_exact(Fs, k.kS36), kf - 1));
-    t.tsum += fx_to(fd, ef + fh - 2102) - Sd * aS;
+    const double aS = fma(0.25, Fu, fx_to_even(fx_mul_exact(Fs, k.kS36), kf - 1));
+    t.tsum += fx_to_even(fd, ef + fh - 2102) - Sd * aS;
     const double sD = (0.25 * Sd) * t.rD;
     const double aD = -fma(sD, Fu, t.uy_);
     t.nuE = ph.omega * fma(aD, fma(t.E4, t.rs, 2.0), t.aE);
@@ -1373,7 +1375,7 @@ __global__ void __launch_bounds__(kAdjFxThreads, kAdjFxBlocks)
                 const bool back = (bounced >> i) & 1u;
                 const long long at = (long long)(back ? opp_rt(i) : i) * S + (back ? 0 : off);
                 Lo[RLB_CHK_OFF(at, idx, 38ll * S)] = fma(ph.fx.omw, col[i][tid], nuS);
-                Lo[RLB_CHK_OFF(19 * S + at, idx, 38ll * S)] = fma(ph.fx.omw, col[19 + i][tid], fx_to(kt, ek - 1083));
+                Lo[RLB_CHK_OFF(19 * S + at, idx, 38ll * S)] = fma(ph.fx.omw, col[19 + i][tid], fx_to_even(kt, ek - 1083));
             };
             put(v.ax, am, kE + ka);
             put(v.ax + 1, ap, kE - ka);
@@ -1535,7 +1537,7 @@ __global__ void __launch_bounds__(128)
                 const bool bk = (back >> n) & 1u;
                 const long long at = (long long)(bk ? opp_rt(i) : i) * S + idx + (bk ? 0 : o.src(i));
                 Lout[RLB_CHK(at, 38ll * S)] = fma(ph.fx.omw, uf[n], t.nuS);
-                Lout[RLB_CHK(19 * S + at, 38ll * S)] = fma(ph.fx.omw, ug[n], i == 0 ? t.nuE : fx_to(kt, ek - 1083));
+                Lout[RLB_CHK(19 * S + at, 38ll * S)] = fma(ph.fx.omw, ug[n], i == 0 ? t.nuE : fx_to_even(kt, ek - 1083));
             }
         }
         if (j == 0) tau_acc = t.tsum * c.inv_tau2;
@@ -2148,8 +2150,8 @@ __global__ void __launch_bounds__(128, 6) k_adjoint_macro(const T* __restrict__ 
 #pragma unroll
                 for (int i = 0; i < 19; ++i) put(i, aS);
                 auto gput = [&](int p, int64_t t) {
-                    put(20 + 2 * p, fx_to(kE + t, ek - 1083));
-                    put(21 + 2 * p, fx_to(kE - t, ek - 1083));
+                    put(20 + 2 * p, fx_to_even(kE + t, ek - 1083));
+                    put(21 + 2 * p, fx_to_even(kE - t, ek - 1083));
                 };
                 put(19, vE);
                 gput(0, kx), gput(1, ky), gput(2, kz), gput(3, kx + ky), gput(4, kx - ky), gput(5, kx + kz), gput(6, kx - kz);

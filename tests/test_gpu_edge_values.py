@@ -358,3 +358,70 @@ def test_macro_of_a_rest_population_far_above_the_others():
     sim.close()
     assert np.all(np.abs(e - want[1]) <= 64 * U * want[1])
     assert np.all(np.abs(b - want[2]) <= 64 * U * np.abs(want[2]) + 5e-324 * 64)
+
+
+@pytest.mark.parametrize("size", [(16, 16, 16), (64, 64, 4)], ids=["eight_lanes", "staged"])
+def test_lambda_has_no_common_rounding_error(size):
+    """lambda_t of one FP64 adjoint step for lambda of one sign that grows along
+    x, as next to an outflow plane: rounding ties in v_E + e.v_d one way is an
+    error that every step repeats.  The reference is formed in extended
+    precision.  A value carries three roundings of up to half a unit of 2^-52 of
+    the cell's largest lambda (the sums, the conversion, the relaxation); the
+    bound is 4 standard deviations of the mean over the cells, with the values
+    of a cell taken as fully correlated."""
+    from paper_0912_2913_gb300 import RLB
+
+    nx, ny, nz = size
+    N, tau = nx * ny * nz, 0.9
+    rng = np.random.default_rng(21)
+    ev = np.asarray(oracle.lattice()[0], int)
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    p = oracle.Params(nx=nx, ny=ny, nz=nz, tau=tau)
+    b = np.zeros((3, nz, ny, nx))
+    b[0] = rng.uniform(-0.05, 0.05, b[0].shape)
+    h = oracle.init(p, *rng.uniform(0.9, 1.1, (2,) + b[0].shape), b)
+    h *= 1 + 1e-3 * rng.uniform(-1, 1, h.shape)
+    mu = np.empty_like(h)
+    mu[..., 0, :] = rng.uniform(1, 2, h.shape[:3])[..., None]
+    mu[..., 1, :] = rng.uniform(30, 60, h.shape[:3])[..., None] * np.array([1.0, 2.06, 0.0])[ev[:, 0]]
+
+    # nu = (1 - 1/tau) mu + (d eq / d h)^T mu / tau, cell by cell
+    L = np.longdouble
+    hl, ml = h.reshape(N, 2, 19).astype(L), mu.reshape(N, 2, 19).astype(L)
+    E, S = hl[:, 1].sum(1), hl[:, 0].sum(1)
+    M = [(hl[:, 1] * ev[:, k]).sum(1) for k in range(3)]
+    s = np.sqrt(4 * E * E - 3 * sum(m * m for m in M))
+    eps, D = s - E, 2 * E + s
+    u = [3 * m / D for m in M]
+    b2 = sum(v * v for v in u)
+    g2 = 1 / (1 - b2)
+    eg = eps * g2
+    aS, ae, dg2, db2, ab = 0, 0, 0, 0, [0, 0, 0]
+    for i in range(19):
+        q = sum(int(ev[i, k]) * u[k] for k in range(3))
+        mf, mg = ml[:, 0, i] * w[i], ml[:, 1, i] * w[i]
+        aS = aS + mf * (1 + 3 * q)
+        br = 6 * q * q - 2 * b2 + 4 * q if i else 4 - 2 * b2
+        ae = ae + mg * ((1 if i else -3) + g2 * br)
+        dg2, db2 = dg2 + mg * eps * br, db2 - 2 * mg * eg
+        ab = [ab[k] + int(ev[i, k]) * (3 * S * mf + eg * (12 * q + 4) * mg) for k in range(3)]
+    ab = [ab[k] + 2 * (db2 + dg2 * g2 * g2) * u[k] for k in range(3)]
+    abD = sum(ab[k] * u[k] for k in range(3)) / D
+    dE = 4 * E / s - 1
+    vE, vd = ae * dE - abD * (3 + dE), [3 * ab[k] / D + 3 * (abD - ae) / s * M[k] for k in range(3)]
+    om = L(1.0 / tau)
+    want = (1 - om) * ml[:, 1] + om * np.stack([vE + sum(int(ev[i, k]) * vd[k] for k in range(3)) for i in range(19)], 1)
+
+    a = np.empty_like(h)
+    for i in range(19):  # the state a step gathers h from
+        a[..., i] = np.roll(h[..., i], tuple(-ev[i][c] for c in (2, 1, 0)), axis=(0, 1, 2))
+    sim = RLB(nx, ny, nz, tau, precision="fp64", device="cuda:0")
+    lo, acc = sim.new_state(), torch.zeros(4, dtype=torch.float64, device="cuda")
+    sim.adjoint_step(sim.cells_to_state(_cuda(a)), sim.cells_to_state(_cuda(mu)), lo, acc[0:1], acc[1:4])
+    out = sim.state_to_cells(lo).cpu().numpy()
+    sim.close()
+    got = np.stack([np.roll(out[..., 1, i], tuple(ev[i][c] for c in (2, 1, 0)), axis=(0, 1, 2)).reshape(N) for i in range(19)], 1)
+    err = ((got.astype(L) - want) / np.abs(ml[:, 1]).max(1)[:, None]).astype(np.float64)[:, ev[:, 0] > 0].mean(1)
+    sigma = 2 * U * np.sqrt(3 / 12)
+    assert np.abs(err).max() <= 16 * U
+    assert abs(err.mean()) <= 4 * sigma / np.sqrt(N), (err.mean(), sigma / np.sqrt(N))
