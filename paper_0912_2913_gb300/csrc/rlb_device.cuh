@@ -229,7 +229,7 @@ __device__ __forceinline__ int dup_of(int x, int nx) {
     return (XBC != XBC_PERIODIC && x == nx - 2) ? 1 : ((XBC == XBC_OUTFLOW_BOTH && x == 1) ? -1 : 0);
 }
 template <int XBC>
-__device__ __forceinline__ bool dup_both(int nx) {
+__host__ __device__ __forceinline__ bool dup_both(int nx) {
     return XBC == XBC_OUTFLOW_BOTH && nx == 3;
 }
 

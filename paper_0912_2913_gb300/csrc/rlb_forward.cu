@@ -1,7 +1,7 @@
-// rlb_forward.cu -- forward kernels of librlb: the FP32 fused stream-and-collide
-// step (the FP64 one: rlb_step64.cu) of the relativistic lattice Boltzmann scheme (Eqs. lbe1, lbe2 with the
-// eps = 3P equilibria Eqs. equil1s, equil2as, equil2bs), the equilibrium
-// initialisation and the macroscopic output.
+// rlb_forward.cu -- the FP32 fused stream-and-collide step of the relativistic
+// lattice Boltzmann scheme (Eqs. lbe1, lbe2 with the eps = 3P equilibria Eqs.
+// equil1s, equil2as, equil2bs); the FP64 one is in rlb_step64.cu, the
+// equilibrium initialisation and the macroscopic output in rlb_fields.cu.
 //
 // One thread owns one cell.  A step pulls the 38 populations that arrive at
 // the cell (h_i(x) = A_i(x - e_i), link bounce-back h_i(x) = A_opp(i)(x) when
@@ -56,8 +56,11 @@ void set_last_launch_count(int n) { g_last_launches = n; }
 // COMP: the compensated collision (collide_cell_f32c), run for c_l > 1.
 // EARLY: the f populations are loaded before the g phase's arithmetic.
 // TB: threads per block the register budget is cut for.
+// BOTH: the one fluid plane of three is copied by both outflow ghosts (a test
+// of nx beside the stores cost a lattice that is not so narrow 10 to 50 % of
+// its step: 1600 cells 2.9 -> 4.3 us).
 template <int XBC, bool SOLID, int MINB, bool PREF, typename I = long long, bool COMP = false, bool EARLY = false,
-          int TB = 256>
+          int TB = 256, bool BOTH = false>
 __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__ A, float* __restrict__ B, Geom g,
                                                        Dev32 c, Counters cnt, int count, long long step_index) {
     const int idx = dependent_begin(blockIdx.x * blockDim.x + threadIdx.x);
@@ -85,7 +88,6 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
     PullOffsets o(g, x, y, z);
     if (keep) o.xm = o.xp = o.ym = o.yp = o.zm = o.zp = 0;
     const int dup = dup_of<XBC>(x, g.nx);
-    const bool both = dup_both<XBC>(g.nx);
     float* Bc = B + idx;
     float* Bgc = Bg + idx;
     auto put = [&](int q, float v, float old) {
@@ -95,16 +97,11 @@ __global__ void __launch_bounds__(TB, MINB) k_step_f32(const float* __restrict__
             b[RLB_CHK_OFF(pq(q) * S, idx, lim)] = v;
             // the outflow copy: dup (+-1) moves the pointer, so that the
             // unsigned offset never has to hold a negative value
-            if (dup) {
-                (b + dup)[RLB_CHK_OFF(pq(q) * S, idx + dup, lim)] = v;
-                if (both) (b - 1)[RLB_CHK_OFF(pq(q) * S, idx - 1, lim)] = v;
-            }
+            if (dup) (b + dup)[RLB_CHK_OFF(pq(q) * S, idx + dup, lim)] = v;
         } else {
             Bc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v;
-            if (dup) {
-                Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
-                if (both) Bc[RLB_CHK_OFF(q * S - 1, idx, 38ll * S)] = v;
-            }
+            if (dup) Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
+            if (BOTH) Bc[RLB_CHK_OFF(q * S - 1, idx, 38ll * S)] = v;
         }
     };
     if (PREF) {
@@ -179,21 +176,14 @@ __global__ void __launch_bounds__(256, 3) k_step_f32_pipe(const float* __restric
         }
         const PullOffsets o(g, x, y, z);
         const int dup = dup_of<XBC>(x, g.nx);
-        const bool both = dup_both<XBC>(g.nx);
         float* Bc = B + idx;
         auto put = [&](int q, float v, float) {
             if (CS) {
                 __stcs(Bc + q * S, v);
-                if (dup) {
-                    __stcs(Bc + q * S + dup, v);
-                    if (both) __stcs(Bc + q * S - 1, v);
-                }
+                if (dup) __stcs(Bc + q * S + dup, v);
             } else {
                 Bc[RLB_CHK_OFF(q * S, idx, 38ll * S)] = v;
-                if (dup) {
-                    Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
-                    if (both) Bc[RLB_CHK_OFF(q * S - 1, idx, 38ll * S)] = v;
-                }
+                if (dup) Bc[RLB_CHK_OFF(q * S + dup, idx, 38ll * S)] = v;
             }
         };
         if (SOLID && is_solid(__ldg(RLB_CHK_PTR(A, 19 * S + idx, 38ll * S)))) {
@@ -357,6 +347,19 @@ static void launch_step_t(int prec, const Geom& g, const Phys& ph, const void* A
         const int cs = count ? 1 : 0;
         const bool idx32 = 38 * g.S < (1ll << 31);
         const bool split32 = !idx32 && 19 * g.S < (1ll << 32);  // unsigned offsets per population set
+        if constexpr (XBC == XBC_OUTFLOW_BOTH) {
+            if (dup_both<XBC>(g.nx)) {  // every variant of the tuning knobs has the same bits
+                const int t = tb < 128 ? tb : 128;
+                auto go = [&](auto kern) {
+                    launch_dependent(kern, blocks_for(g.N, t), t, 0, st, (const float*)A, (float*)B, g, c, cnt, cs, step_index);
+                };
+                if (ph.c_l > 1.0)
+                    go(k_step_f32<XBC, SOLID, 5, false, long long, true, false, 128, true>);
+                else
+                    go(k_step_f32<XBC, SOLID, 7, false, long long, false, true, 128, true>);
+                return;
+            }
+        }
         if (ph.c_l > 1.0) {
             // lattice speeds above 1: the compensated collision (one launch
             // shape; the TMA-staged and tuning variants use the binary32 one).
