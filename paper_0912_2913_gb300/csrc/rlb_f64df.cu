@@ -70,7 +70,8 @@ __device__ __forceinline__ double relax(dfl h, dfl eq, dfl om) {
 
 }  // namespace
 
-template <int XBC, bool SOLID>
+// BOTH: nx = 3 with outflow at both ends (x = 1 is copied by both ghosts)
+template <int XBC, bool SOLID, bool BOTH = false>
 __global__ void __launch_bounds__(128) k_step_f64_df(const double* __restrict__ A, double* __restrict__ B, Geom g,
                                                      Phys ph, F64dfConst k, Counters cnt, int count,
                                                      long long step_index) {
@@ -95,13 +96,10 @@ __global__ void __launch_bounds__(128) k_step_f64_df(const double* __restrict__ 
     }
     const PullOffsets o(g, x, y, z);
     const int dup = dup_of<XBC>(x, g.nx);
-    const bool both = dup_both<XBC>(g.nx);
     auto put = [&](int q, double v) {
         B[RLB_CHK(q * S + idx, 38ll * S)] = v;
-        if (dup) {
-            B[RLB_CHK(q * S + idx + dup, 38ll * S)] = v;
-            if (both) B[RLB_CHK(q * S + idx - 1, 38ll * S)] = v;
-        }
+        if (dup) B[RLB_CHK(q * S + idx + dup, 38ll * S)] = v;
+        if (BOTH) B[RLB_CHK(q * S + idx - 1, 38ll * S)] = v;
     };
     // ---- g phase: energy-momentum populations (they alone fix eps, beta) ----
     dfl G[19];
@@ -211,7 +209,12 @@ cudaError_t launch_step_f64_df(const Geom& g, const Phys& ph, const void* A, voi
         case XBC_INFLOW_OUTFLOW:
             k_step_f64_df<XBC_INFLOW_OUTFLOW, true><<<nb, threads, 0, st>>>(a, b, g, ph, k, cnt, cs, step_index);
             break;
-        default: k_step_f64_df<XBC_OUTFLOW_BOTH, true><<<nb, threads, 0, st>>>(a, b, g, ph, k, cnt, cs, step_index); break;
+        default:
+            if (dup_both<XBC_OUTFLOW_BOTH>(g.nx))
+                k_step_f64_df<XBC_OUTFLOW_BOTH, true, true><<<nb, threads, 0, st>>>(a, b, g, ph, k, cnt, cs, step_index);
+            else
+                k_step_f64_df<XBC_OUTFLOW_BOTH, true><<<nb, threads, 0, st>>>(a, b, g, ph, k, cnt, cs, step_index);
+            break;
     }
     return cudaGetLastError();
 }
