@@ -934,25 +934,28 @@ __global__ void __launch_bounds__(128, MINB)
 //
 // k_adjoint_step<double> (the other lattice speeds) issues 408 FP64
 // instructions per collided cell, 26,500 clocks of a scheduler's FP64 pipe per
-// 32 cells, against 5,400 for the cell's 912 bytes at the HBM rate; here 110
-// remain (72 for recovery and algebra, 38 relaxations) beside 6,000
+// 32 cells, against 5,400 for the cell's 912 bytes at the HBM rate; here 118
+// remain (80 for recovery and algebra, 38 relaxations) beside 6,624
 // instructions in all.  What bounds it now is the speed of a warp: with 12
-// warps per SM 46 % of the issue slots and 51 % of the FP64 pipe are used, the
+// warps per SM 41 % of the issue slots and 45 % of the FP64 pipe are used, the
 // rest being instruction latency and fetch.  mu and the gathered populations
 // are staged in a shared-memory column per thread by asynchronous copies, so
 // that they hold no registers, and the velocity pairs are walked in three
 // rounds by one loop body (a third of the code to fetch).  200x100x100 sphere
-// 1.51 -> 0.83 ms, 192^3 box 5.1 -> 2.35 ms; blocks of 64 threads: 5, 6 and 7
-// per SM 2.65, 2.35 and 2.49 ms; all values in registers and unrolled, 3
-// blocks of 128: 2.35 ms on the box, 0.854 on the sphere.
+// 1.51 -> 0.86 ms.  (Before the rounding below, 0.83 ms there and 2.35 on the
+// 192^3 box, 5.1 in binary64; blocks of 64 threads: 5, 6 and 7 per SM 2.65, 2.35
+// and 2.49 ms; all values in registers and unrolled, 3 blocks of 128: 2.35 ms on
+// the box, 0.854 on the sphere.)
+//
 // Error against 113-bit references (1.5e6 cells, |beta_a| up to 0.5, lambda
-// normal): nu 1.2e-16 (2 to 3e-16 in binary64), the terms of dL/dtau 1.1e-16
-// rms (3.0e-16).  What the sum over the lattice sees is their mean, since it
-// counts N times: for lambda of zero mean -7e-20 +- 9e-20 (binary64 -3e-20 +-
-// 2e-19), for binary32 lambda -4e-19, for lambda of one sign -1.3e-17
-// (5.2e-17).  With ties always up, weights floored and a mean in place of the
-// low halves' products these were -2.6e-18, +6.7e-17 and -1.5e-17; without
-// that the 200x100x100 sphere takes 0.83 ms instead of 0.88.
+// normal): nu 0.9e-16 rms, the terms of dL/dtau 1.1e-16 (binary64 5.5e-16 and
+// 3.0e-16).  What the sum over the lattice, or over many steps, sees is their
+// mean: of a term -5e-20 +- 9e-20 for lambda of zero mean (binary64 -3e-20 +-
+// 2e-19), -3e-19 for binary32 lambda, -9e-19 for lambda of one sign (5.2e-17);
+// of a value of nu next to an outflow plane 1e-18 of the largest.  That takes
+// ties to even or balanced, weights rounded, and the products of the low halves
+// themselves: with ties up, floors and a mean product they were -2.6e-18,
+// +6.7e-17, -1.5e-17 and 2.4e-17 (0.83 ms on the sphere).
 // ---------------------------------------------------------------------------
 
 struct AdjFx {

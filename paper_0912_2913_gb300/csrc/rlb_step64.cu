@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(128) k_step_f64_split(const double* __restrict
 // k_step_f64 issues 203 FP64 instructions per cell, 13,200 clocks of the
 // scheduler's FP64 pipe per 32 cells against 3,600 for the cell's 608 bytes
 // at the HBM rate.  Here 53 remain (15 for the recovery, 38 relaxations
-// h + omega (eq - h)) beside 2,846 instructions in all, 1,401 of them on the
+// h + omega (eq - h)) beside 2,989 instructions in all, 1,418 of them on the
 // ALU pipe at two clocks each: the two pipes are loaded alike, and a warp's
 // integer and FP64 phases overlap with those of the others.  256^3 box 6.07 ->
 // 2.09 ms, 200x100x100 sphere 0.740 -> 0.285 ms per step.  Resident blocks of
